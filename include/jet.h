@@ -95,11 +95,15 @@ extern "C" {
  *   coarsen_target = 0              stop coarsening at <= max(8k, 256) vertices (Sec. 3)
  *   max_levels = 64, max_iters_per_level = 10000 (safety caps), hem_rounds = 8
  * Execution choice (no counterpart in the paper; results do not depend on it):
- *   cluster_max_n = 4096            levels with at most this many vertices run their whole
- *                                   refinement loop in one thread-block-cluster launch; larger
- *                                   levels use the CUDA-graph loop; 0 = never
- *   cluster_blocks = 0              blocks (of 1024 threads) of that cluster: 0 = the largest the
- *                                   device runs (up to 16), else a power of two in [2, 16]
+ *   cluster_max_n = 65536           levels with at most this many vertices that fit the shared
+ *                                   memory of one thread-block cluster are refined there, the whole
+ *                                   chain of them (coarsest first) in one launch; larger levels, and
+ *                                   dense ones (more than 400,000 CSR entries and more than 40 per
+ *                                   vertex), use the CUDA-graph loop; 0 = never.  Levels of up to 4096
+ *                                   vertices (with a value above the default: of up to that many)
+ *                                   run in one cluster launch also when they do not fit
+ *   cluster_blocks = 0              blocks of that cluster: 0 = chosen by the level's size (up to
+ *                                   16), else a power of two in [2, 16]
  *   barrier_polls = 0               polls a block of the persistent level loop (JET_FLAG_GRID_LOOP)
  *                                   makes at a grid barrier before it gives up and the call returns
  *                                   JET_ETIMEOUT; 0 = 2^22 (about a second or more, far above any
@@ -155,7 +159,8 @@ typedef struct {
     int64_t sel_launches[JET_MAX_LEVELS];  /* Jetlp select passes per level */
     int64_t sel_bytes[JET_MAX_LEVELS];     /* their algorithmic bytes, summed */
     float sel_ms[JET_MAX_LEVELS];          /* their CUDA-event time, summed (JET_FLAG_PROFILE only) */
-    float ms_level[JET_MAX_LEVELS];        /* CUDA-event time of each level's projection + refinement */
+    float ms_level[JET_MAX_LEVELS];        /* time of each level's projection + refinement: CUDA events, or the
+                                              device's clock where one launch ran several levels */
     int32_t cluster_blocks[JET_MAX_LEVELS]; /* blocks of the thread-block cluster that ran the level's
                                                loop; 0 where the CUDA-graph or host loop ran it */
     /* per level and refinement kernel (JET_K_*): launches (0 where one cluster or cooperative launch
@@ -247,8 +252,8 @@ int jet_partition_host(jet_ctx *ctx, int32_t n, const int64_t *xadj, const int32
  * is one jet_partition (device arrays, its own k, eps and seed; results
  * bit-identical to a jet_partition call with the same arguments); `workers`
  * host threads (<= 0: 8) each drive their own stream and memory pool on the
- * context's device, so small graphs, whose refinement is latency-bound, fill
- * the GPU together.  The work starts after what is already enqueued on the
+ * context's device; a graph's coarse levels occupy a few SMs, so that graphs
+ * whose refinement is latency-bound share the GPU.  The work starts after what is already enqueued on the
  * context's stream and is complete when the call returns.  Returns JET_OK
  * when every item succeeded or returned a warning, else the status of the
  * first failed item (each item's own status is in its `status`). */
@@ -271,9 +276,9 @@ int jet_partition_batch(jet_ctx *ctx, int32_t count, jet_batch_item *items, int3
  * are bit-identical under every choice).  Times `items` (a batch, or one
  * graph with count = 1) with jet_partition_batch under each candidate, one
  * choice (stage) at a time, each stage keeping the best of the earlier ones:
- *   JET_TUNE_CLUSTER_BLOCKS  cluster_blocks in {16, 8, 4, 2} (at cluster_max_n 4096)
- *   JET_TUNE_CLUSTER_MAX_N   cluster_max_n in {0, 1024, 2048, 4096, 8192, 16384} (the largest
- *                            level that runs its whole refinement loop in one cluster launch)
+ *   JET_TUNE_CLUSTER_BLOCKS  cluster_blocks in {16, 8, 4, 2} (at the default cluster_max_n)
+ *   JET_TUNE_CLUSTER_MAX_N   cluster_max_n in {0, 4096, 8192, 16384, 32768, 65536} (the largest
+ *                            level that is refined in a cluster)
  *   JET_TUNE_WORKERS         workers in {1, 2, 4, 8, 16} (count > 1 only)
  *   JET_TUNE_LIST_BLOCKS     list_blocks_per_sm in {2, 4, 8}
  *   JET_TUNE_APPLY_BLOCKS    apply_blocks_per_sm in {1, 2, 4}

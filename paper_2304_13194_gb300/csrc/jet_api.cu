@@ -224,10 +224,9 @@ struct EventTimer {
 };
 
 int uncoarsen(Ctx &c, const jet_hier *h, int32_t k, double eps, uint64_t seed, const int32_t *init_coarsest,
-              int32_t *part_out, int64_t *cut_out, jet_stats *st, int32_t top, bool top_refined) {
+              int32_t *part_out, int64_t *cut_out, jet_stats *st) {
     cudaStream_t s = c.stream;
-    int32_t l = top >= 0 ? top : h->levels - 1;
-    if (l >= h->levels || (top >= 0 && !init_coarsest)) return JET_EINVAL;
+    const int32_t l = h->levels - 1;
     int32_t nmax = 1;
     for (int32_t i = 1; i <= l; ++i) nmax = std::max(nmax, h->n[i]);
     DevBuf pa, pb;
@@ -286,7 +285,48 @@ int uncoarsen(Ctx &c, const jet_hier *h, int32_t k, double eps, uint64_t seed, c
         }
     } runs;
     runs.s = s;
-    for (int32_t i = l; i >= 0; --i) {
+    // the coarse levels that a cluster can hold: one launch for the whole
+    // chain, from the coarsest to level `chain_end`
+    int32_t next = l;                      // coarsest level not in the chain
+    int32_t chain_end = l + 1, chain_cs = 0;
+    if (!(c.opt.flags & (JET_FLAG_HOSTLOOP | JET_FLAG_PROFILE))) {
+        for (int32_t i = l; i >= 0; --i) {
+            int cs = 0;
+            JET_TRY(resident_cluster(c, h->n[i], h->nnz[i], k, &cs));
+            if (cs == 0) break;
+            chain_cs = std::max(chain_cs, cs);
+            chain_end = i;
+        }
+    }
+    if (chain_end <= l) {
+        ResChainLevel lv[JET_MAX_LEVELS];
+        const int32_t *start = cur;
+        for (int32_t i = l; i >= chain_end; --i) {
+            ResChainLevel &q = lv[l - i];
+            q.g = level_graph(i);
+            q.seed = level_seed(seed, i);
+            q.slot = i;
+            q.is_finest = i == 0;
+            q.cmap = i < l ? h->cmap[i] : nullptr;
+            int32_t *dst = i == 0 ? part_out : (i < l ? other : cur);
+            if (i < l) {
+                other = cur;
+                cur = dst;
+            }
+            q.out = dst;
+            LevelRun &run = runs.r[i];
+            run.slot = i;
+            run.want_trace = i == 0;
+            run.g = q.g;
+            run.k = k;
+            run.resident = chain_cs;
+        }
+        runs.lo = chain_end;
+        runs.hi = l;
+        JET_TRY(resident_enqueue(c, lv, l - chain_end + 1, k, eps, W, chain_cs, start, chain_end == 0));
+        next = chain_end - 1;
+    }
+    for (int32_t i = next; i >= 0; --i) {
         DGraph g = level_graph(i);
         if (st && lev[(size_t)i + 1]) cudaEventRecord(lev[(size_t)i + 1], s);
         if (i < l) {
@@ -297,7 +337,6 @@ int uncoarsen(Ctx &c, const jet_hier *h, int32_t k, double eps, uint64_t seed, c
             cur = dst;
         }
         if (i == 0) cudaEventRecord(ev.e[2], s);
-        if (i == l && top_refined) continue;   // the given partition is already refined there
         LevelRun &run = runs.r[i];
         run.slot = i;
         run.want_trace = i == 0;
@@ -311,7 +350,6 @@ int uncoarsen(Ctx &c, const jet_hier *h, int32_t k, double eps, uint64_t seed, c
     runs.done = true;
     int first_err = JET_OK;
     for (int32_t i = l; i >= 0; --i) {
-        if (i == l && top_refined) continue;
         LevelReport rep;
         int r = refine_level_finish(c, runs.r[i], &cut, &maxw, &rep);
         if (r < 0) {
@@ -329,6 +367,7 @@ int uncoarsen(Ctx &c, const jet_hier *h, int32_t k, double eps, uint64_t seed, c
             st->sel_bytes[i] = rep.sel_bytes;
             st->sel_ms[i] = rep.sel_ms;
             st->cluster_blocks[i] = rep.cluster;
+            st->ms_level[i] = rep.ms;
             st->bytes_model += rep.bytes_model;
             for (int kk = 0; kk < JET_KERNELS; ++kk) {
                 st->kern_launches[i][kk] = rep.kern_launches[kk];
@@ -340,7 +379,7 @@ int uncoarsen(Ctx &c, const jet_hier *h, int32_t k, double eps, uint64_t seed, c
     if (first_err != JET_OK) return first_err;
     if (st) {
         // level i ran between the events recorded at i + 1 and at i
-        for (int32_t i = l; i >= 0; --i) {
+        for (int32_t i = next; i >= 0; --i) {
             float t = 0.f;
             if (lev[(size_t)i + 1] && lev[(size_t)i] &&
                 cudaEventElapsedTime(&t, lev[(size_t)i + 1], lev[(size_t)i]) == cudaSuccess)
@@ -357,7 +396,7 @@ int uncoarsen(Ctx &c, const jet_hier *h, int32_t k, double eps, uint64_t seed, c
         st->fin_edge_iters = fin_edge_iters;
         st->ms_init = ev.ms(0, 1);
         st->ms_refine = ev.ms(1, 3);
-        st->ms_refine_finest = ev.ms(2, 3);
+        st->ms_refine_finest = next >= 0 ? ev.ms(2, 3) : st->ms_level[0];
         st->cut = cut;
         st->max_part_w = maxw;
     }
@@ -385,7 +424,7 @@ void jet_options_default(jet_options *o) {
     o->max_iters_per_level = 10000;
     o->hem_rounds = 8;
     o->flags = 0;
-    o->cluster_max_n = 4096;
+    o->cluster_max_n = kClusterMaxNDefault;
     o->cluster_blocks = 0;
     o->barrier_polls = 0;
     o->list_blocks_per_sm = o->list_items_per_block = o->apply_blocks_per_sm = o->scan_blocks_per_sm = 0;
@@ -601,15 +640,10 @@ int jet_partition(jet_ctx *ctx, int32_t n, const int64_t *xadj, const int32_t *a
     return r;
 }
 
-// Batched form.  Three stages, each bit-identical to jet_partition per item:
-//  1. the workers (host threads, each with its own context, stream and pool)
-//     coarsen every graph and compute the greedy start of its coarsest level;
-//  2. the small levels of all graphs — each graph's chain of levels of at
-//     most cluster_max_n vertices, coarsest first — are refined in one
-//     persistent cluster launch that takes graphs from a work queue
-//     (refine_small_chains);
-//  3. the workers refine every graph's larger levels (projection + the
-//     CUDA-graph loop per level).
+// Batched form: the workers (host threads, each with its own context, stream
+// and pool) take graphs from a counter and partition them one after another,
+// each bit-identical to jet_partition.  A graph's coarse levels are one
+// resident-chain launch on a few SMs, so the workers' graphs share the GPU.
 int jet_partition_batch(jet_ctx *ctx, int32_t count, jet_batch_item *items, int32_t workers) {
     if (!ctx || count < 0 || (count > 0 && !items)) return JET_EINVAL;
     if (count == 0) return JET_OK;
@@ -645,131 +679,38 @@ int jet_partition_batch(jet_ctx *ctx, int32_t count, jet_batch_item *items, int3
         JET_TRY(jet_ctx_create(c.device, w.s, &wo, &w.wc));
     }
     JET_TRY(use_device(c));
-    struct Item {
-        jet_hier *h = nullptr;
-        DevBuf init;                 // greedy start of the coarsest level (worker's pool)
-        int64_t W = 0;
-        int32_t bottom = -1;         // finest level of the small chain (-1: none)
-        int32_t chain = -1;
-        bool done = false;
-        double ms = 0;
-        ~Item() {
-            if (h) jet_hier_destroy(h);
-        }
-    };
-    std::vector<Item> st((size_t)count);
     std::vector<int> wstat((size_t)workers, JET_OK);
-    // runs fn(worker context, item) over all items on the workers
-    auto run_workers = [&](auto &&fn) {
-        std::atomic<int32_t> next{0};
-        auto body = [&](int w) {
-            jet_ctx *wc = wk[(size_t)w].wc;
-            for (;;) {
-                int32_t i = next.fetch_add(1);
-                if (i >= count) break;
-                if (st[(size_t)i].done) continue;
-                auto t0 = std::chrono::steady_clock::now();
-                fn(wc, i);
-                st[(size_t)i].ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
-            }
-            if (cudaStreamSynchronize(wk[(size_t)w].s) != cudaSuccess) {
-                cudaGetLastError();
-                wstat[(size_t)w] = JET_ECUDA;
-            }
-        };
-        std::vector<std::thread> pool;
-        int started = 0;
-        try {
-            pool.reserve((size_t)workers);
-            for (int w = 0; w < workers; ++w) {
-                pool.emplace_back(body, w);
-                ++started;
-            }
-        } catch (...) {   // no exception crosses the C ABI: the workers that started take every item
-            if (started == 0) body(0);   // none did: the calling thread takes the whole batch
+    std::atomic<int32_t> next{0};
+    auto body = [&](int w) {
+        jet_ctx *wc = wk[(size_t)w].wc;
+        for (;;) {
+            const int32_t i = next.fetch_add(1);
+            if (i >= count) break;
+            jet_batch_item &it = items[i];
+            auto t0 = std::chrono::steady_clock::now();
+            it.cut = 0;
+            it.status = it.n == 0 ? JET_OK
+                                  : jet_partition(wc, it.n, it.xadj, it.adjncy, it.vwgt, it.adjwgt, it.k, it.eps,
+                                                  it.seed, it.part_out, &it.cut, nullptr);
+            it.ms = (float)std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
         }
-        for (auto &t : pool) t.join();
+        if (cudaStreamSynchronize(wk[(size_t)w].s) != cudaSuccess) {
+            cudaGetLastError();
+            wstat[(size_t)w] = JET_ECUDA;
+        }
     };
-    const int32_t thr = c.opt.cluster_max_n;
-    // stage 1: coarsening and the greedy start of the coarsest level
-    run_workers([&](jet_ctx *wc, int32_t i) {
-        jet_batch_item &it = items[i];
-        Item &s1 = st[(size_t)i];
-        it.cut = 0;
-        it.status = JET_OK;
-        if (it.n == 0) {
-            s1.done = true;
-            return;
+    std::vector<std::thread> pool;
+    int started = 0;
+    try {
+        pool.reserve((size_t)workers);
+        for (int w = 0; w < workers; ++w) {
+            pool.emplace_back(body, w);
+            ++started;
         }
-        int r = jet_coarsen(wc, it.n, it.xadj, it.adjncy, it.vwgt, it.adjwgt, it.k, it.seed, &s1.h);
-        if (r < 0) { it.status = r; s1.done = true; return; }
-        Ctx &w = wc->c;
-        const jet_hier *h = s1.h;
-        const int32_t l = h->levels - 1;
-        DGraph gl;
-        gl.n = h->n[l]; gl.nnz = h->nnz[l]; gl.xadj = h->xadj[l]; gl.adj = h->adj[l]; gl.vw = h->vw[l]; gl.ew = h->ew[l];
-        r = use_device(w);
-        if (r >= 0) r = dev_alloc(s1.init, (size_t)std::max<int32_t>(gl.n, 1) * 4, w.stream);
-        if (r >= 0) r = initial_partition(w, gl, it.k, s1.init.as<int32_t>());
-        if (r >= 0) r = total_vweight(w, gl, s1.W);
-        if (r < 0) { it.status = r; s1.done = true; return; }
-        if (thr > 0 && h->n[l] <= thr) {
-            int32_t b = l;
-            while (b > 0 && h->n[b - 1] <= thr) --b;
-            s1.bottom = b;
-        }
-    });
-    for (int w = 0; w < workers; ++w)
-        if (wstat[(size_t)w] != JET_OK) return wstat[(size_t)w];
-    // stage 2: every graph's small levels in one persistent launch
-    std::vector<SmallChain> chains;
-    std::vector<DevBuf> chain_out;
-    for (int32_t i = 0; i < count; ++i) {
-        Item &s1 = st[(size_t)i];
-        if (s1.done || s1.bottom < 0) continue;
-        const jet_batch_item &it = items[i];
-        SmallChain ch;
-        ch.h = s1.h;
-        ch.top = s1.h->levels - 1;
-        ch.bottom = s1.bottom;
-        ch.k = it.k;
-        ch.eps = it.eps;
-        ch.seed = it.seed;
-        ch.W = s1.W;
-        ch.init = s1.init.as<int32_t>();
-        if (s1.bottom == 0) {
-            ch.out = it.part_out;
-        } else {
-            chain_out.emplace_back();
-            JET_TRY(dev_alloc(chain_out.back(), (size_t)s1.h->n[s1.bottom] * 4, c.stream));
-            ch.out = chain_out.back().as<int32_t>();
-        }
-        s1.chain = (int32_t)chains.size();
-        chains.push_back(ch);
+    } catch (...) {   // no exception crosses the C ABI: the workers that started take every item
+        if (started == 0) body(0);   // none did: the calling thread takes the whole batch
     }
-    int ran = 0;
-    JET_TRY(refine_small_chains(c, chains.data(), (int32_t)chains.size(), c.opt.cluster_blocks, &ran));
-    // stage 3: the larger levels
-    run_workers([&](jet_ctx *wc, int32_t i) {
-        jet_batch_item &it = items[i];
-        Item &s1 = st[(size_t)i];
-        const SmallChain *ch = (ran && s1.chain >= 0) ? &chains[(size_t)s1.chain] : nullptr;
-        int r;
-        if (ch && ch->bottom == 0) {
-            it.cut = ch->cut;
-            r = ch->status;
-        } else if (ch) {
-            r = use_device(wc->c);
-            if (r >= 0) r = uncoarsen(wc->c, s1.h, it.k, it.eps, it.seed, ch->out, it.part_out, &it.cut, nullptr,
-                                      ch->bottom, true);
-        } else {
-            r = use_device(wc->c);
-            if (r >= 0) r = uncoarsen(wc->c, s1.h, it.k, it.eps, it.seed, s1.init.as<int32_t>(), it.part_out, &it.cut,
-                                      nullptr);
-        }
-        it.status = r;
-    });
-    for (int32_t i = 0; i < count; ++i) items[i].ms = (float)st[(size_t)i].ms;
+    for (auto &t : pool) t.join();
     for (int w = 0; w < workers; ++w)
         if (wstat[(size_t)w] != JET_OK) return wstat[(size_t)w];
     for (int32_t i = 0; i < count; ++i)
@@ -820,7 +761,7 @@ int jet_autotune(jet_ctx *ctx, int32_t count, jet_batch_item *items, int32_t rep
         return JET_OK;
     };
     static const int32_t blocks[] = {16, 8, 4, 2};
-    static const int32_t thresholds[] = {0, 1024, 2048, 4096, 8192, 16384};
+    static const int32_t thresholds[] = {0, 4096, 8192, 16384, 32768, kClusterMaxNDefault};
     static const int32_t wcands[] = {1, 2, 4, 8, 16};
     static const int32_t list_bpsm[] = {2, 4, 8};
     static const int32_t apply_bpsm[] = {1, 2, 4};
@@ -829,7 +770,7 @@ int jet_autotune(jet_ctx *ctx, int32_t count, jet_batch_item *items, int32_t rep
     static const int32_t hubs[] = {256, 1024, 4096};
     const jet_options saved = c.opt;
     jet_options &o = c.opt;
-    o.cluster_max_n = 4096;
+    o.cluster_max_n = kClusterMaxNDefault;
     o.list_blocks_per_sm = 4;
     o.apply_blocks_per_sm = 4;
     o.list_items_per_block = 64;

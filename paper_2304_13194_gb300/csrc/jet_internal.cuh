@@ -25,6 +25,8 @@ constexpr int kTB = 256;                   // default block size
 #define JET_RB_TILE 256
 #endif
 constexpr int kRbTile = JET_RB_TILE;       // vertices per rebalancing tile (ordered prefixes; one block each)
+constexpr int kClusterMaxNDefault = 65536; // jet_options.cluster_max_n
+constexpr int kClusterLoopMaxN = 4096;     // levels up to this size: cluster loop also without a resident chain
 constexpr int kTrace = 4096;               // per-level trace records kept on the device
 
 enum Mode : int32_t { MODE_LP = 0, MODE_RW = 1, MODE_RS = 2, MODE_DONE = 3 };
@@ -462,20 +464,33 @@ struct LevelReport {
     int64_t sel_launches = 0, sel_bytes = 0, bytes_model = 0;
     float sel_ms = 0.f;
     int32_t cluster = 0;   // blocks of the cluster that ran the level loop (0: graph or host loop)
+    float ms = 0.f;        // the level's time inside a resident chain (0: timed by events)
     // per refinement kernel (JET_K_*): launches, algorithmic bytes, CUDA-event ms (profiling only)
     int64_t kern_launches[JET_KERNELS] = {};
     int64_t kern_bytes[JET_KERNELS] = {};
     float kern_ms[JET_KERNELS] = {};
 };
 
+// Outcome of one level of a resident chain (jet_resident.cu), written by the
+// kernel into pinned host memory.
+struct ResStat {
+    int64_t best_cut, best_maxw;
+    int64_t kbytes[JET_K_COUNT];
+    int64_t ns;              // the level's time in the launch
+    int32_t it, best_bal, hit_cap, pad;
+    int32_t kcount[4];
+};
+
 // Pinned host buffer of a context: scalar readbacks in the first 4 KB, then
 // one control block per level of an uncoarsening (copied back when the level
-// is enqueued, read after the last level), then the finest level's trace.
+// is enqueued, read after the last level), then the finest level's trace,
+// then one outcome per level of a resident chain.
 constexpr size_t kPinnedScalarBytes = 4096;
 constexpr size_t kPinnedCtlStride = (sizeof(Ctl) + 255) & ~size_t(255);
 constexpr size_t kPinnedCtlOff = kPinnedScalarBytes;
 constexpr size_t kPinnedTraceOff = kPinnedCtlOff + kPinnedCtlStride * JET_MAX_LEVELS;
-constexpr size_t kPinnedBytes = kPinnedTraceOff + sizeof(TraceRec) * (size_t)kTrace;
+constexpr size_t kPinnedResOff = kPinnedTraceOff + ((sizeof(TraceRec) * (size_t)kTrace + 255) & ~size_t(255));
+constexpr size_t kPinnedBytes = kPinnedResOff + sizeof(ResStat) * JET_MAX_LEVELS;
 
 struct Ctx {
     int64_t launches = 0;        // kernels launched (graph-loop iterations counted per executed kernel)
@@ -526,6 +541,7 @@ struct LevelRun {
     DGraph g;
     int32_t k = 0;
     int32_t cluster = 0, grid = 0, hostloop = 0;
+    int32_t resident = 0;             // blocks of the cluster whose resident chain runs the level (0: none)
     int nk_branch[3] = {0, 0, 0}, nk_tail = 0;
     cudaGraphExec_t exec = nullptr;   // the level's CUDA-graph loop (destroyed by refine_level_finish)
     LevelReport rep;                  // host-loop profile (kern_ms, sel_ms)
@@ -535,25 +551,23 @@ int refine_level_enqueue(Ctx &c, const DGraph &g, int32_t k, double eps, int32_t
                          int32_t *part_inout, int64_t W, LevelRun &run);
 int refine_level_finish(Ctx &c, LevelRun &run, int64_t *cut_out, int64_t *maxw_out, LevelReport *rep);
 void refine_level_abandon(LevelRun &run);   // after an error: release what the run holds
-// The batched form's small levels: one graph's chain of levels of at most
-// cluster_max_n vertices, refined with those of the other chains in one
-// persistent cluster launch (refine_small_chains).
-struct SmallChain {
-    const jet_hier *h = nullptr;
-    int32_t top = 0, bottom = 0;     // the coarsest level and the finest small level (top >= bottom)
-    int32_t k = 2;
-    double eps = 0.03;
-    uint64_t seed = 1;               // the partition's seed (level seeds derive from it)
-    int64_t W = 0;                   // total vertex weight
-    const int32_t *init = nullptr;   // device: start partition of level `top`
-    int32_t *out = nullptr;          // device: receives the refined partition of level `bottom`
-    int64_t cut = 0, maxw = 0;       // out: of level `bottom`
-    int32_t status = JET_OK;         // out: of level `bottom`
+// jet_resident.cu: a chain of levels in one cluster launch, each level kept in
+// the cluster's shared memory.
+struct ResChainLevel {
+    DGraph g;
+    const int32_t *cmap = nullptr;   // from the level before it in the chain (null: starts from the given partition as it is)
+    int32_t *out = nullptr;          // receives the level's refined partition
+    uint64_t seed = 0;               // the level's Jetrw seed
+    int32_t slot = 0;                // outcome slot in the context's pinned buffer
+    bool is_finest = false;
 };
-// cluster_blocks: blocks of each cluster (0 = 4).  On success every chain's
-// `out` holds its result; JET_ECUDA with *ran = 0 when the device cannot
-// co-schedule one cluster (the caller refines the levels one by one).
-int refine_small_chains(Ctx &c, SmallChain *chains, int32_t nchains, int32_t cluster_blocks, int *ran);
+// Blocks of the cluster that keeps a level of n vertices and nnz entries (0: it
+// does not fit, or the options exclude it).
+int resident_cluster(Ctx &c, int64_t n, int64_t nnz, int32_t k, int *cs);
+// Enqueues the chain (no host wait); init: the partition its first level
+// starts from.  Outcomes are read by refine_level_finish.
+int resident_enqueue(Ctx &c, const ResChainLevel *lv, int32_t nlv, int32_t k, double eps, int64_t W, int cs,
+                     const int32_t *init, bool want_trace);
 uint64_t level_seed(uint64_t seed, int32_t level);   // Jetrw seed of hierarchy level `level`
 
 // Enqueue + synchronise + finish.  W_known: -1 = computed on the device.
@@ -623,11 +637,8 @@ int check_part(Ctx &c, int32_t n, const int32_t *part, int32_t k);   // JET_EINV
 int prepare_graph(Ctx &c, int32_t n, const int64_t *xadj, const int32_t *adjncy, const int32_t *vwgt,
                   const int32_t *adjwgt, DGraph &g, DevBuf &ones, bool need_vw);
 // Alg. 1 after coarsening; init_coarsest (device, n of the coarsest level)
-// replaces the greedy initial partition when not null.  With top >= 0 the
-// uncoarsening starts at level `top` from init_coarsest (n[top] entries):
-// refined there too unless top_refined, then projected and refined on
-// every finer level.
+// replaces the greedy initial partition when not null.
 int uncoarsen(Ctx &c, const jet_hier *h, int32_t k, double eps, uint64_t seed, const int32_t *init_coarsest,
-              int32_t *part_out, int64_t *cut_out, jet_stats *st, int32_t top = -1, bool top_refined = false);
+              int32_t *part_out, int64_t *cut_out, jet_stats *st);
 
 }  // namespace jet

@@ -427,16 +427,19 @@ __device__ __forceinline__ void reset_counters(Ctl *ctl) {
 // partition during this iteration (the afterburner for Jetlp, rb_scan for
 // rebalancing) when the previous controller asked for it; the copy after
 // the level's last iteration is not a refinement kernel.
+// The model is linear in n, T, k and the counters, so sums over iterations of
+// one kind (n, T and k times their number) give the bytes of all of them.
 struct IterCounts {
-    int64_t nx, nm, degx, degm, nbnd, nexam, degexam, ncand, na;
-    bool copied;
+    int64_t nx, nm, degx, degm, nbnd, nexam, degexam, ncand;
+    int64_t tna;          // T nA
+    int64_t copy_bytes;   // 8n when the iteration copied the best partition
 };
-__device__ __forceinline__ void iter_bytes(const Level &L, int32_t kind, const IterCounts &q, int64_t *b /* [JET_K_COUNT] */) {
-    const int64_t n = L.g.n, beta = L.g.ew ? 8 : 4, T = L.ntiles, k = L.k;
-    const int64_t cp = q.copied ? 8 * n : 0;
+__device__ __forceinline__ void iter_bytes(int64_t n, int64_t beta, int64_t T, int64_t k, uint32_t abl, int32_t kind,
+                                           const IterCounts &q, int64_t *b /* [JET_K_COUNT] */) {
+    const int64_t cp = q.copy_bytes;
     for (int i = 0; i < JET_K_COUNT; ++i) b[i] = 0;
     if (kind == MODE_LP) {
-        const bool ab = !(L.abl & (ABL_NO_AFTERBURN | ABL_BASELINE_LP));
+        const bool ab = !(abl & (ABL_NO_AFTERBURN | ABL_BASELINE_LP));
         const int64_t w = q.nexam, X = q.nx, M = q.nm;
         b[JET_K_LP_SCAN] = 4 * n + 4 * q.nbnd + 4 * w;
         b[JET_K_LP_SELECT] = 24 * w + beta * q.degexam + 12 * X;
@@ -444,7 +447,7 @@ __device__ __forceinline__ void iter_bytes(const Level &L, int32_t kind, const I
         b[JET_K_APPLY] = 40 * M + beta * q.degm + 16 * k + 8 * X;
     } else {
         const bool rs = kind == MODE_RS;
-        const int64_t c = q.ncand, r = q.nbnd, M = q.nm, tn = T * q.na;
+        const int64_t c = q.ncand, r = q.nbnd, M = q.nm, tn = q.tna;
         b[JET_K_RB_SCAN] = cp + 8 * n + 16 * c + 4 * r;
         b[JET_K_RB_CAND] = (rs ? 28 : 32) * r + beta * q.degexam;
         b[JET_K_RB_TILEHIST] = 4 * n + 4 * c + 4 * tn;
@@ -536,9 +539,9 @@ __device__ inline int32_t ph_controller(const Level &L) {
         }
         {
             const IterCounts q{kind == MODE_LP ? (int64_t)nX : 0, nM, degx, degm, nbnd, nexam, degexam, ncand,
-                               kind == MODE_LP ? 0 : nA, copied != 0};
+                               kind == MODE_LP ? 0 : (int64_t)L.ntiles * nA, copied ? 8 * (int64_t)L.g.n : 0};
             int64_t kb[JET_K_COUNT];
-            iter_bytes(L, kind, q, kb);
+            iter_bytes(L.g.n, L.g.ew ? 8 : 4, L.ntiles, L.k, L.abl, kind, q, kb);
 #pragma unroll
             for (int i = 0; i < JET_K_COUNT; ++i) ctl->kbytes[i] = kb0[i] + kb[i];
         }

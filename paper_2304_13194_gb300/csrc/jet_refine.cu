@@ -1,16 +1,18 @@
 // Jet refinement on one level (Sec. 4): Jetlp (Alg. 4), Jetrw (Alg. 5),
 // Jetrs (Sec. 4.2.2) and the driver of Alg. 3, for sm_103a.
 //
-// The passes themselves are device functions in jet_phases.cuh.  They run in
-// one of two ways:
+// The passes themselves are device functions in jet_phases.cuh.  Levels that a
+// cluster's shared memory can hold are refined in jet_resident.cu; for the
+// others the passes run in one of two ways:
 //  * large levels: one kernel per phase, and the whole level loop is a CUDA
 //    graph with a WHILE node around SWITCH nodes over {Jetlp, Jetrw, Jetrs}
 //    (two iterations per loop body); the controller, in the last block of
 //    the apply kernel, sets the conditionals, so no host round trip happens
 //    per iteration (the paper blames that round trip for its weaker
 //    coarse-level speedup, Sec. 6.2);
-//  * small levels: one thread block cluster (up to 16 SMs) runs every
-//    iteration of the level in a single launch, the phases separated by the
+//  * small levels whose state does not fit there (many parts): one thread
+//    block cluster (up to 16 SMs) runs every iteration of the level in a
+//    single launch on the state in global memory, the phases separated by the
 //    hardware cluster barrier — no launch or graph node per phase.
 #include "jet_phases.cuh"
 
@@ -418,141 +420,6 @@ __global__ void __launch_bounds__(kTB, JET_ROW_MINB) k_refine_grid(Level L) {
         if (!grid_sync(L, [&] { ph_controller(L); })) return;
     }
     ph_copy_best(L, G);
-}
-
-// ---------------------------------------------------------------------------
-// batched form: the small levels of many graphs in one persistent launch
-// ---------------------------------------------------------------------------
-// A job is one graph's chain of small levels, coarsest first (the levels of
-// at most cluster_max_n vertices form the coarse end of its hierarchy).  The
-// clusters of one launch take jobs from a counter; a cluster runs the whole
-// chain of its job: per level the projection of the coarser level's
-// partition, the level's start state (the work of setup_level and
-// enqueue_init, as cluster phases), the whole Alg. 3 loop, and the P_best
-// copy; then it takes the next job.  Every decision is the one the
-// per-level launches take, so results are bit-identical.
-struct BatchLevel {
-    DGraph g;
-    const int32_t *cmap;     // this level -> the next coarser one (unused on the job's coarsest level)
-    uint64_t seed;           // Jetrw seed of the level
-    int32_t cq16;            // first-filter ratio c of the level (c_fine on level 0)
-    int32_t pad;
-};
-struct BatchStat {           // the control block's outcome of one level
-    int64_t best_cut, best_maxw;
-    int64_t kbytes[JET_K_COUNT];
-    int32_t it, best_bal, hit_cap, pad;
-    int32_t kcount[4];
-};
-struct BatchJob {
-    Level L;                 // buffers sized for the chain's largest level; the level fields are set per level
-    const BatchLevel *lv;    // [nlv], coarsest first
-    BatchStat *stat;         // [nlv]
-    const int32_t *init;     // start partition of the coarsest level
-    int32_t *part[2];        // level partitions, alternating (level i in part[i & 1])
-    int32_t *out;            // receives the finest level's partition (may be null)
-    int64_t *cut2;           // scratch: twice the start cut of a level
-    int64_t Llim, opt, sigma;
-    int32_t nlv, pad;
-};
-
-// Start of one level inside a job (all blocks of the cluster): projection,
-// per-vertex start values, cut / part weights / ext / weighted degree, the
-// long-row count, then the control block (block 0) and P_best = P_0.
-__device__ inline void batch_level_start(const BatchJob &job, const Level &L, int32_t i, Grid G, char *arena,
-                                         cg::cluster_group &cl) {
-    const int64_t n = L.g.n;
-    const int64_t t0 = (int64_t)G.bid * blockDim.x + threadIdx.x, stride = (int64_t)G.nb * blockDim.x;
-    int32_t *cur = L.part;
-    if (i == 0) {
-        for (int64_t v = t0; v < n; v += stride) cur[v] = job.init[v];
-    } else {
-        const int32_t *prev = job.part[(i - 1) & 1];
-        const int32_t *cmap = job.lv[i].cmap;
-        for (int64_t v = t0; v < n; v += stride) cur[v] = prev[cmap[v]];
-    }
-    for (int64_t v = t0; v < n; v += stride) {
-        L.lstamp[v] = -2;
-        L.mstamp[v] = -2;
-        L.prio[v] = kNoneGain;
-    }
-    if (G.bid == 0) {
-        int64_t *w = reinterpret_cast<int64_t *>(L.ctl);
-        for (int q = threadIdx.x; q < (int)(sizeof(Ctl) / 8); q += blockDim.x) w[q] = 0;
-        for (int p = threadIdx.x; p < L.k; p += blockDim.x) L.pw[p] = 0;
-        if (threadIdx.x == 0) job.cut2[0] = 0;
-    }
-    cl.sync();
-    for (int64_t v0 = (int64_t)G.bid * blockDim.x; v0 < n; v0 += stride) {
-        const int64_t v = v0 + threadIdx.x;
-        const bool big = v < n && ld_xadj(L.g.xadj, v + 1) - ld_xadj(L.g.xadj, v) > kSmallDeg;
-        const unsigned m = __ballot_sync(0xffffffffu, big);
-        if (lane_id() == 0 && m) atomicAdd(&L.ctl->nbig, __popc(m));
-    }
-    if (L.g.ew) ph_cut_pw<true>(L.g, L.k, cur, L.pw, job.cut2, L.ext, L.wdeg, G, arena);
-    else ph_cut_pw<false>(L.g, L.k, cur, L.pw, job.cut2, L.ext, L.wdeg, G, arena);
-    cl.sync();
-    if (G.bid == 0) {
-        if (threadIdx.x == 0) {
-            L.ctl->L = job.Llim;
-            L.ctl->opt = job.opt;
-            L.ctl->sigma = job.sigma;
-        }
-        __syncthreads();
-        ph_ctl_init(L, job.cut2);
-    }
-    for (int64_t v = t0; v < n; v += stride) L.best[v] = cur[v];
-    cl.sync();
-}
-
-__global__ void __launch_bounds__(kClusterThreads, 1) k_refine_batch(const BatchJob *jobs, int32_t njobs,
-                                                                     int32_t *queue) {
-    cg::cluster_group cl = cg::this_cluster();
-    const Grid G{(int)cl.block_rank(), (int)cl.num_blocks()};
-    char *arena = JET_ARENA;
-    __shared__ int s_job;
-    __shared__ Level L;   // the level's parameters, in shared memory rather than on each thread's stack
-    for (;;) {
-        if (G.bid == 0 && threadIdx.x == 0) s_job = atomicAdd(queue, 1);
-        cl.sync();
-        const int j = *cl.map_shared_rank(&s_job, 0);
-        cl.sync();   // every block has read the job before block 0 takes the next
-        if (j >= njobs) break;
-        const BatchJob &job = jobs[j];
-        for (int32_t i = 0; i < job.nlv; ++i) {
-            if (threadIdx.x == 0) {
-                const BatchLevel &bl = job.lv[i];
-                L = job.L;
-                L.g = bl.g;
-                L.seed = bl.seed;
-                L.cq16 = bl.cq16;
-                L.ntiles = (int32_t)(((int64_t)bl.g.n + kClusterThreads - 1) / kClusterThreads);
-                if (L.ntiles < 1) L.ntiles = 1;
-                L.part = job.part[i & 1];
-            }
-            __syncthreads();
-            batch_level_start(job, L, i, G, arena, cl);
-            if (L.g.ew) cluster_level_loop<true>(L, G, arena, cl);
-            else cluster_level_loop<false>(L, G, arena, cl);
-            cl.sync();
-            // P_best is the level's result
-            const int64_t n = L.g.n, t0 = (int64_t)G.bid * blockDim.x + threadIdx.x, stride = (int64_t)G.nb * blockDim.x;
-            int32_t *dst = (i + 1 == job.nlv && job.out) ? job.out : L.part;
-            for (int64_t v = t0; v < n; v += stride) dst[v] = L.best[v];
-            if (G.bid == 0 && threadIdx.x == 0) {
-                const Ctl *c = L.ctl;
-                BatchStat &st = job.stat[i];
-                st.best_cut = c->best_cut;
-                st.best_maxw = c->best_maxw;
-                for (int q = 0; q < JET_K_COUNT; ++q) st.kbytes[q] = c->kbytes[q];
-                st.it = c->it;
-                st.best_bal = c->best_bal;
-                st.hit_cap = c->hit_cap;
-                for (int q = 0; q < 4; ++q) st.kcount[q] = c->kcount[q];
-            }
-            cl.sync();
-        }
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1114,10 +981,14 @@ int run_grid(Ctx &c, const Level &L, int *ran) {
 
 size_t cluster_smem(int32_t k) { return (arena_bytes(k, kClusterThreads) + 255) & ~size_t(255); }
 
-// Cluster size usable for this level (0: use the graph loop).
+// Cluster size usable for this level (0: use the graph loop).  Levels that
+// the resident chain cannot hold get here: up to kClusterLoopMaxN vertices
+// this loop is the faster one, beyond that only on request (a cluster_max_n
+// above the default).
 int pick_cluster(Ctx &c, const Level &L, int *cs) {
     *cs = 0;
     if (L.g.n <= 0 || L.g.n > c.opt.cluster_max_n) return JET_OK;
+    if (L.g.n > kClusterLoopMaxN && c.opt.cluster_max_n <= kClusterMaxNDefault) return JET_OK;
     if (L.g.ew) JET_TRY(cluster_size<true>(c.device, cluster_smem(L.k), cs));
     else JET_TRY(cluster_size<false>(c.device, cluster_smem(L.k), cs));
     if (c.opt.cluster_blocks > 0 && *cs > c.opt.cluster_blocks) *cs = c.opt.cluster_blocks;
@@ -1196,6 +1067,17 @@ int refine_level_enqueue(Ctx &c, const DGraph &g, int32_t k, double eps, int32_t
     run.g = g;
     run.k = k;
     if (run.slot < 0 || run.slot >= JET_MAX_LEVELS) return JET_EINVAL;
+    run.hostloop = (c.opt.flags & (JET_FLAG_HOSTLOOP | JET_FLAG_PROFILE)) != 0;
+    if (!run.hostloop) JET_TRY(resident_cluster(c, g.n, g.nnz, k, &run.resident));
+    if (run.resident > 0) {
+        ResChainLevel lv;
+        lv.g = g;
+        lv.out = part_inout;
+        lv.seed = seed;
+        lv.slot = run.slot;
+        lv.is_finest = is_finest != 0;
+        return resident_enqueue(c, &lv, 1, k, eps, W, run.resident, part_inout, run.want_trace);
+    }
     int64_t opt = 0;
     int64_t L_lim = balance_limit(W, k, eps, &opt);
     int64_t sigma = opt + (L_lim - opt) / 2;
@@ -1206,7 +1088,6 @@ int refine_level_enqueue(Ctx &c, const DGraph &g, int32_t k, double eps, int32_t
     L.part = part_inout;
     fill_level_params(c, L, is_finest, seed);
     JET_TRY(enqueue_init(c, B, L_lim, opt, sigma));
-    run.hostloop = (c.opt.flags & (JET_FLAG_HOSTLOOP | JET_FLAG_PROFILE)) != 0;
     if (!run.hostloop) JET_TRY(pick_cluster(c, L, &run.cluster));
     if (g.n > 0) {
         if (run.hostloop) {
@@ -1241,6 +1122,31 @@ void refine_level_abandon(LevelRun &run) {
 int refine_level_finish(Ctx &c, LevelRun &run, int64_t *cut_out, int64_t *maxw_out, LevelReport *rep_out) {
     refine_level_abandon(run);
     const char *pin = reinterpret_cast<const char *>(c.pinned);
+    auto keep_trace = [&](int32_t iters) {
+        c.last_trace.iters = iters;
+        const int32_t nrec = std::min<int32_t>(iters, kTrace);
+        const TraceRec *ht = reinterpret_cast<const TraceRec *>(pin + kPinnedTraceOff);
+        c.last_trace.rec.assign(ht, ht + std::max<int32_t>(nrec, 0));
+    };
+    if (run.resident > 0) {
+        const ResStat &r = reinterpret_cast<const ResStat *>(pin + kPinnedResOff)[run.slot];
+        LevelReport rep;
+        rep.cluster = run.resident;
+        rep.iters = r.it;
+        for (int kd = 0; kd < 3; ++kd) rep.kinds[kd] = r.kcount[kd];
+        for (int i = 0; i < JET_K_COUNT; ++i) {
+            rep.kern_bytes[i] = r.kbytes[i];
+            rep.bytes_model += r.kbytes[i];
+        }
+        rep.sel_bytes = r.kbytes[JET_K_LP_SCAN] + r.kbytes[JET_K_LP_SELECT];
+        rep.sel_launches = r.kcount[MODE_LP];
+        rep.ms = (float)((double)r.ns * 1e-6);
+        if (run.want_trace) keep_trace(r.it);
+        if (rep_out) *rep_out = rep;
+        if (cut_out) *cut_out = r.best_cut;
+        if (maxw_out) *maxw_out = r.best_maxw;
+        return !r.best_bal ? JET_WUNBALANCED : (r.hit_cap ? JET_WITERLIMIT : JET_OK);
+    }
     Ctl h;
     memcpy(&h, pin + kPinnedCtlOff + kPinnedCtlStride * (size_t)run.slot, sizeof(Ctl));
     if (h.bar_err) {
@@ -1278,12 +1184,7 @@ int refine_level_finish(Ctx &c, LevelRun &run, int64_t *cut_out, int64_t *maxw_o
     }
     rep.sel_bytes = h.kbytes[JET_K_LP_SCAN] + h.kbytes[JET_K_LP_SELECT];
     rep.sel_launches = h.kcount[MODE_LP];
-    if (run.want_trace) {
-        c.last_trace.iters = iters;
-        const int32_t nrec = std::min<int32_t>(iters, kTrace);
-        const TraceRec *ht = reinterpret_cast<const TraceRec *>(pin + kPinnedTraceOff);
-        c.last_trace.rec.assign(ht, ht + std::max<int32_t>(nrec, 0));
-    }
+    if (run.want_trace) keep_trace(iters);
     if (rep_out) *rep_out = rep;
     if (cut_out) *cut_out = h.best_cut;
     if (maxw_out) *maxw_out = h.best_maxw;
@@ -1311,133 +1212,6 @@ int refine_level(Ctx &c, const DGraph &g, int32_t k, double eps, int32_t is_fine
         return JET_ECUDA;
     }
     return refine_level_finish(c, run, cut_out, maxw_out, rep_out);
-}
-
-// ---- batched form: small levels of many graphs ----------------------------
-
-int refine_small_chains(Ctx &c, SmallChain *chains, int32_t nchains, int32_t cluster_blocks, int *ran) {
-    *ran = 0;
-    if (nchains <= 0) {
-        *ran = 1;
-        return JET_OK;
-    }
-    cudaStream_t s = c.stream;
-    JET_TRY(allow_large_arenas(c.device));
-    int32_t kmax = 1;
-    int64_t nlv_total = 0;
-    size_t total = 0;
-    std::vector<size_t> off((size_t)nchains);
-    for (int32_t j = 0; j < nchains; ++j) {
-        const SmallChain &ch = chains[j];
-        int64_t nmax = 1;
-        for (int32_t lv = ch.bottom; lv <= ch.top; ++lv) nmax = std::max<int64_t>(nmax, ch.h->n[lv]);
-        size_t vb = 0, mb = 0;
-        level_bytes(nmax, ch.k, false, &vb, &mb);
-        off[(size_t)j] = total;
-        total += align256(vb) + align256(mb) + 2 * align256((size_t)nmax * 4);
-        nlv_total += ch.top - ch.bottom + 1;
-        kmax = std::max(kmax, ch.k);
-    }
-    const size_t jobs_off = total;
-    const size_t lv_off = jobs_off + align256(sizeof(BatchJob) * (size_t)nchains);
-    const size_t st_off = lv_off + align256(sizeof(BatchLevel) * (size_t)nlv_total);
-    const size_t q_off = st_off + align256(sizeof(BatchStat) * (size_t)nlv_total);
-    DevBuf buf;
-    JET_TRY(dev_alloc(buf, q_off + 256, s));
-    char *base = buf.as<char>();
-    BatchJob *d_jobs = reinterpret_cast<BatchJob *>(base + jobs_off);
-    BatchLevel *d_lv = reinterpret_cast<BatchLevel *>(base + lv_off);
-    BatchStat *d_st = reinterpret_cast<BatchStat *>(base + st_off);
-    int32_t *d_queue = reinterpret_cast<int32_t *>(base + q_off);
-    std::vector<BatchJob> jobs((size_t)nchains);
-    std::vector<BatchLevel> lvs((size_t)nlv_total);
-    int64_t li = 0;
-    for (int32_t j = 0; j < nchains; ++j) {
-        const SmallChain &ch = chains[j];
-        int64_t nmax = 1;
-        for (int32_t lv = ch.bottom; lv <= ch.top; ++lv) nmax = std::max<int64_t>(nmax, ch.h->n[lv]);
-        size_t vb = 0, mb = 0;
-        level_bytes(nmax, ch.k, false, &vb, &mb);
-        char *p = base + off[(size_t)j];
-        BatchJob &jb = jobs[(size_t)j];
-        memset(&jb, 0, sizeof(jb));
-        Level &L = jb.L;
-        carve_level(L, p, p + align256(vb), nmax, ch.k, false, &jb.cut2);
-        fill_level_params(c, L, 0, 0);   // per-level fields (c, seed, graph) are set in the kernel
-        jb.part[0] = reinterpret_cast<int32_t *>(p + align256(vb) + align256(mb));
-        jb.part[1] = jb.part[0] + align256((size_t)nmax * 4) / 4;
-        jb.init = ch.init;
-        jb.out = ch.out;
-        jb.lv = d_lv + li;
-        jb.stat = d_st + li;
-        jb.nlv = ch.top - ch.bottom + 1;
-        jb.Llim = balance_limit(ch.W, ch.k, ch.eps, &jb.opt);
-        jb.sigma = jb.opt + (jb.Llim - jb.opt) / 2;
-        for (int32_t lv = ch.top; lv >= ch.bottom; --lv, ++li) {
-            BatchLevel &bl = lvs[(size_t)li];
-            memset(&bl, 0, sizeof(bl));
-            bl.g.n = ch.h->n[lv]; bl.g.nnz = ch.h->nnz[lv]; bl.g.xadj = ch.h->xadj[lv]; bl.g.adj = ch.h->adj[lv];
-            bl.g.vw = ch.h->vw[lv]; bl.g.ew = ch.h->ew[lv];
-            bl.cmap = ch.h->cmap[lv];
-            bl.seed = level_seed(ch.seed, lv);
-            bl.cq16 = (int32_t)llround((lv == 0 ? c.opt.c_fine : c.opt.c_coarse) * 65536.0);
-        }
-    }
-    // launch shape: clusters of cluster_blocks blocks, as many as are co-resident
-    const size_t smem = cluster_smem(kmax);
-    JET_CUDA_TRY(cudaFuncSetAttribute(k_refine_batch, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    JET_CUDA_TRY(cudaFuncSetAttribute(k_refine_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int cs = cluster_blocks > 0 ? cluster_blocks : 4;
-    int nclusters = 0;
-    for (; cs >= 2; cs /= 2) {
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(cs);
-        cfg.blockDim = dim3(kClusterThreads);
-        cfg.dynamicSmemBytes = smem;
-        cudaLaunchAttribute at{};
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = cs;
-        at.val.clusterDim.y = 1;
-        at.val.clusterDim.z = 1;
-        cfg.attrs = &at;
-        cfg.numAttrs = 1;
-        cudaError_t e = cudaOccupancyMaxActiveClusters(&nclusters, k_refine_batch, &cfg);
-        if (e != cudaSuccess) { cudaGetLastError(); nclusters = 0; }
-        if (nclusters >= 1) break;
-    }
-    if (nclusters < 1) return JET_OK;   // *ran = 0: the caller takes the levels one by one
-    nclusters = std::min(nclusters, nchains);
-    JET_CUDA_TRY(cudaMemcpyAsync(d_jobs, jobs.data(), sizeof(BatchJob) * (size_t)nchains, cudaMemcpyHostToDevice, s));
-    JET_CUDA_TRY(cudaMemcpyAsync(d_lv, lvs.data(), sizeof(BatchLevel) * (size_t)nlv_total, cudaMemcpyHostToDevice, s));
-    JET_CUDA_TRY(cudaMemsetAsync(d_queue, 0, 4, s));
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(nclusters * cs));
-    cfg.blockDim = dim3(kClusterThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = cs;
-    at.val.clusterDim.y = 1;
-    at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    JET_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_refine_batch, (const BatchJob *)d_jobs, nchains, d_queue));
-    c.launches += 1;
-    std::vector<BatchStat> st((size_t)nlv_total);
-    JET_CUDA_TRY(cudaMemcpyAsync(st.data(), d_st, sizeof(BatchStat) * (size_t)nlv_total, cudaMemcpyDeviceToHost, s));
-    JET_CUDA_TRY(cudaStreamSynchronize(s));   // also keeps the host arrays of the copies alive until done
-    li = 0;
-    for (int32_t j = 0; j < nchains; ++j) {
-        SmallChain &ch = chains[j];
-        li += ch.top - ch.bottom + 1;
-        const BatchStat &b = st[(size_t)li - 1];   // the chain's finest level
-        ch.cut = b.best_cut;
-        ch.maxw = b.best_maxw;
-        ch.status = !b.best_bal ? JET_WUNBALANCED : (b.hit_cap ? JET_WITERLIMIT : JET_OK);
-    }
-    *ran = 1;
-    return JET_OK;
 }
 
 // ---- single passes --------------------------------------------------------
