@@ -90,25 +90,18 @@ uint64_t level_seed(uint64_t seed, int32_t level) {
 // ---------------------------------------------------------------------------
 // input checks
 // ---------------------------------------------------------------------------
-struct CheckOut {
-    long long sum_vw, sum_ew, bad;
-};
-
+// The graph check of JET_FLAG_VALIDATE: every entry has its reverse, once,
+// with the same weight; weights are positive; ids in range.
 __global__ void k_check(int32_t n, const int64_t *xadj, const int32_t *adj, const int32_t *vw, const int32_t *ew,
-                        int validate, CheckOut *out) {
+                        unsigned long long *out_bad) {
     __shared__ long long sh[40];
-    long long svw = 0, sew = 0, bad = 0;
+    long long bad = 0;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
         int64_t beg = xadj[v], end = xadj[v + 1];
-        svw += vw ? vw[v] : 1;
-        if (validate) {
-            if (end < beg) { bad = 1; continue; }
-            if (vw && vw[v] <= 0) bad = 1;
-        }
+        if (end < beg) { bad = 1; continue; }
+        if (vw && vw[v] <= 0) bad = 1;
         for (int64_t j = beg; j < end; ++j) {
             int32_t w = ew ? ew[j] : 1;
-            sew += w;
-            if (!validate) continue;
             int32_t u = adj[j];
             if (u < 0 || u >= n || u == (int32_t)v || w <= 0) { bad = 1; continue; }
             // exactly one entry (v, w) in u's row: symmetric and no parallel edge
@@ -120,13 +113,64 @@ __global__ void k_check(int32_t n, const int64_t *xadj, const int32_t *adj, cons
             if (cnt != 1 || !wok) bad = 1;
         }
     }
+    bad = block_sum_i64(bad, sh);
+    if (threadIdx.x == 0 && bad) atomicAdd(out_bad, (unsigned long long)bad);
+}
+
+// f applied to every p[i], i < count, over the whole grid: 16 bytes per load and
+// four loads in flight where the array is aligned.
+template <class F>
+__device__ __forceinline__ void for_each_i32(const int32_t *p, int64_t count, F &&f) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    int64_t done = 0;
+    if ((reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+        const int4 *q = reinterpret_cast<const int4 *>(p);
+        const int64_t n4 = count / 4;
+        for (int64_t i = t; i < n4; i += 4 * stride) {
+            int4 x[4];
+#pragma unroll
+            for (int z = 0; z < 4; ++z)
+                if (i + z * stride < n4) x[z] = __ldcs(q + i + z * stride);
+#pragma unroll
+            for (int z = 0; z < 4; ++z)
+                if (i + z * stride < n4) { f(x[z].x); f(x[z].y); f(x[z].z); f(x[z].w); }
+        }
+        done = n4 * 4;
+    }
+    for (int64_t i = done + t; i < count; i += stride) f(p[i]);
+}
+
+// Input sums and the part range, over the flat arrays: bound by reading them
+// once (a weighted R-MAT graph of scale 20, 32M entries: 1.4 ms before, when
+// one thread walked each row and the longest row set the time).  The last
+// block hands the outcome to the host and clears the state.
+__global__ void __launch_bounds__(kTB) k_check_input(int32_t n, const int64_t *xadj, const int32_t *vw, const int32_t *ew,
+                                                     const int32_t *part, int32_t k, CheckState *st, CheckOut *out) {
+    __shared__ long long sh[40];
+    __shared__ int s_last;
+    const int64_t beg = xadj[0], end = xadj[n];
+    long long svw = 0, sew = 0, bad = 0;
+    if (vw) for_each_i32(vw, n, [&](int32_t x) { svw += x; });
+    if (ew && beg >= 0 && end > beg) for_each_i32(ew + beg, end - beg, [&](int32_t x) { sew += x; });
+    if (part) for_each_i32(part, n, [&](int32_t x) { bad |= x < 0 || x >= k; });
     svw = block_sum_i64(svw, sh);
     sew = block_sum_i64(sew, sh);
     bad = block_sum_i64(bad, sh);
     if (threadIdx.x == 0) {
-        atomic_add_i64(reinterpret_cast<int64_t *>(&out->sum_vw), svw);
-        atomic_add_i64(reinterpret_cast<int64_t *>(&out->sum_ew), sew);
-        if (bad) atomic_add_i64(reinterpret_cast<int64_t *>(&out->bad), bad);
+        if (svw) atomicAdd(&st->sum_vw, (unsigned long long)svw);
+        if (sew) atomicAdd(&st->sum_ew, (unsigned long long)sew);
+        if (bad) atomicAdd(&st->bad_part, (unsigned long long)bad);
+        __threadfence();
+        s_last = atomicAdd(&st->ticket, 1u) == gridDim.x - 1;
+        if (s_last) {
+            __threadfence();
+            out->sum_vw = vw ? (int64_t)atomicExch(&st->sum_vw, 0ull) : n;
+            out->sum_ew = ew ? (int64_t)atomicExch(&st->sum_ew, 0ull) : (end > beg ? end - beg : 0);
+            out->bad_part = (int64_t)atomicExch(&st->bad_part, 0ull);
+            out->bad = 0;
+            out->nnz = end;
+            st->ticket = 0;
+        }
     }
 }
 
@@ -134,40 +178,47 @@ __global__ void k_ones32(int32_t *p, int64_t n) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) p[i] = 1;
 }
 
-__global__ void k_check_part(int32_t n, const int32_t *part, int32_t k, int *bad) {
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
-        if (part[v] < 0 || part[v] >= k) atomicOr(bad, 1);
+int check_input(Ctx &c, int32_t n, const int64_t *xadj, const int32_t *adjncy, const int32_t *vwgt, const int32_t *adjwgt,
+                const int32_t *part, int32_t k, CheckOut &out) {
+    cudaStream_t s = c.stream;
+    // four 16-byte loads a thread and pass; the entry count is not known here
+    const int blocks = adjwgt ? num_sms() * 8 : std::min(num_sms() * 8, grid_for(n, kTB * 16));
+    k_check_input<<<blocks, kTB, 0, s>>>(n, xadj, vwgt, adjwgt, part, k, c.check, reinterpret_cast<CheckOut *>(c.pinned));
+    JET_CUDA_TRY(cudaGetLastError());
+    JET_CUDA_TRY(cudaStreamSynchronize(s));
+    memcpy(&out, c.pinned, sizeof(out));
+    if (out.nnz < 0) return JET_EGRAPH;
+    if (out.nnz > 0 && !adjncy) return JET_EINVAL;
+    return JET_OK;
 }
 
 // Argument checks plus the overflow limits of jet.h (and the full graph
 // check with JET_FLAG_VALIDATE).  Fills g; materialises unit vertex weights
 // into `ones` when vwgt is NULL.
 int prepare_graph(Ctx &c, int32_t n, const int64_t *xadj, const int32_t *adjncy, const int32_t *vwgt,
-                  const int32_t *adjwgt, DGraph &g, DevBuf &ones, bool need_vw) {
+                  const int32_t *adjwgt, DGraph &g, DevBuf &ones, bool need_vw, bool check_part, const int32_t *part,
+                  int32_t k, int64_t *W) {
     if (n < 0 || !xadj) return JET_EINVAL;
     cudaStream_t s = c.stream;
-    int64_t nnz = 0;
-    JET_CUDA_TRY(cudaMemcpyAsync(c.pinned, xadj + n, 8, cudaMemcpyDeviceToHost, s));
-    JET_CUDA_TRY(cudaStreamSynchronize(s));
-    nnz = c.pinned[0];
-    if (nnz < 0) return JET_EGRAPH;
-    if (nnz > 0 && !adjncy) return JET_EINVAL;
-    DevBuf cb;
-    JET_TRY(dev_alloc(cb, sizeof(CheckOut), s));
-    JET_CUDA_TRY(cudaMemsetAsync(cb.p, 0, sizeof(CheckOut), s));
-    int validate = (c.opt.flags & JET_FLAG_VALIDATE) ? 1 : 0;
-    if (n > 0)
-        k_check<<<std::min(num_sms() * 8, grid_for(n, kTB)), kTB, 0, s>>>(n, xadj, adjncy, vwgt, adjwgt, validate,
-                                                                         cb.as<CheckOut>());
-    JET_CUDA_TRY(cudaGetLastError());
-    JET_CUDA_TRY(cudaMemcpyAsync(c.pinned, cb.p, sizeof(CheckOut), cudaMemcpyDeviceToHost, s));
-    JET_CUDA_TRY(cudaStreamSynchronize(s));
     CheckOut h;
-    memcpy(&h, c.pinned, sizeof(h));
-    if (h.bad) return JET_EGRAPH;
+    JET_TRY(check_input(c, n, xadj, adjncy, vwgt, adjwgt, check_part ? part : nullptr, k, h));
+    if (c.opt.flags & JET_FLAG_VALIDATE) {
+        DevBuf cb;
+        JET_TRY(dev_alloc(cb, 16, s));
+        JET_CUDA_TRY(cudaMemsetAsync(cb.p, 0, 16, s));
+        if (n > 0)
+            k_check<<<std::min(num_sms() * 8, grid_for(n, kTB)), kTB, 0, s>>>(n, xadj, adjncy, vwgt, adjwgt,
+                                                                             cb.as<unsigned long long>());
+        JET_CUDA_TRY(cudaGetLastError());
+        JET_CUDA_TRY(cudaMemcpyAsync(c.pinned, cb.p, 8, cudaMemcpyDeviceToHost, s));
+        JET_CUDA_TRY(cudaStreamSynchronize(s));
+        if (c.pinned[0]) return JET_EGRAPH;
+    }
     if (h.sum_vw >= (1LL << 31) || h.sum_ew >= (1LL << 31)) return JET_EOVERFLOW;
+    if (check_part && n > 0 && (!part || h.bad_part)) return JET_EINVAL;
+    if (W) *W = h.sum_vw;
     g.n = n;
-    g.nnz = nnz;
+    g.nnz = h.nnz;
     g.xadj = xadj;
     g.adj = adjncy;
     g.ew = adjwgt;
@@ -179,19 +230,6 @@ int prepare_graph(Ctx &c, int32_t n, const int64_t *xadj, const int32_t *adjncy,
         g.vw = ones.as<int32_t>();
     }
     return JET_OK;
-}
-
-int check_part(Ctx &c, int32_t n, const int32_t *part, int32_t k) {
-    if (n == 0) return JET_OK;
-    if (!part) return JET_EINVAL;
-    DevBuf b;
-    JET_TRY(dev_alloc(b, 16, c.stream));
-    JET_CUDA_TRY(cudaMemsetAsync(b.p, 0, 16, c.stream));
-    k_check_part<<<grid_for(n, kTB, 8192), kTB, 0, c.stream>>>(n, part, k, b.as<int>());
-    JET_CUDA_TRY(cudaGetLastError());
-    JET_CUDA_TRY(cudaMemcpyAsync(c.pinned, b.p, 4, cudaMemcpyDeviceToHost, c.stream));
-    JET_CUDA_TRY(cudaStreamSynchronize(c.stream));
-    return (c.pinned[0] & 0xFFFFFFFF) ? JET_EINVAL : JET_OK;
 }
 
 bool bad_k_eps(int32_t k, double eps) { return k < 1 || k > JET_MAX_K || !(eps >= 0.0) || !std::isfinite(eps); }
@@ -253,9 +291,7 @@ int uncoarsen(Ctx &c, const jet_hier *h, int32_t k, double eps, uint64_t seed, c
     int status = JET_OK;
     int64_t cut = 0, maxw = 0;
     int64_t edge_iters = 0, fin_edge_iters = 0;
-    // every level has the finest graph's total vertex weight (contraction sums them)
-    int64_t W = 0;
-    JET_TRY(total_vweight(c, level_graph(l), W));
+    const int64_t W = h->W;   // every level has the finest graph's total vertex weight (contraction sums them)
     // level boundaries, read once after the loop (no synchronisation per level)
     std::vector<cudaEvent_t> lev;
     struct EvFree {
@@ -473,6 +509,20 @@ int jet_ctx_create(int device, void *cuda_stream, const jet_options *opt, jet_ct
         cudaGetLastError();
         c->c.pool = nullptr;
     }
+    // state of the input checks (zero between them)
+    void *chk = nullptr;
+    cudaError_t e = c->c.pool ? cudaMallocFromPoolAsync(&chk, sizeof(CheckState), c->c.pool, c->c.stream)
+                              : cudaMallocAsync(&chk, sizeof(CheckState), c->c.stream);
+    if (e == cudaSuccess) {
+        c->c.check = static_cast<CheckState *>(chk);
+        e = cudaMemsetAsync(chk, 0, sizeof(CheckState), c->c.stream);
+    }
+    if (e != cudaSuccess) {
+        record_cuda_error(e, "context state", __FILE__, __LINE__);
+        cudaGetLastError();
+        jet_ctx_destroy(c);
+        return e == cudaErrorMemoryAllocation ? JET_ENOMEM : JET_ECUDA;
+    }
     *out = c;
     return JET_OK;
 }
@@ -480,6 +530,7 @@ int jet_ctx_create(int device, void *cuda_stream, const jet_options *opt, jet_ct
 void jet_ctx_destroy(jet_ctx *ctx) {
     if (!ctx) return;
     cudaSetDevice(ctx->c.device);
+    if (ctx->c.check) cudaFreeAsync(ctx->c.check, ctx->c.stream);
     cudaStreamSynchronize(ctx->c.stream);
     if (ctx->c.pinned) cudaFreeHost(ctx->c.pinned);
     if (t_pool == ctx->c.pool) t_pool = nullptr;
@@ -497,10 +548,12 @@ int jet_coarsen(jet_ctx *ctx, int32_t n, const int64_t *xadj, const int32_t *adj
     JET_TRY(use_device(c));
     DGraph g;
     DevBuf ones;
-    JET_TRY(prepare_graph(c, n, xadj, adjncy, vwgt, adjwgt, g, ones, false));
+    int64_t W = 0;
+    JET_TRY(prepare_graph(c, n, xadj, adjncy, vwgt, adjwgt, g, ones, false, false, nullptr, 0, &W));
     jet_hier *h = new (std::nothrow) jet_hier;
     if (!h) return JET_ENOMEM;
     h->ctx = ctx;
+    h->W = W;
     EventTimer ev;
     cudaEventRecord(ev.e[0], c.stream);
     int64_t l0 = c.launches;
@@ -585,7 +638,7 @@ int jet_coarsest_refined(jet_ctx *ctx, const jet_hier *h, int32_t k, double eps,
     JET_TRY(initial_partition(c, g, k, part_out));
     int64_t cut = 0, maxw = 0;
     LevelReport rep;
-    int r = refine_level(c, g, k, eps, l == 0, level_seed(seed, l), part_out, &cut, &maxw, &rep);
+    int r = refine_level(c, g, k, eps, l == 0, level_seed(seed, l), part_out, &cut, &maxw, &rep, h->W);
     if (r < 0) return r;
     JET_TRY(sync_stream(c));
     if (cut_out) *cut_out = cut;
@@ -600,15 +653,15 @@ int jet_refine(jet_ctx *ctx, int32_t n, const int64_t *xadj, const int32_t *adjn
     JET_TRY(use_device(c));
     DGraph g;
     DevBuf ones;
-    JET_TRY(prepare_graph(c, n, xadj, adjncy, vwgt, adjwgt, g, ones, true));
-    JET_TRY(check_part(c, n, part_inout, k));
+    int64_t W = 0;
+    JET_TRY(prepare_graph(c, n, xadj, adjncy, vwgt, adjwgt, g, ones, true, true, part_inout, k, &W));
     if (n == 0) {
         if (cut_out) *cut_out = 0;
         c.last_trace.rec.clear();
         c.last_trace.iters = 0;
         return JET_OK;
     }
-    return refine_level(c, g, k, eps, is_finest ? 1 : 0, seed, part_inout, cut_out, nullptr, nullptr);
+    return refine_level(c, g, k, eps, is_finest ? 1 : 0, seed, part_inout, cut_out, nullptr, nullptr, W);
 }
 
 int jet_last_trace(jet_ctx *ctx, int32_t cap, int32_t *kind, int64_t *nx, int64_t *nm, int64_t *cut, int64_t *maxw,
@@ -838,8 +891,7 @@ int jet_cut(jet_ctx *ctx, int32_t n, const int64_t *xadj, const int32_t *adjncy,
     JET_TRY(use_device(c));
     DGraph g;
     DevBuf ones;
-    JET_TRY(prepare_graph(c, n, xadj, adjncy, vwgt, adjwgt, g, ones, true));
-    JET_TRY(check_part(c, n, part, k));
+    JET_TRY(prepare_graph(c, n, xadj, adjncy, vwgt, adjwgt, g, ones, false, true, part, k));
     return cut_and_weights(c, g, k, part, cut_out, pw_out);
 }
 
@@ -852,8 +904,7 @@ int jet_lp_pass(jet_ctx *ctx, int32_t n, const int64_t *xadj, const int32_t *adj
     JET_TRY(use_device(c));
     DGraph g;
     DevBuf ones;
-    JET_TRY(prepare_graph(c, n, xadj, adjncy, vwgt, adjwgt, g, ones, true));
-    JET_TRY(check_part(c, n, part, k));
+    JET_TRY(prepare_graph(c, n, xadj, adjncy, vwgt, adjwgt, g, ones, false, true, part, k));
     return lp_pass(c, g, k, part, locked, cval, flags, pd_out, gain_out, inx_out, f2_out, inm_out);
 }
 
@@ -866,9 +917,9 @@ int jet_rebalance_pass(jet_ctx *ctx, int32_t n, const int64_t *xadj, const int32
     JET_TRY(use_device(c));
     DGraph g;
     DevBuf ones;
-    JET_TRY(prepare_graph(c, n, xadj, adjncy, vwgt, adjwgt, g, ones, true));
-    JET_TRY(check_part(c, n, part, k));
-    return rebalance_pass(c, g, k, eps, strong, seed, iter, part, dest_out, loss_out, nmoves_out, ncand_out);
+    int64_t W = 0;
+    JET_TRY(prepare_graph(c, n, xadj, adjncy, vwgt, adjwgt, g, ones, true, true, part, k, &W));
+    return rebalance_pass(c, g, W, k, eps, strong, seed, iter, part, dest_out, loss_out, nmoves_out, ncand_out);
 }
 
 int jet_hem(jet_ctx *ctx, int32_t n, const int64_t *xadj, const int32_t *adjncy, const int32_t *adjwgt, uint64_t seed,
@@ -878,7 +929,7 @@ int jet_hem(jet_ctx *ctx, int32_t n, const int64_t *xadj, const int32_t *adjncy,
     JET_TRY(use_device(c));
     DGraph g;
     DevBuf ones;
-    JET_TRY(prepare_graph(c, n, xadj, adjncy, nullptr, adjwgt, g, ones, true));
+    JET_TRY(prepare_graph(c, n, xadj, adjncy, nullptr, adjwgt, g, ones, false));
     JET_TRY(hem(c, g, seed, level, rounds, mate_out));
     return sync_stream(c);
 }

@@ -98,6 +98,16 @@ struct DGraph {
     const int32_t *ew = nullptr;   // null: unit edge weights
 };
 
+// Outcome of the input checks, written into pinned host memory, and the
+// device state of the kernel that makes them (zero between its launches).
+struct CheckOut {
+    int64_t sum_vw, sum_ew, bad, bad_part, nnz;
+};
+struct CheckState {
+    unsigned long long sum_vw, sum_ew, bad_part;
+    uint32_t ticket, pad;
+};
+
 // ---------------------------------------------------------------------------
 // device control block of one refinement level (Alg. 3 state)
 // ---------------------------------------------------------------------------
@@ -486,6 +496,7 @@ struct ResStat {
 // is enqueued, read after the last level), then the finest level's trace,
 // then one outcome per level of a resident chain.
 constexpr size_t kPinnedScalarBytes = 4096;
+static_assert(sizeof(Ctl) <= kPinnedScalarBytes && sizeof(CheckOut) <= kPinnedScalarBytes, "scalar readbacks");
 constexpr size_t kPinnedCtlStride = (sizeof(Ctl) + 255) & ~size_t(255);
 constexpr size_t kPinnedCtlOff = kPinnedScalarBytes;
 constexpr size_t kPinnedTraceOff = kPinnedCtlOff + kPinnedCtlStride * JET_MAX_LEVELS;
@@ -498,6 +509,7 @@ struct Ctx {
     cudaStream_t stream = nullptr;
     jet_options opt{};
     int64_t *pinned = nullptr;   // pinned host buffer (layout: kPinned* below)
+    CheckState *check = nullptr; // device: state of the input checks
     cudaMemPool_t pool = nullptr; // the context's stream-ordered pool (keeps its memory between calls)
     TraceHost last_trace;
 };
@@ -514,6 +526,7 @@ struct jet_hier {
     jet_ctx *ctx = nullptr;
     int32_t levels = 0;
     int32_t k = 0;
+    int64_t W = 0;            // total vertex weight (every level's)
     int32_t n[JET_MAX_LEVELS] = {};
     int64_t nnz[JET_MAX_LEVELS] = {};
     const int64_t *xadj[JET_MAX_LEVELS] = {};
@@ -570,11 +583,9 @@ int resident_enqueue(Ctx &c, const ResChainLevel *lv, int32_t nlv, int32_t k, do
                      const int32_t *init, bool want_trace);
 uint64_t level_seed(uint64_t seed, int32_t level);   // Jetrw seed of hierarchy level `level`
 
-// Enqueue + synchronise + finish.  W_known: -1 = computed on the device.
+// Enqueue + synchronise + finish.
 int refine_level(Ctx &c, const DGraph &g, int32_t k, double eps, int32_t is_finest, uint64_t seed,
-                 int32_t *part_inout, int64_t *cut_out, int64_t *maxw_out, LevelReport *rep, int64_t W_known = -1);
-// Sum of the vertex weights (one device reduction and a readback).
-int total_vweight(Ctx &c, const DGraph &g, int64_t &W);
+                 int32_t *part_inout, int64_t *cut_out, int64_t *maxw_out, LevelReport *rep, int64_t W);
 int lp_pass(Ctx &c, const DGraph &g, int32_t k, const int32_t *part, const uint8_t *locked, double cval,
             uint32_t flags, int32_t *pd_out, int32_t *gain_out, uint8_t *inx_out, int32_t *f2_out,
             uint8_t *inm_out);
@@ -589,7 +600,7 @@ constexpr size_t lp_scratch_bytes(int64_t n) {
 int lp_pass_in_scratch(Ctx &c, const DGraph &g, int32_t k, const int32_t *part, const uint8_t *locked, double cval,
                        uint32_t flags, int32_t *pd_out, int32_t *gain_out, uint8_t *inx_out, int32_t *f2_out,
                        uint8_t *inm_out, char *scratch);
-int rebalance_pass(Ctx &c, const DGraph &g, int32_t k, double eps, int32_t strong, uint64_t seed, int32_t iter,
+int rebalance_pass(Ctx &c, const DGraph &g, int64_t W, int32_t k, double eps, int32_t strong, uint64_t seed, int32_t iter,
                    const int32_t *part, int32_t *dest_out, int32_t *loss_out, int64_t *nmoves, int64_t *ncand);
 int cut_and_weights(Ctx &c, const DGraph &g, int32_t k, const int32_t *part, int64_t *cut_out, int64_t *pw_dev);
 
@@ -633,9 +644,15 @@ int64_t balance_limit(int64_t W, int32_t k, double eps, int64_t *opt);
 int sync_stream(Ctx &c);
 int use_device(Ctx &c);
 bool bad_k_eps(int32_t k, double eps);
-int check_part(Ctx &c, int32_t n, const int32_t *part, int32_t k);   // JET_EINVAL unless every part is in [0, k)
+// Weight sums, entry count and (part not null) the part range of an input in
+// one launch and one host wait; JET_OK when the sums could be taken.
+int check_input(Ctx &c, int32_t n, const int64_t *xadj, const int32_t *adjncy, const int32_t *vwgt, const int32_t *adjwgt,
+                const int32_t *part, int32_t k, CheckOut &out);
+// Argument and overflow checks; fills g (W: the total vertex weight).  With
+// check_part also JET_EINVAL unless every part is in [0, k).
 int prepare_graph(Ctx &c, int32_t n, const int64_t *xadj, const int32_t *adjncy, const int32_t *vwgt,
-                  const int32_t *adjwgt, DGraph &g, DevBuf &ones, bool need_vw);
+                  const int32_t *adjwgt, DGraph &g, DevBuf &ones, bool need_vw, bool check_part = false,
+                  const int32_t *part = nullptr, int32_t k = 0, int64_t *W = nullptr);
 // Alg. 1 after coarsening; init_coarsest (device, n of the coarsest level)
 // replaces the greedy initial partition when not null.
 int uncoarsen(Ctx &c, const jet_hier *h, int32_t k, double eps, uint64_t seed, const int32_t *init_coarsest,

@@ -870,8 +870,7 @@ int jet_lip_labels(jet_ctx *ctx, int32_t n, const int64_t *xadj, const int32_t *
     JET_TRY(use_device(c));
     DGraph g;
     DevBuf ones;
-    JET_TRY(graph_of(c, n, xadj, adjncy, nullptr, nullptr, g, ones));
-    JET_TRY(check_part(c, n, part, k));
+    JET_TRY(prepare_graph(c, n, xadj, adjncy, nullptr, nullptr, g, ones, true, true, part, k));
     if (n == 0) return JET_OK;
     DevBuf buf;
     const size_t kb = align256c((size_t)k * 8);

@@ -14,37 +14,12 @@
 
 namespace jet {
 
-constexpr size_t kNoallocCheckBytes = 256;
-constexpr size_t kNoallocCheckOffset = lp_scratch_bytes(JET_NOALLOC_MAX_N);
-constexpr size_t kNoallocBytes = kNoallocCheckOffset + kNoallocCheckBytes;
+constexpr size_t kNoallocBytes = lp_scratch_bytes(JET_NOALLOC_MAX_N);
 
 // The whole scratch of jet_lp_pass_noalloc (about 10 MiB), shared by every
 // call on a device.  In host code this name is only a stand-in: the device
 // address comes from cudaGetSymbolAddress below.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocBytes];
-
-// Overflow limits of jet.h and the part range, written into the check slot at
-// the end of the array (sum_vw, sum_ew, bad part).
-__global__ void k_noalloc_check(int32_t n, const int64_t *xadj, const int32_t *vw, const int32_t *ew,
-                                const int32_t *part, int32_t k) {
-    __shared__ long long sh[40];
-    long long *out = reinterpret_cast<long long *>(g_noalloc_scratch + kNoallocCheckOffset);
-    long long svw = 0, sew = 0, bad = 0;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-        svw += vw ? vw[v] : 1;
-        int64_t e = xadj[v + 1];
-        for (int64_t j = xadj[v]; j < e; ++j) sew += ew ? ew[j] : 1;
-        if (part[v] < 0 || part[v] >= k) bad = 1;
-    }
-    svw = block_sum_i64(svw, sh);
-    sew = block_sum_i64(sew, sh);
-    bad = block_sum_i64(bad, sh);
-    if (threadIdx.x == 0) {
-        atomic_add_i64(reinterpret_cast<int64_t *>(&out[0]), svw);
-        atomic_add_i64(reinterpret_cast<int64_t *>(&out[1]), sew);
-        if (bad) atomic_add_i64(reinterpret_cast<int64_t *>(&out[2]), bad);
-    }
-}
 
 // Device address of g_noalloc_scratch, looked up once per device with that
 // device current.
@@ -87,23 +62,13 @@ extern "C" int jet_lp_pass_noalloc(jet_ctx *ctx, int32_t n, const int64_t *xadj,
     JET_TRY(noalloc_scratch(c.device, &scratch));
     if (n == 0) return JET_OK;
     if (!part) return JET_EINVAL;
-    cudaStream_t s = c.stream;
-    JET_CUDA_TRY(cudaMemcpyAsync(c.pinned, xadj + n, 8, cudaMemcpyDeviceToHost, s));
-    JET_CUDA_TRY(cudaStreamSynchronize(s));
-    int64_t nnz = c.pinned[0];
-    if (nnz < 0) return JET_EGRAPH;
-    if (nnz > 0 && !adjncy) return JET_EINVAL;
-    char *check = scratch + kNoallocCheckOffset;
-    JET_CUDA_TRY(cudaMemsetAsync(check, 0, kNoallocCheckBytes, s));
-    k_noalloc_check<<<std::min(num_sms() * 8, grid_for(n, kTB)), kTB, 0, s>>>(n, xadj, vwgt, adjwgt, part, k);
-    JET_CUDA_TRY(cudaGetLastError());
-    JET_CUDA_TRY(cudaMemcpyAsync(c.pinned, check, 24, cudaMemcpyDeviceToHost, s));
-    JET_CUDA_TRY(cudaStreamSynchronize(s));
-    if (c.pinned[2]) return JET_EINVAL;
-    if (c.pinned[0] >= (1LL << 31) || c.pinned[1] >= (1LL << 31)) return JET_EOVERFLOW;
+    CheckOut h;
+    JET_TRY(check_input(c, n, xadj, adjncy, vwgt, adjwgt, part, k, h));
+    if (h.bad_part) return JET_EINVAL;
+    if (h.sum_vw >= (1LL << 31) || h.sum_ew >= (1LL << 31)) return JET_EOVERFLOW;
     DGraph g;
     g.n = n;
-    g.nnz = nnz;
+    g.nnz = h.nnz;
     g.xadj = xadj;
     g.adj = adjncy;
     g.vw = vwgt;   // the Jetlp pass never reads vertex weights

@@ -39,7 +39,8 @@ extern __shared__ __align__(16) unsigned char jet_arena[];
 template <bool EW>
 __device__ inline void ph_cut_pw(const DGraph &g, int32_t k, const int32_t *__restrict__ part,
                                  int64_t *__restrict__ pw, int64_t *__restrict__ cut2, int32_t *__restrict__ ext,
-                                 int32_t *__restrict__ wdeg, Grid G, char *arena) {
+                                 int32_t *__restrict__ wdeg, Grid G, char *arena, int32_t *nbig = nullptr) {
+    bool anybig = false;
     long long *shpw = reinterpret_cast<long long *>(arena);
     int32_t *stage = reinterpret_cast<int32_t *>(arena + align16((size_t)k * 8));
     __shared__ long long red[40];
@@ -105,20 +106,15 @@ __device__ inline void ph_cut_pw(const DGraph &g, int32_t k, const int32_t *__re
             const int32_t p = part[v];
             atomicAdd(reinterpret_cast<unsigned long long *>(&shpw[p]), (unsigned long long)(long long)(g.vw ? g.vw[v] : 1));
             const int64_t b = ld_xadj(g.xadj, v), e = ld_xadj(g.xadj, v + 1);
+            anybig |= e - b > kSmallDeg;
             if (e - b > 2 * kSmallDeg) {
                 big = true;
             } else {
-                int32_t nx = 0, wd = 0, cv = 0;
-                for (int64_t j = b; j < e; ++j) {
-                    const int32_t w = edge_w<EW>(g, j);
-                    const bool other = part[g.adj[j]] != p;
-                    cv += other ? w : 0;
-                    nx += other ? 1 : 0;
-                    wd += w;
-                }
+                long long cv = 0, nx = 0, wd = 0;
+                row_share(b, e, 1, p, cv, nx, wd);
                 c += cv;
-                if (ext) ext[v] = nx;
-                if (wdeg) wdeg[v] = wd;
+                if (ext) ext[v] = (int32_t)nx;
+                if (wdeg) wdeg[v] = (int32_t)wd;
             }
         }
         bigs.add(big, (int32_t)v);
@@ -127,6 +123,7 @@ __device__ inline void ph_cut_pw(const DGraph &g, int32_t k, const int32_t *__re
     bigs.drain(true, g.xadj, warp_row, block_row);
     c = block_sum_i64(c, red);
     if (threadIdx.x == 0 && c) atomic_add_i64(cut2, c);
+    if (nbig && __syncthreads_or(anybig) && threadIdx.x == 0) atomicAdd(nbig, 1);   // only whether there are any matters
     __syncthreads();
     for (int i = threadIdx.x; i < k; i += blockDim.x)
         if (shpw[i]) atomic_add_i64(&pw[i], shpw[i]);
@@ -136,8 +133,9 @@ __device__ inline void ph_cut_pw(const DGraph &g, int32_t k, const int32_t *__re
 template <bool EW>
 __global__ void __launch_bounds__(kTB) k_cut_pw(DGraph g, int32_t k, const int32_t *__restrict__ part,
                                                  int64_t *__restrict__ pw, int64_t *__restrict__ cut2,
-                                                 int32_t *__restrict__ ext, int32_t *__restrict__ wdeg) {
-    ph_cut_pw<EW>(g, k, part, pw, cut2, ext, wdeg, launch_grid(), reinterpret_cast<char *>(jet_arena));
+                                                 int32_t *__restrict__ ext, int32_t *__restrict__ wdeg, int32_t *nbig) {
+    pdl_enter();
+    ph_cut_pw<EW>(g, k, part, pw, cut2, ext, wdeg, launch_grid(), reinterpret_cast<char *>(jet_arena), nbig);
 }
 
 // dynamic shared memory of k_cut_pw
@@ -158,6 +156,7 @@ size_t sm_cut_pw(int32_t k) { return align16((size_t)k * 8) + (size_t)kBigCap * 
 // from the initial cut and part weights.
 __global__ void __launch_bounds__(1024) k_ctl_init(Level L, const int64_t *cut2, int64_t Llim, int64_t opt,
                                                    int64_t sigma) {
+    pdl_enter();
     if (threadIdx.x == 0) {
         L.ctl->L = Llim;
         L.ctl->opt = opt;
@@ -425,27 +424,68 @@ __global__ void __launch_bounds__(kTB, JET_ROW_MINB) k_refine_grid(Level L) {
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-// Vertices with rows longer than kSmallDeg (only whether there are any
-// matters), counted into the level's control block.
-__global__ void k_count_big(DGraph g, int32_t *count) {
-    int32_t v = blockIdx.x * blockDim.x + threadIdx.x;
-    bool big = v < g.n && ld_xadj(g.xadj, (int64_t)v + 1) - ld_xadj(g.xadj, v) > kSmallDeg;
-    unsigned m = __ballot_sync(0xffffffffu, big);
-    if (lane_id() == 0 && m) atomicAdd(count, __popc(m));
-}
-
-__global__ void k_fill_i32(int32_t *p, int64_t n, int32_t val) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        p[i] = val;
-}
-
-__global__ void k_sum_vw(DGraph g, int64_t *out) {
-    __shared__ long long red[40];
-    long long s = 0;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < g.n; v += (int64_t)gridDim.x * blockDim.x)
-        s += g.vw[v];
-    s = block_sum_i64(s, red);
-    if (threadIdx.x == 0 && s) atomic_add_i64(out, s);
+// Start values of a level's arrays in one pass over the vertices (one launch
+// where the fills, the copies and the clearing of the control block took up to
+// ten): stamps, priorities, the best partition, and what the single passes add
+// (null pointers are left out): locks from a mask, rebalancing keys, defaults of
+// the Jetlp outputs.
+struct LevelInit {
+    const uint8_t *locked;        // lock mask (only with use_locked; null: nothing locked)
+    int32_t *best, *key;          // = part, = -1
+    int32_t *pd, *gain, *f2;      // = part, = kNoneGain, = 0
+    int64_t *cut2;
+    int32_t use_locked;
+};
+__global__ void __launch_bounds__(kTB) k_level_init(Level L, LevelInit a) {
+    pdl_enter();
+    if (blockIdx.x == 0) {
+        int64_t *w = reinterpret_cast<int64_t *>(L.ctl);
+        for (int i = threadIdx.x; i < (int)(sizeof(Ctl) / 8); i += blockDim.x) w[i] = 0;
+        for (int i = threadIdx.x; i < L.k; i += blockDim.x) L.pw[i] = 0;
+        if (threadIdx.x < 2) a.cut2[threadIdx.x] = 0;
+    }
+    const int64_t n = L.g.n, nq = (n + 3) / 4;
+    const bool vec = (reinterpret_cast<uintptr_t>(L.part) & 15) == 0;
+    auto put = [&](int32_t *p, int64_t v0, int m, int4 x) {   // the library's own arrays are 256-byte aligned, the caller's may not be
+        if (m == 4 && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+            *reinterpret_cast<int4 *>(p + v0) = x;
+            return;
+        }
+        const int32_t e[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (i < m) p[v0 + i] = e[i];
+    };
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nq; q += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t v0 = 4 * q;
+        const int m = (int)min((int64_t)4, n - v0);
+        const int4 none = make_int4(-2, -2, -2, -2), gain = make_int4(kNoneGain, kNoneGain, kNoneGain, kNoneGain);
+        int4 p = make_int4(0, 0, 0, 0), lock = none;
+        if (a.best || a.pd) {
+            if (m == 4 && vec) {
+                p = *reinterpret_cast<const int4 *>(L.part + v0);
+            } else {
+                p.x = L.part[v0];
+                if (m > 1) p.y = L.part[v0 + 1];
+                if (m > 2) p.z = L.part[v0 + 2];
+                if (m > 3) p.w = L.part[v0 + 3];
+            }
+        }
+        if (a.use_locked && a.locked) {
+            if (a.locked[v0]) lock.x = 0;
+            if (m > 1 && a.locked[v0 + 1]) lock.y = 0;
+            if (m > 2 && a.locked[v0 + 2]) lock.z = 0;
+            if (m > 3 && a.locked[v0 + 3]) lock.w = 0;
+        }
+        put(L.lstamp, v0, m, lock);
+        put(L.mstamp, v0, m, none);
+        put(L.prio, v0, m, gain);
+        if (a.best) put(a.best, v0, m, p);
+        if (a.key) put(a.key, v0, m, make_int4(-1, -1, -1, -1));
+        if (a.pd) put(a.pd, v0, m, p);
+        if (a.gain) put(a.gain, v0, m, gain);
+        if (a.f2) put(a.f2, v0, m, make_int4(0, 0, 0, 0));
+    }
 }
 
 namespace {
@@ -508,8 +548,7 @@ void carve_level(Level &L, char *vert, char *misc, int64_t nmax, int32_t k, bool
     L.k = k;
 }
 
-// Buffers and start state of one level, enqueued on the context's stream (no
-// host wait): the control block gets the level's long-row count.
+// Buffers of one level.
 int setup_level(Ctx &c, const DGraph &g, int32_t k, LevelBufs &B) {
     JET_TRY(allow_large_arenas(c.device));
     cudaStream_t s = c.stream;
@@ -521,16 +560,6 @@ int setup_level(Ctx &c, const DGraph &g, int32_t k, LevelBufs &B) {
     Level &L = B.L;
     carve_level(L, B.vert.as<char>(), B.misc.as<char>(), n, k, true, &B.cut2);
     L.g = g;
-    JET_CUDA_TRY(cudaMemsetAsync(L.ctl, 0, sizeof(Ctl), s));
-    JET_CUDA_TRY(cudaMemsetAsync(L.pw, 0, (size_t)k * 8, s));
-    JET_CUDA_TRY(cudaMemsetAsync(B.cut2, 0, 16, s));
-    if (n > 0) {
-        k_count_big<<<grid_for(n, kTB), kTB, 0, s>>>(g, &L.ctl->nbig);
-        k_fill_i32<<<grid_for(n, kTB, 4096), kTB, 0, s>>>(L.lstamp, n, -2);
-        k_fill_i32<<<grid_for(n, kTB, 4096), kTB, 0, s>>>(L.mstamp, n, -2);
-        k_fill_i32<<<grid_for(n, kTB, 4096), kTB, 0, s>>>(L.prio, n, kNoneGain);
-    }
-    JET_CUDA_TRY(cudaGetLastError());
     return JET_OK;
 }
 
@@ -678,27 +707,31 @@ int enqueue_final_copy(const Level &L, cudaStream_t s) {
     return JET_OK;
 }
 
-// Level start: part weights, cut, control block, P_best = P_0 (no host wait).
-int enqueue_init(Ctx &c, LevelBufs &B, int64_t L_lim, int64_t opt, int64_t sigma) {
+// Start values, then ext, the weighted degrees (wdeg), part weights, twice the
+// cut and whether there are long rows (into the control block).  No host wait.
+int enqueue_start(Ctx &c, const Level &L, const LevelInit &init, int32_t *wdeg) {
     cudaStream_t s = c.stream;
-    Level &L = B.L;
-    int64_t n = L.g.n;
+    const int64_t n = L.g.n;
+    JET_CUDA_TRY(launch_pdl(k_level_init, grid_for((n + 3) / 4, kTB, num_sms() * 8), kTB, 0, s, false, L, init));
+    c.launches += 1;
     if (n > 0) {
-        int gcut = std::min(list_grid(), grid_for(n, kTB));
-        if (L.g.ew) k_cut_pw<true><<<gcut, kTB, sm_cut_pw(L.k), s>>>(L.g, L.k, L.part, L.pw, B.cut2, L.ext, L.wdeg);
-        else k_cut_pw<false><<<gcut, kTB, sm_cut_pw(L.k), s>>>(L.g, L.k, L.part, L.pw, B.cut2, L.ext, L.wdeg);
+        const int gcut = std::min(list_grid(), grid_for(n, kTB));
+        JET_CUDA_TRY(launch_pdl(L.g.ew ? k_cut_pw<true> : k_cut_pw<false>, gcut, kTB, sm_cut_pw(L.k), s, true, L.g, L.k,
+                                (const int32_t *)L.part, L.pw, init.cut2, L.ext, wdeg, &L.ctl->nbig));
         c.launches += 1;
     }
-    k_ctl_init<<<1, 1024, 0, s>>>(L, B.cut2, L_lim, opt, sigma);
-    c.launches += 1;
-    if (n > 0) JET_CUDA_TRY(cudaMemcpyAsync(L.best, L.part, (size_t)n * 4, cudaMemcpyDeviceToDevice, s));
-    JET_CUDA_TRY(cudaGetLastError());
     return JET_OK;
 }
 
-int read_ctl(Ctx &c, const Level &L, Ctl &h) {
-    JET_CUDA_TRY(cudaMemcpyAsync(&h, L.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, c.stream));
-    JET_CUDA_TRY(cudaStreamSynchronize(c.stream));
+// Level start: part weights, cut, control block, P_best = P_0.
+int enqueue_init(Ctx &c, LevelBufs &B, int64_t L_lim, int64_t opt, int64_t sigma) {
+    const Level &L = B.L;
+    LevelInit init{};
+    init.best = L.best;
+    init.cut2 = B.cut2;
+    JET_TRY(enqueue_start(c, L, init, L.wdeg));
+    JET_CUDA_TRY(launch_pdl(k_ctl_init, 1, 1024, 0, c.stream, true, L, (const int64_t *)B.cut2, L_lim, opt, sigma));
+    c.launches += 1;
     return JET_OK;
 }
 
@@ -1002,22 +1035,6 @@ int run_cluster(Ctx &c, const Level &L, int cs) {
 
 }  // namespace
 
-// Weight of the whole graph (needed for the balance limit).
-int total_vweight(Ctx &c, const DGraph &g, int64_t &W) {
-    DevBuf t;
-    JET_TRY(dev_alloc(t, 16, c.stream));
-    JET_CUDA_TRY(cudaMemsetAsync(t.p, 0, 16, c.stream));
-    if (g.n > 0) {
-        k_sum_vw<<<std::min(list_grid(), grid_for(g.n, kTB)), kTB, 0, c.stream>>>(g, t.as<int64_t>());
-        c.launches += 1;
-    }
-    JET_CUDA_TRY(cudaGetLastError());
-    JET_CUDA_TRY(cudaMemcpyAsync(c.pinned, t.p, 8, cudaMemcpyDeviceToHost, c.stream));
-    JET_CUDA_TRY(cudaStreamSynchronize(c.stream));
-    W = c.pinned[0];
-    return JET_OK;
-}
-
 // Blocks of the rebalancing scan resident on one SM (per device, once).
 static int rb_scan_resident() {
     static std::mutex mu;
@@ -1083,7 +1100,6 @@ int refine_level_enqueue(Ctx &c, const DGraph &g, int32_t k, double eps, int32_t
     int64_t sigma = opt + (L_lim - opt) / 2;
     LevelBufs B;
     JET_TRY(setup_level(c, g, k, B));
-    c.launches += g.n > 0 ? 4 : 0;
     Level &L = B.L;
     L.part = part_inout;
     fill_level_params(c, L, is_finest, seed);
@@ -1194,9 +1210,7 @@ int refine_level_finish(Ctx &c, LevelRun &run, int64_t *cut_out, int64_t *maxw_o
 }
 
 int refine_level(Ctx &c, const DGraph &g, int32_t k, double eps, int32_t is_finest, uint64_t seed,
-                 int32_t *part_inout, int64_t *cut_out, int64_t *maxw_out, LevelReport *rep_out, int64_t W_known) {
-    int64_t W = W_known;
-    if (W < 0) JET_TRY(total_vweight(c, g, W));
+                 int32_t *part_inout, int64_t *cut_out, int64_t *maxw_out, LevelReport *rep_out, int64_t W) {
     LevelRun run;
     run.slot = 0;
     run.want_trace = true;
@@ -1216,25 +1230,36 @@ int refine_level(Ctx &c, const DGraph &g, int32_t k, double eps, int32_t is_fine
 
 // ---- single passes --------------------------------------------------------
 
-__global__ void k_locks_from_mask(const uint8_t *locked, int32_t *lstamp, int64_t n) {
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
-        lstamp[v] = (locked && locked[v]) ? 0 : -2;
-}
-
-__global__ void k_set_epoch(Ctl *ctl, int32_t epoch, int32_t mode) {
-    ctl->lp_epoch = epoch;
-    ctl->mode = mode;
-    ctl->it = 0;
-    ctl->ticket = 0;
-    reset_counters(ctl);
-}
-
 __global__ void k_export_lp(Level L, uint8_t *inx, uint8_t *inm) {
     const int32_t it = L.ctl->it;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < L.g.n; v += (int64_t)gridDim.x * blockDim.x) {
         if (inx) inx[v] = L.prio[v] != kNoneGain;
         if (inm) inm[v] = L.mstamp[v] == it;
     }
+}
+
+// The pass on a level whose arrays are in place (ex: every output set).  The
+// cleared control block says Jetlp, iteration 0, locks of epoch 0.
+static int run_lp_pass(Ctx &c, Level &L, int64_t *cut2, const uint8_t *locked, double cval, uint32_t flags, LpExport ex,
+                       uint8_t *inx_out, uint8_t *inm_out) {
+    cudaStream_t s = c.stream;
+    fill_level_params(c, L, 1, 0);
+    L.cq16 = (int32_t)llround(cval * 65536.0);
+    L.abl = flags & ABL_ALL;
+    LevelInit init{};
+    init.locked = locked;
+    init.use_locked = 1;
+    init.pd = ex.pd;       // the select writes P_d and F only for the vertices it examines
+    init.gain = ex.gain;
+    init.f2 = ex.f2;
+    init.cut2 = cut2;
+    JET_TRY(enqueue_start(c, L, init, nullptr));
+    int nk = 0;
+    JET_TRY(enqueue_lp(L, s, &nk, ex));
+    k_export_lp<<<grid_for(L.g.n, kTB, 4096), kTB, 0, s>>>(L, inx_out, inm_out);
+    JET_CUDA_TRY(cudaGetLastError());
+    JET_CUDA_TRY(cudaStreamSynchronize(s));
+    return JET_OK;
 }
 
 int lp_pass(Ctx &c, const DGraph &g, int32_t k, const int32_t *part, const uint8_t *locked, double cval, uint32_t flags,
@@ -1245,16 +1270,6 @@ int lp_pass(Ctx &c, const DGraph &g, int32_t k, const int32_t *part, const uint8
     JET_TRY(setup_level(c, g, k, B));
     Level &L = B.L;
     L.part = const_cast<int32_t *>(part);   // read only in this pass
-    fill_level_params(c, L, 1, 0);
-    L.cq16 = (int32_t)llround(cval * 65536.0);
-    L.abl = flags & ABL_ALL;
-    {
-        int gcut = std::min(list_grid(), grid_for(g.n, kTB));
-        if (g.ew) k_cut_pw<true><<<gcut, kTB, sm_cut_pw(k), s>>>(g, k, L.part, L.pw, B.cut2, L.ext, nullptr);
-        else k_cut_pw<false><<<gcut, kTB, sm_cut_pw(k), s>>>(g, k, L.part, L.pw, B.cut2, L.ext, nullptr);
-    }
-    k_locks_from_mask<<<grid_for(g.n, kTB, 4096), kTB, 0, s>>>(locked, L.lstamp, g.n);
-    k_set_epoch<<<1, 1, 0, s>>>(L.ctl, 0, MODE_LP);
     DevBuf tmp_pd, tmp_gain;
     LpExport ex{pd_out, gain_out, f2_out};
     if (!ex.pd || !ex.gain) {
@@ -1263,16 +1278,7 @@ int lp_pass(Ctx &c, const DGraph &g, int32_t k, const int32_t *part, const uint8
         if (!ex.pd) ex.pd = tmp_pd.as<int32_t>();
         if (!ex.gain) ex.gain = tmp_gain.as<int32_t>();
     }
-    if (f2_out) JET_CUDA_TRY(cudaMemsetAsync(f2_out, 0, (size_t)g.n * 4, s));
-    // the select writes P_d and F only for the vertices it examines
-    JET_CUDA_TRY(cudaMemcpyAsync(ex.pd, part, (size_t)g.n * 4, cudaMemcpyDeviceToDevice, s));
-    k_fill_i32<<<grid_for(g.n, kTB, 4096), kTB, 0, s>>>(ex.gain, g.n, kNoneGain);
-    int nk = 0;
-    JET_TRY(enqueue_lp(L, s, &nk, ex));
-    k_export_lp<<<grid_for(g.n, kTB, 4096), kTB, 0, s>>>(L, inx_out, inm_out);
-    JET_CUDA_TRY(cudaGetLastError());
-    JET_CUDA_TRY(cudaStreamSynchronize(s));
-    return JET_OK;
+    return run_lp_pass(c, L, B.cut2, locked, cval, flags, ex, inx_out, inm_out);
 }
 
 __global__ void k_export_rb(Level L, int32_t *dest, int32_t *loss) {
@@ -1283,33 +1289,31 @@ __global__ void k_export_rb(Level L, int32_t *dest, int32_t *loss) {
     }
 }
 
-__global__ void __launch_bounds__(1024) k_rb_pass_init(Level L, const int64_t *cut2, int32_t mode) {
+// Control block of a single rebalancing pass (the rest of it is cleared).
+__global__ void __launch_bounds__(1024) k_rb_pass_init(Level L, const int64_t *cut2, int32_t mode, int32_t iter, int64_t Llim,
+                                                       int64_t opt, int64_t sigma) {
     __shared__ long long sh[40];
     __shared__ long long spw[JET_MAX_K];
+    pdl_enter();
     Ctl *ctl = L.ctl;
     if (threadIdx.x == 0) {
+        ctl->L = Llim;
+        ctl->opt = opt;
+        ctl->sigma = sigma;
         ctl->cut = *cut2 / 2;
-        ctl->it = 0; ctl->mode = mode;
-        ctl->ticket = 0;
-        reset_counters(ctl);
+        ctl->it = iter;
+        ctl->mode = mode;
     }
     block_max_pw(L.pw, L.k, sh, spw);   // part weights into shared memory
-    compute_classes(L, sh, spw, ctl->L, ctl->sigma);
+    compute_classes(L, sh, spw, Llim, sigma);
 }
 
-__global__ void k_clear_keys(Level L) {
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < L.g.n; v += (int64_t)gridDim.x * blockDim.x)
-        L.key[v] = -1;
-}
-
-int rebalance_pass(Ctx &c, const DGraph &g, int32_t k, double eps, int32_t strong, uint64_t seed, int32_t iter,
+int rebalance_pass(Ctx &c, const DGraph &g, int64_t W, int32_t k, double eps, int32_t strong, uint64_t seed, int32_t iter,
                    const int32_t *part, int32_t *dest_out, int32_t *loss_out, int64_t *nmoves, int64_t *ncand) {
     cudaStream_t s = c.stream;
     if (nmoves) *nmoves = 0;
     if (ncand) *ncand = 0;
     if (g.n == 0) return JET_OK;
-    int64_t W = 0;
-    JET_TRY(total_vweight(c, g, W));
     int64_t opt = 0;
     int64_t L_lim = balance_limit(W, k, eps, &opt);
     int64_t sigma = opt + (L_lim - opt) / 2;
@@ -1318,25 +1322,23 @@ int rebalance_pass(Ctx &c, const DGraph &g, int32_t k, double eps, int32_t stron
     Level &L = B.L;
     L.part = const_cast<int32_t *>(part);   // read only in this pass
     fill_level_params(c, L, 1, seed);
-    int64_t consts[3] = {L_lim, opt, sigma};
-    JET_CUDA_TRY(cudaMemcpyAsync(&L.ctl->L, consts, sizeof(consts), cudaMemcpyHostToDevice, s));
-    int gcut = std::min(list_grid(), grid_for(g.n, kTB));
-    if (g.ew) k_cut_pw<true><<<gcut, kTB, sm_cut_pw(k), s>>>(g, k, L.part, L.pw, B.cut2, L.ext, L.wdeg);
-    else k_cut_pw<false><<<gcut, kTB, sm_cut_pw(k), s>>>(g, k, L.part, L.pw, B.cut2, L.ext, L.wdeg);
     L.rbloss = loss_out;
-    k_rb_pass_init<<<1, 1024, 0, s>>>(L, B.cut2, strong ? MODE_RS : MODE_RW);
-    // the pass API takes the iteration index as a parameter: set ctl->it
-    JET_CUDA_TRY(cudaMemcpyAsync(&L.ctl->it, &iter, 4, cudaMemcpyHostToDevice, s));
-    k_clear_keys<<<grid_for(g.n, kTB, 4096), kTB, 0, s>>>(L);
+    LevelInit init{};
+    init.key = L.key;
+    init.cut2 = B.cut2;
+    JET_TRY(enqueue_start(c, L, init, L.wdeg));
+    JET_CUDA_TRY(launch_pdl(k_rb_pass_init, 1, 1024, 0, s, true, L, (const int64_t *)B.cut2,
+                            (int32_t)(strong ? MODE_RS : MODE_RW), iter, L_lim, opt, sigma));
     int nk = 0;
     JET_TRY(enqueue_rb(L, s, strong != 0, &nk));
-    Ctl h;
-    JET_TRY(read_ctl(c, L, h));
-    if (nmoves) *nmoves = (int64_t)h.nM + h.nMh;
-    if (ncand) *ncand = h.ncand;
     k_export_rb<<<grid_for(g.n, kTB, 4096), kTB, 0, s>>>(L, dest_out, loss_out);
     JET_CUDA_TRY(cudaGetLastError());
+    JET_CUDA_TRY(cudaMemcpyAsync(c.pinned, L.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
     JET_CUDA_TRY(cudaStreamSynchronize(s));
+    Ctl h;
+    memcpy(&h, c.pinned, sizeof(h));
+    if (nmoves) *nmoves = (int64_t)h.nM + h.nMh;
+    if (ncand) *ncand = h.ncand;
     return JET_OK;
 }
 
@@ -1350,8 +1352,8 @@ int cut_and_weights(Ctx &c, const DGraph &g, int32_t k, const int32_t *part, int
     JET_CUDA_TRY(cudaMemsetAsync(pw, 0, (size_t)k * 8, s));
     if (g.n > 0) {
         int gcut = std::min(list_grid(), grid_for(g.n, kTB));
-        if (g.ew) k_cut_pw<true><<<gcut, kTB, sm_cut_pw(k), s>>>(g, k, part, pw, cut2, nullptr, nullptr);
-        else k_cut_pw<false><<<gcut, kTB, sm_cut_pw(k), s>>>(g, k, part, pw, cut2, nullptr, nullptr);
+        if (g.ew) k_cut_pw<true><<<gcut, kTB, sm_cut_pw(k), s>>>(g, k, part, pw, cut2, nullptr, nullptr, nullptr);
+        else k_cut_pw<false><<<gcut, kTB, sm_cut_pw(k), s>>>(g, k, part, pw, cut2, nullptr, nullptr, nullptr);
     }
     JET_CUDA_TRY(cudaGetLastError());
     JET_CUDA_TRY(cudaMemcpyAsync(c.pinned, cut2, 8, cudaMemcpyDeviceToHost, s));
@@ -1367,7 +1369,6 @@ int cut_and_weights(Ctx &c, const DGraph &g, int32_t k, const int32_t *part, int
 int lp_pass_in_scratch(Ctx &c, const DGraph &g, int32_t k, const int32_t *part, const uint8_t *locked, double cval,
                        uint32_t flags, int32_t *pd_out, int32_t *gain_out, uint8_t *inx_out, int32_t *f2_out,
                        uint8_t *inm_out, char *scratch) {
-    cudaStream_t s = c.stream;
     if (g.n == 0) return JET_OK;
     JET_TRY(allow_large_arenas(c.device));
     size_t nn = (size_t)g.n;
@@ -1388,34 +1389,9 @@ int lp_pass_in_scratch(Ctx &c, const DGraph &g, int32_t k, const int32_t *part, 
     L.pw = reinterpret_cast<int64_t *>(p);
     p += align256c((size_t)JET_MAX_K * 8);
     int64_t *cut2 = reinterpret_cast<int64_t *>(p);
-    fill_level_params(c, L, 1, 0);
-    L.cq16 = (int32_t)llround(cval * 65536.0);
-    L.abl = flags & ABL_ALL;
-    // the array keeps the previous call's contents: clear what must start at zero
-    JET_CUDA_TRY(cudaMemsetAsync(L.ctl, 0, sizeof(Ctl), s));
-    JET_CUDA_TRY(cudaMemsetAsync(L.pw, 0, (size_t)k * 8, s));
-    JET_CUDA_TRY(cudaMemsetAsync(cut2, 0, 16, s));
-    {
-        int gcut = std::min(list_grid(), grid_for(g.n, kTB));
-        if (g.ew) k_cut_pw<true><<<gcut, kTB, sm_cut_pw(k), s>>>(g, k, L.part, L.pw, cut2, L.ext, nullptr);
-        else k_cut_pw<false><<<gcut, kTB, sm_cut_pw(k), s>>>(g, k, L.part, L.pw, cut2, L.ext, nullptr);
-    }
-    k_count_big<<<grid_for(g.n, kTB), kTB, 0, s>>>(g, &L.ctl->nbig);
-    k_fill_i32<<<grid_for(g.n, kTB, 4096), kTB, 0, s>>>(L.mstamp, g.n, -2);
-    k_fill_i32<<<grid_for(g.n, kTB, 4096), kTB, 0, s>>>(L.prio, g.n, kNoneGain);
-    k_locks_from_mask<<<grid_for(g.n, kTB, 4096), kTB, 0, s>>>(locked, L.lstamp, g.n);
-    k_set_epoch<<<1, 1, 0, s>>>(L.ctl, 0, MODE_LP);
-    JET_CUDA_TRY(cudaGetLastError());
+    // the array keeps the previous call's contents; the start clears what the pass reads
     LpExport ex{pd_out ? pd_out : tmp_pd, gain_out ? gain_out : tmp_gain, f2_out};
-    if (f2_out) JET_CUDA_TRY(cudaMemsetAsync(f2_out, 0, nn * 4, s));
-    JET_CUDA_TRY(cudaMemcpyAsync(ex.pd, part, nn * 4, cudaMemcpyDeviceToDevice, s));
-    k_fill_i32<<<grid_for(g.n, kTB, 4096), kTB, 0, s>>>(ex.gain, g.n, kNoneGain);
-    int nk = 0;
-    JET_TRY(enqueue_lp(L, s, &nk, ex));
-    k_export_lp<<<grid_for(g.n, kTB, 4096), kTB, 0, s>>>(L, inx_out, inm_out);
-    JET_CUDA_TRY(cudaGetLastError());
-    JET_CUDA_TRY(cudaStreamSynchronize(s));
-    return JET_OK;
+    return run_lp_pass(c, L, cut2, locked, cval, flags, ex, inx_out, inm_out);
 }
 
 }  // namespace jet
