@@ -11,15 +11,19 @@
 //   k_agg_fwd / k_agg_bwd   mean aggregation over CSR and its transpose, one
 //                           warp per vertex (gather form both ways: the
 //                           transpose reads each neighbour's 1/deg share, so
-//                           no atomics and a fixed summation order);
-//   k_gemm_rows             row-parallel C = A B (+ bias, relu): 64 rows per
-//                           block, A and B staged in shared memory as bf16,
+//                           no atomics and a fixed summation order), four
+//                           neighbours' rows in flight;
+//   k_gemm_rows             row-parallel C = A B (+ bias, relu, or masked by an
+//                           activation): 32 rows per block, A and B staged in
+//                           shared memory as bf16, fragments by ldmatrix,
 //                           mma.sync m16n8k16 with float32 accumulators;
 //   k_gemm_tn + k_tn_reduce weight gradients A^T B over all rows: each block
-//                           reduces a fixed 512-row chunk on the tensor cores,
-//                           the partial sums are added in block order
-//                           (deterministic, no atomics);
-//   k_softmax_ce, k_adam, the feature kernels and the balanced decode.
+//                           reduces a fixed 256-row chunk for 32 rows of the
+//                           result on the tensor cores, the partial sums are
+//                           added in chunk order (deterministic, no atomics);
+//   k_softmax_ce (the last block adds the loss up), k_adam, the feature kernels
+//   and the balanced decode.
+// Consecutive launches overlap their set-up (programmatic launch).
 // All sizes here are small (the coarsest graph has a few hundred to a few
 // thousand vertices, a training batch some tens of thousands): the dense
 // layers are K <= 256, N <= 256 products whose cost is launch latency, so
@@ -43,11 +47,12 @@ namespace {
 constexpr int kF = JET_LIP_FEATURES;
 constexpr int kHd = JET_LIP_HIDDEN;
 constexpr int kLayers = 3;
-constexpr int kGemmBM = 64;        // rows per block of k_gemm_rows (4 warps x 16 rows)
-constexpr int kTnRows = 64;        // rows staged per step of k_gemm_tn
+constexpr int kGemmBM = 32;        // rows per block of k_gemm_rows (2 warps x 16 rows, two column halves)
+constexpr int kTnRows = 128;       // rows staged per step of k_gemm_tn
+constexpr int kTnCols = 32;        // rows of the result (columns of A) per block of k_gemm_tn
 constexpr int kTnChunk = 256;      // rows per block of k_gemm_tn (a constant: the summation order is fixed)
 constexpr int kTnWarps = 8;
-constexpr int kTnMaxTiles = 16;    // 16x8 output tiles per warp of k_gemm_tn
+constexpr int kTnMaxTiles = 8;     // 16x8 output tiles per warp of k_gemm_tn
 constexpr int kGemmSmemMax = 100 * 1024;
 
 int din_of(int l) { return l == 0 ? kF : kHd; }
@@ -87,61 +92,108 @@ __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4],
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// Two consecutive bf16 (the lower index in the low half).
-__device__ __forceinline__ uint32_t ld_pair(const __nv_bfloat16 *p) { return *reinterpret_cast<const uint32_t *>(p); }
+// Four 8x8 bf16 tiles whose row addresses the lanes give (lane i: row i % 8 of
+// tile i / 8); trans: every tile transposed.
+template <bool TRANS>
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const __nv_bfloat16 *p) {
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    if (TRANS)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
 
-// C = A B over M rows, bf16 operands rounded from float32 as they are staged,
-// float32 accumulation.  A(r, kk) = A[r*lda + kk] for kk < Kv; B(kk, c) =
-// B[kk*ldb + c], or B[c*ldb + kk] with TRANS_B, for kk < Kv and c < Nv;
-// zero beyond.  Kp (multiple of 16) and Np (multiple of 8, <= 256) are the
-// padded sizes.  For c < Nv: Y[r*ldy + c] = acc + bias[c] (when Y), R[r*ldr
-// + c] = max(acc + bias[c], 0) (when R).  Block: 128 threads, 64 rows.
-template <bool TRANS_B>
-__global__ void __launch_bounds__(128) k_gemm_rows(int32_t M, int Kp, int Kv, int Np, int Nv, const float *A, int lda,
-                                                   const float *B, int ldb, const float *bias, float *Y, int ldy,
-                                                   float *R, int ldr) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int sk = Kp + 8;                                                  // staged row stride (bf16)
-    __nv_bfloat16 *As = reinterpret_cast<__nv_bfloat16 *>(smem_raw);      // [kGemmBM][sk]
-    __nv_bfloat16 *Bt = As + kGemmBM * sk;                                  // [Np][sk]: B transposed
-    const int64_t r0 = (int64_t)blockIdx.x * kGemmBM;
-    for (int i = threadIdx.x; i < kGemmBM * Kp; i += blockDim.x) {
-        const int r = i / Kp, kk = i - r * Kp;
-        const float x = (r0 + r < M && kk < Kv) ? A[(r0 + r) * lda + kk] : 0.f;
-        As[r * sk + kk] = __float2bfloat16_rn(x);
-    }
-    for (int i = threadIdx.x; i < Np * Kp; i += blockDim.x) {
-        int c, kk;
-        if (TRANS_B) { c = i / Kp; kk = i - c * Kp; }   // walk the source contiguously
-        else { kk = i / Np; c = i - kk * Np; }
-        float x = 0.f;
-        if (kk < Kv && c < Nv) x = TRANS_B ? B[(int64_t)c * ldb + kk] : B[(int64_t)kk * ldb + c];
-        Bt[c * sk + kk] = __float2bfloat16_rn(x);
-    }
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int rw = warp * 16;
-    for (int nc = 0; nc < Np; nc += 64) {
-        const int nt = min(8, (Np - nc) >> 3);
-        float acc[8][4];
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+    const __nv_bfloat162 x = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t *>(&x);
+}
+
+// rows x cols (cols a multiple of 4) of src (row stride ld, zero from row vrows
+// and column vcols on) into dst as bf16, row stride ds; the whole block.  16-byte
+// loads where the rows allow them, four in flight per thread.
+__device__ __forceinline__ void stage_bf16(__nv_bfloat16 *dst, int ds, int rows, int cols, const float *src, int64_t ld,
+                                           int64_t vrows, int vcols) {
+    const int c4 = cols >> 2, total = rows * c4;
+    const bool vec = ((reinterpret_cast<uintptr_t>(src) | (uintptr_t)(ld * 4) | (uintptr_t)(vcols * 4)) & 15) == 0;
+    for (int i0 = threadIdx.x; i0 < total; i0 += 4 * blockDim.x) {
+        float4 x[4];
+        int r[4], c[4];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-        for (int k0 = 0; k0 < Kp; k0 += 16) {
-            uint32_t a[4];
-            a[0] = ld_pair(As + (rw + g) * sk + k0 + 2 * t);
-            a[1] = ld_pair(As + (rw + g + 8) * sk + k0 + 2 * t);
-            a[2] = ld_pair(As + (rw + g) * sk + k0 + 2 * t + 8);
-            a[3] = ld_pair(As + (rw + g + 8) * sk + k0 + 2 * t + 8);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                if (j < nt) {
-                    const __nv_bfloat16 *bp = Bt + (nc + j * 8 + g) * sk + k0 + 2 * t;
-                    mma_16816(acc[j], a, ld_pair(bp), ld_pair(bp + 8));
+        for (int q = 0; q < 4; ++q) {
+            const int i = i0 + q * blockDim.x;
+            r[q] = i / c4;
+            c[q] = (i - r[q] * c4) * 4;
+            x[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (i < total && r[q] < vrows) {
+                const float *p = src + r[q] * ld + c[q];
+                if (vec) {
+                    if (c[q] < vcols) x[q] = *reinterpret_cast<const float4 *>(p);
+                } else {
+                    if (c[q] < vcols) x[q].x = p[0];
+                    if (c[q] + 1 < vcols) x[q].y = p[1];
+                    if (c[q] + 2 < vcols) x[q].z = p[2];
+                    if (c[q] + 3 < vcols) x[q].w = p[3];
                 }
             }
         }
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int q = 0; q < 4; ++q)
+            if (i0 + q * (int)blockDim.x < total)
+                *reinterpret_cast<uint2 *>(dst + r[q] * ds + c[q]) = make_uint2(pack_bf16(x[q].x, x[q].y), pack_bf16(x[q].z, x[q].w));
+    }
+}
+
+// C = A B over M rows, bf16 operands rounded from float32 as they are staged,
+// float32 accumulation.  A(r, kk) = A[r*lda + kk] for kk < Kv; B(kk, c) =
+// B[kk*ldb + c], or B[c*ldb + kk] with TRANS_B, for kk < Kv and c < Nv;
+// zero beyond.  Kp and Np (multiples of 16, Np <= 256) are the padded sizes.
+// For c < Nv: Y[r*ldy + c] = acc + bias[c] (when Y; with mask 0 where
+// mask[r*ldm + c] <= 0), R[r*ldr + c] = max(acc + bias[c], 0) (when R).  Block:
+// 128 threads, 32 rows; warps 0-1 take the even 32-column groups, 2-3 the odd
+// ones.  Bound by staging (a few KB per block) and launch latency: 12,800 x 128
+// by 128 x 64 took 46 us with scalar loads, index divisions per element and
+// transposing stores.  With 16-byte loads, ldmatrix and half the rows per block a
+// loss and gradient pass at that size (k = 64) went from 632 to 257 us in all.
+template <bool TRANS_B>
+__global__ void __launch_bounds__(128) k_gemm_rows(int32_t M, int Kp, int Kv, int Np, int Nv, const float *A, int lda,
+                                                   const float *B, int ldb, const float *bias, const float *mask, int ldm,
+                                                   float *Y, int ldy, float *R, int ldr) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int sk = Kp + 8, sn = Np + 8;                                     // staged row strides (bf16)
+    __nv_bfloat16 *As = reinterpret_cast<__nv_bfloat16 *>(smem_raw);      // [kGemmBM][sk]
+    __nv_bfloat16 *Bs = As + kGemmBM * sk;                                  // TRANS_B: [Np][sk], else [Kp][sn]
+    const int64_t r0 = (int64_t)blockIdx.x * kGemmBM;
+    // the weights may be read before the wait: a pass starts with a full dependency on the work before it
+    // (k_agg_fwd<kF>, k_softmax_ce) and writes no weight
+    if (TRANS_B) stage_bf16(Bs, sk, Np, Kp, B, ldb, Nv, Kv);
+    else stage_bf16(Bs, sn, Kp, Np, B, ldb, Kv, Nv);
+    pdl_enter();
+    stage_bf16(As, sk, kGemmBM, Kp, A + r0 * lda, lda, M - r0, Kv);
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int rw = (warp & 1) * 16;
+    const int l8 = lane & 7, m1 = (lane >> 3) & 1, m2 = lane >> 4;   // row in a tile; tile bits of this lane's address
+    for (int nc = (warp >> 1) * 32; nc < Np; nc += 64) {
+        const int nt = min(4, (Np - nc) >> 3);
+        float acc[4][4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
+        for (int k0 = 0; k0 < Kp; k0 += 16) {
+            uint32_t a[4], b[4];
+            ldsm4<false>(a, As + (rw + l8 + 8 * m1) * sk + k0 + 8 * m2);
+#pragma unroll
+            for (int j = 0; j < 4; j += 2) {
+                if (j >= nt) continue;
+                if (TRANS_B) ldsm4<false>(b, Bs + (nc + j * 8 + l8 + 8 * m2) * sk + k0 + 8 * m1);
+                else ldsm4<true>(b, Bs + (k0 + l8 + 8 * m1) * sn + nc + j * 8 + 8 * m2);
+                mma_16816(acc[j], a, b[0], b[1]);
+                mma_16816(acc[j + 1], a, b[2], b[3]);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
             if (j >= nt) continue;
 #pragma unroll
             for (int h = 0; h < 4; ++h) {
@@ -149,7 +201,7 @@ __global__ void __launch_bounds__(128) k_gemm_rows(int32_t M, int Kp, int Kv, in
                 const int col = nc + j * 8 + 2 * t + (h & 1);
                 if (r < M && col < Nv) {
                     const float y = acc[j][h] + (bias ? bias[col] : 0.f);
-                    if (Y) Y[r * ldy + col] = y;
+                    if (Y) Y[r * ldy + col] = !mask || mask[r * ldm + col] > 0.f ? y : 0.f;
                     if (R) R[r * ldr + col] = fmaxf(y, 0.f);
                 }
             }
@@ -157,62 +209,49 @@ __global__ void __launch_bounds__(128) k_gemm_rows(int32_t M, int Kp, int Kv, in
     }
 }
 
-// Partial weight gradients over the rows [blockIdx.x * kTnChunk, + kTnChunk):
-// P[blk][i*Np + c] = sum_r A(r, i) B(r, c) with bf16 operands and float32
-// accumulation (i < Kp, c < Np; A(r, i) = A[r*lda + i] for i < Kv, B(r, c) =
-// B[r*ldb + c] for c < Nv, zero beyond), and CS[blk][c] = sum_r B(r, c) in
-// float32: thread t stages the columns t % 64 + 64 g of the rows t / 64 + 4 j
-// and keeps their running sums, which the four row classes then add in a
-// fixed order.  Requires (Kp/16) (Np/8) <= kTnWarps * kTnMaxTiles, Np <= 256
-// and 256 threads.
+// Partial weight gradients over the rows [blockIdx.x * kTnChunk, + kTnChunk)
+// for the result rows [blockIdx.y * kTnCols, + kTnCols): P[blk][i*Np + c] =
+// sum_r A(r, i) B(r, c) with bf16 operands and float32 accumulation (i < Kp,
+// c < Np; A(r, i) = A[r*lda + i] for i < Kv, B(r, c) = B[r*ldb + c] for c < Nv,
+// zero beyond).  Both operands are staged as they lie and transposed by
+// ldmatrix.  The blocks with blockIdx.y = 0 also sum the columns, CS[blk][c] =
+// sum_r B(r, c) in float32: thread t adds the column t % 64 + 64 g of the rows
+// t / 64 + 4 j, and the four row classes are added in a fixed order.  Requires
+// Np <= 256 and 256 threads.  (One block per chunk took 66 us at 12,800 rows:
+// 50 blocks on 152 SMs.)
 __global__ void __launch_bounds__(256) k_gemm_tn(int32_t M, int Kp, int Kv, int Np, int Nv, const float *A, int lda,
                                                  const float *B, int ldb, float *P, float *CS) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int sr = kTnRows + 8;
-    __nv_bfloat16 *At = reinterpret_cast<__nv_bfloat16 *>(smem_raw);   // [Kp][sr]
-    __nv_bfloat16 *Bt = At + Kp * sr;                                    // [Np][sr]
+    const int i0 = blockIdx.y * kTnCols, iw = min(kTnCols, Kp - i0);     // 16 or 32 result rows
+    const int sa = kTnCols + 8, sb = Np + 8;
+    __nv_bfloat16 *As = reinterpret_cast<__nv_bfloat16 *>(smem_raw);   // [kTnRows][sa]
+    __nv_bfloat16 *Bs = As + kTnRows * sa;                               // [kTnRows][sb]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int mt = Kp >> 4, ntiles = mt * (Np >> 3);
+    const int l8 = lane & 7, m1 = (lane >> 3) & 1, m2 = lane >> 4;
+    const int mt = iw >> 4, pairs = mt * (Np >> 4);                      // 16x16 output tiles, taken in turn by the warps
     float acc[kTnMaxTiles][4];
 #pragma unroll
     for (int q = 0; q < kTnMaxTiles; ++q) acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.f;
     const int64_t c0 = (int64_t)blockIdx.x * kTnChunk;
     const int64_t c1 = min((int64_t)M, c0 + kTnChunk);
-    const int tc = threadIdx.x & 63, tr = threadIdx.x >> 6;   // column lane, row class (0..3)
-    float cs[4] = {0.f, 0.f, 0.f, 0.f};
+    pdl_enter();
     for (int64_t r0 = c0; r0 < c1; r0 += kTnRows) {
         __syncthreads();
-        for (int i = threadIdx.x; i < kTnRows * Kp; i += blockDim.x) {
-            const int r = i / Kp, kk = i - r * Kp;
-            const float x = (r0 + r < c1 && kk < Kv) ? A[(r0 + r) * lda + kk] : 0.f;
-            At[kk * sr + r] = __float2bfloat16_rn(x);
-        }
-#pragma unroll
-        for (int gcol = 0; gcol < 4; ++gcol) {
-            const int c = tc + 64 * gcol;
-            if (c < Np) {
-                for (int r = tr; r < kTnRows; r += 4) {
-                    const float x = (r0 + r < c1 && c < Nv) ? B[(r0 + r) * ldb + c] : 0.f;
-                    cs[gcol] += x;
-                    Bt[c * sr + r] = __float2bfloat16_rn(x);
-                }
-            }
-        }
+        stage_bf16(As, sa, kTnRows, iw, A + r0 * lda + i0, lda, c1 - r0, min(iw, max(0, Kv - i0)));
+        stage_bf16(Bs, sb, kTnRows, Np, B + r0 * ldb, ldb, c1 - r0, Nv);
         __syncthreads();
 #pragma unroll
-        for (int q = 0; q < kTnMaxTiles; ++q) {
+        for (int q = 0; q < kTnMaxTiles / 2; ++q) {
             const int tile = warp + q * kTnWarps;
-            if (tile < ntiles) {
-                const int i0 = (tile % mt) * 16, n0 = (tile / mt) * 8;
+            if (tile < pairs) {
+                const int ti = (tile % mt) * 16, n0 = (tile / mt) * 16;
 #pragma unroll
                 for (int k0 = 0; k0 < kTnRows; k0 += 16) {
-                    uint32_t a[4];
-                    a[0] = ld_pair(At + (i0 + g) * sr + k0 + 2 * t);
-                    a[1] = ld_pair(At + (i0 + g + 8) * sr + k0 + 2 * t);
-                    a[2] = ld_pair(At + (i0 + g) * sr + k0 + 2 * t + 8);
-                    a[3] = ld_pair(At + (i0 + g + 8) * sr + k0 + 2 * t + 8);
-                    const __nv_bfloat16 *bp = Bt + (n0 + g) * sr + k0 + 2 * t;
-                    mma_16816(acc[q], a, ld_pair(bp), ld_pair(bp + 8));
+                    uint32_t a[4], b[4];
+                    ldsm4<true>(a, As + (k0 + l8 + 8 * m2) * sa + ti + 8 * m1);
+                    ldsm4<true>(b, Bs + (k0 + l8 + 8 * m1) * sb + n0 + 8 * m2);
+                    mma_16816(acc[2 * q], a, b[0], b[1]);
+                    mma_16816(acc[2 * q + 1], a, b[2], b[3]);
                 }
             }
         }
@@ -220,14 +259,25 @@ __global__ void __launch_bounds__(256) k_gemm_tn(int32_t M, int Kp, int Kv, int 
     float *Pb = P + (int64_t)blockIdx.x * Kp * Np;
 #pragma unroll
     for (int q = 0; q < kTnMaxTiles; ++q) {
-        const int tile = warp + q * kTnWarps;
-        if (tile < ntiles) {
-            const int i0 = (tile % mt) * 16, n0 = (tile / mt) * 8;
+        const int tile = warp + (q >> 1) * kTnWarps;
+        if (tile < pairs) {
+            const int ti = i0 + (tile % mt) * 16, n0 = (tile / mt) * 16 + (q & 1) * 8;
 #pragma unroll
-            for (int h = 0; h < 4; ++h) Pb[(i0 + g + (h >> 1) * 8) * Np + n0 + 2 * t + (h & 1)] = acc[q][h];
+            for (int h = 0; h < 4; ++h) Pb[(ti + g + (h >> 1) * 8) * Np + n0 + 2 * t + (h & 1)] = acc[q][h];
         }
     }
-    // column sums: the four row classes in order
+    if (blockIdx.y != 0) return;
+    // column sums: each row class in order, then the four classes in order
+    const int tc = threadIdx.x & 63, tr = threadIdx.x >> 6;   // column lane, row class (0..3)
+    float cs[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int gcol = 0; gcol < 4; ++gcol) {
+        const int c = tc + 64 * gcol;
+        if (c < Np) {
+#pragma unroll 8
+            for (int r = tr; r < kTnChunk; r += 4) cs[gcol] += (c0 + r < c1 && c < Nv) ? B[(c0 + r) * ldb + c] : 0.f;
+        }
+    }
     __syncthreads();
     float *red = reinterpret_cast<float *>(smem_raw);   // [4][256], the staging tiles are no longer read
 #pragma unroll
@@ -241,16 +291,19 @@ __global__ void __launch_bounds__(256) k_gemm_tn(int32_t M, int Kp, int Kv, int 
 // c < Nv); gb[c] = sum over b of CS[b][c].
 __global__ void k_tn_reduce(int nb, int Kp, int Kv, int Np, int Nv, const float *P, const float *CS, float *gW,
                             float *gb) {
+    pdl_enter();
     const int64_t total = (int64_t)Kv * Nv;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total + Nv;
          e += (int64_t)gridDim.x * blockDim.x) {
         float s = 0.f;
         if (e < total) {
             const int64_t i = e / Nv, c = e - i * Nv;
+#pragma unroll 16
             for (int b = 0; b < nb; ++b) s += P[(int64_t)b * Kp * Np + i * Np + c];
             gW[e] = s;
         } else {
             const int64_t c = e - total;
+#pragma unroll 16
             for (int b = 0; b < nb; ++b) s += CS[(int64_t)b * Np + c];
             gb[c] = s;
         }
@@ -260,52 +313,92 @@ __global__ void k_tn_reduce(int nb, int Kp, int Kv, int Np, int Nv, const float 
 // ---- aggregation over CSR ---------------------------------------------------
 // Z[v][0:d] = H[v] (skipped when H is Z itself), Z[v][d:2d] = mean of H[u]
 // over the neighbours u of v (0 without neighbours).  H row stride ldh, Z
-// row stride 2d.  One warp per vertex, lanes over the d columns.
-__global__ void __launch_bounds__(kTB) k_agg_fwd(DGraph g, int d, const float *H, int ldh, float *Z) {
-    const int warps = blockDim.x >> 5;
-    const int lane = threadIdx.x & 31;
-    const int ldz = 2 * d;
-    for (int64_t v = (int64_t)blockIdx.x * warps + (threadIdx.x >> 5); v < g.n; v += (int64_t)gridDim.x * warps) {
+// row stride 2d.  d = 16: half a warp per vertex, one column per lane; d = 64:
+// a warp per vertex, two columns per lane.  The columns of four neighbours are
+// loaded together and added in row order.
+template <int D>
+__global__ void __launch_bounds__(kTB) k_agg_fwd(DGraph g, const float *H, int ldh, float *Z) {
+    constexpr int kLanes = D == 16 ? 16 : 32, kCols = D / kLanes, U = 4;
+    const int per = blockDim.x / kLanes;
+    const int c0 = (int)(threadIdx.x % kLanes) * kCols;
+    constexpr int ldz = 2 * D;
+    pdl_enter();
+    for (int64_t v = (int64_t)blockIdx.x * per + threadIdx.x / kLanes; v < g.n; v += (int64_t)gridDim.x * per) {
         const int64_t beg = g.xadj[v], end = g.xadj[v + 1];
-        for (int c = lane; c < d; c += 32) {
-            float s = 0.f;
-            for (int64_t j = beg; j < end; ++j) s += H[(int64_t)g.adj[j] * ldh + c];
-            if (H != Z) Z[v * ldz + c] = H[v * ldh + c];
-            Z[v * ldz + d + c] = end > beg ? s / (float)(end - beg) : 0.f;
+        float s[kCols];
+#pragma unroll
+        for (int q = 0; q < kCols; ++q) s[q] = 0.f;
+        for (int64_t j = beg; j < end; j += U) {
+            int32_t u[U];
+            float x[U][kCols];
+#pragma unroll
+            for (int z = 0; z < U; ++z) u[z] = j + z < end ? g.adj[j + z] : -1;
+#pragma unroll
+            for (int z = 0; z < U; ++z)
+#pragma unroll
+                for (int q = 0; q < kCols; ++q) x[z][q] = u[z] >= 0 ? H[(int64_t)u[z] * ldh + c0 + q] : 0.f;
+#pragma unroll
+            for (int z = 0; z < U; ++z)
+#pragma unroll
+                for (int q = 0; q < kCols; ++q)
+                    if (u[z] >= 0) s[q] += x[z][q];
+        }
+#pragma unroll
+        for (int q = 0; q < kCols; ++q) {
+            if (H != Z) Z[v * ldz + c0 + q] = H[v * ldh + c0 + q];
+            Z[v * ldz + D + c0 + q] = end > beg ? s[q] / (float)(end - beg) : 0.f;
         }
     }
 }
 
-// Transpose of the aggregation plus the direct half:
-// dH[u][c] = dZ[u][c] + sum over neighbours v of dZ[v][d + c] / deg(v).
-__global__ void __launch_bounds__(kTB) k_agg_bwd(DGraph g, int d, const float *dZ, float *dH) {
+// Transpose of the aggregation plus the direct half, then the relu:
+// dY[u][c] = dZ[u][c] + sum over neighbours v of dZ[v][64 + c] / deg(v) where
+// H[u*ldh + c] > 0, else 0 (H = relu(Y)).  A warp per vertex, two columns per lane,
+// four neighbours in flight, added in row order.
+__global__ void __launch_bounds__(kTB) k_agg_bwd(DGraph g, const float *dZ, const float *H, int ldh, float *dY) {
+    constexpr int U = 4, ldz = 2 * kHd;
     const int warps = blockDim.x >> 5;
-    const int lane = threadIdx.x & 31;
-    const int ldz = 2 * d;
+    const int c0 = (int)(threadIdx.x & 31) * 2;
+    pdl_enter();
     for (int64_t u = (int64_t)blockIdx.x * warps + (threadIdx.x >> 5); u < g.n; u += (int64_t)gridDim.x * warps) {
         const int64_t beg = g.xadj[u], end = g.xadj[u + 1];
-        for (int c = lane; c < d; c += 32) {
-            float s = dZ[u * ldz + c];
-            for (int64_t j = beg; j < end; ++j) {
-                const int64_t v = g.adj[j];
-                s += dZ[v * ldz + d + c] / (float)(g.xadj[v + 1] - g.xadj[v]);
+        float s0 = dZ[u * ldz + c0], s1 = dZ[u * ldz + c0 + 1];
+        for (int64_t j = beg; j < end; j += U) {
+            int32_t v[U];
+            float x[U][2], deg[U];
+#pragma unroll
+            for (int z = 0; z < U; ++z) v[z] = j + z < end ? g.adj[j + z] : -1;
+#pragma unroll
+            for (int z = 0; z < U; ++z) {
+                const int64_t w = v[z] >= 0 ? v[z] : u;
+                deg[z] = (float)(g.xadj[w + 1] - g.xadj[w]);
+                x[z][0] = dZ[w * ldz + kHd + c0];
+                x[z][1] = dZ[w * ldz + kHd + c0 + 1];
             }
-            dH[u * d + c] = s;
+#pragma unroll
+            for (int z = 0; z < U; ++z)
+                if (v[z] >= 0) {
+                    s0 += x[z][0] / deg[z];
+                    s1 += x[z][1] / deg[z];
+                }
         }
+        dY[u * kHd + c0] = H[u * ldh + c0] > 0.f ? s0 : 0.f;
+        dY[u * kHd + c0 + 1] = H[u * ldh + c0 + 1] > 0.f ? s1 : 0.f;
     }
-}
-
-__global__ void k_relu_bwd(int64_t count, const float *dH, const float *Y, float *dY) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
-        dY[i] = Y[i] > 0.f ? dH[i] : 0.f;
 }
 
 // One warp per row: loss_v = logsumexp(L_v) - L_v[y_v]; dlog_v[c] =
 // (softmax_c - [c = y_v]) / n.  Per-block loss sums (warps in order) in
 // part[blockIdx.x]; a label outside [0, k) sets *bad and its row adds no loss.
+// The last block to finish (*ticket, zero before) adds the blocks' losses over a
+// fixed tree: thread t takes the blocks t, t + 256, ... in order, then pairwise
+// halving.
 __global__ void __launch_bounds__(kTB) k_softmax_ce(int32_t n, int k, const float *L, const int32_t *y, float *dlog,
-                                                    double *part, int *bad) {
+                                                    double *part, int *bad, unsigned *ticket, float *loss) {
     __shared__ double wsum[kTB / 32];
+    __shared__ double sh[kTB];
+    __shared__ int s_last;
+    pdl_enter();
     const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     double acc = 0.0;
@@ -337,19 +430,18 @@ __global__ void __launch_bounds__(kTB) k_softmax_ce(int32_t n, int k, const floa
         double t = 0.0;
         for (int w = 0; w < warps; ++w) t += wsum[w];
         part[blockIdx.x] = t;
+        __threadfence();
+        s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        if (s_last) __threadfence();
     }
-}
-
-// Sum of the per-block losses over a fixed tree (thread t takes the blocks
-// t, t + 256, ... in order, then pairwise halving): one block of 256 threads.
-__global__ void __launch_bounds__(256) k_loss_total(int nb, const double *part, int32_t n, float *loss) {
-    __shared__ double sh[256];
+    __syncthreads();
+    if (!s_last) return;
     double t = 0.0;
-    for (int b = threadIdx.x; b < nb; b += 256) t += part[b];
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += kTB) t += __ldcg(part + b);
     sh[threadIdx.x] = t;
     __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
+    for (int q = kTB / 2; q > 0; q >>= 1) {
+        if ((int)threadIdx.x < q) sh[threadIdx.x] += sh[threadIdx.x + q];
         __syncthreads();
     }
     if (threadIdx.x == 0) *loss = (float)(sh[0] / (double)(n > 0 ? n : 1));
@@ -556,19 +648,15 @@ int grid_rows(int64_t n) { return std::max(1, std::min(num_sms() * 8, grid_for(n
 int grid_elems(int64_t n) { return std::max(1, std::min(num_sms() * 8, grid_for(n, kTB))); }
 
 int gemm_rows(Ctx &c, bool trans_b, int32_t M, int Kp, int Kv, int Np, int Nv, const float *A, int lda, const float *B,
-              int ldb, const float *bias, float *Y, int ldy, float *R, int ldr) {
+              int ldb, const float *bias, const float *mask, int ldm, float *Y, int ldy, float *R, int ldr) {
     if (M <= 0) return JET_OK;
-    const size_t smem = (size_t)(kGemmBM + Np) * (Kp + 8) * 2;
+    const size_t smem = (size_t)(kGemmBM * (Kp + 8) + (trans_b ? Np * (Kp + 8) : Kp * (Np + 8))) * 2;
     const int grid = (int)((M + kGemmBM - 1) / kGemmBM);
-    if (trans_b) {
-        JET_CUDA_TRY(cudaFuncSetAttribute(k_gemm_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmemMax));
-        k_gemm_rows<true><<<grid, 128, smem, c.stream>>>(M, Kp, Kv, Np, Nv, A, lda, B, ldb, bias, Y, ldy, R, ldr);
-    } else {
-        JET_CUDA_TRY(cudaFuncSetAttribute(k_gemm_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmemMax));
-        k_gemm_rows<false><<<grid, 128, smem, c.stream>>>(M, Kp, Kv, Np, Nv, A, lda, B, ldb, bias, Y, ldy, R, ldr);
-    }
+    auto kern = trans_b ? k_gemm_rows<true> : k_gemm_rows<false>;
+    JET_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmemMax));
+    JET_CUDA_TRY(launch_pdl(kern, grid, 128, smem, c.stream, true, M, Kp, Kv, Np, Nv, A, lda, B, ldb, bias, mask, ldm, Y, ldy,
+                            R, ldr));
     c.launches += 1;
-    JET_CUDA_TRY(cudaGetLastError());
     return JET_OK;
 }
 
@@ -578,21 +666,31 @@ int tn_blocks(int32_t M) { return std::max(1, (int)((M + kTnChunk - 1) / kTnChun
 int gemm_tn(Ctx &c, int32_t M, int Kp, int Kv, int Np, int Nv, const float *A, int lda, const float *B, int ldb,
             float *P, float *CS, float *gW, float *gb) {
     const int nb = tn_blocks(M);
-    const size_t smem = (size_t)(Kp + Np) * (kTnRows + 8) * 2;
+    const size_t smem = std::max((size_t)kTnRows * (kTnCols + 8 + Np + 8) * 2, (size_t)4096);
     JET_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tn, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmemMax));
-    k_gemm_tn<<<nb, kTnWarps * 32, smem, c.stream>>>(M, Kp, Kv, Np, Nv, A, lda, B, ldb, P, CS);
-    k_tn_reduce<<<grid_elems((int64_t)Kv * Nv + Nv), kTB, 0, c.stream>>>(nb, Kp, Kv, Np, Nv, P, CS, gW, gb);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)nb, (unsigned)((Kp + kTnCols - 1) / kTnCols));
+    cfg.blockDim = dim3(kTnWarps * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = c.stream;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    JET_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_gemm_tn, M, Kp, Kv, Np, Nv, A, lda, B, ldb, P, CS));
+    JET_CUDA_TRY(launch_pdl(k_tn_reduce, grid_elems((int64_t)Kv * Nv + Nv), kTB, 0, c.stream, true, nb, Kp, Kv, Np, Nv,
+                            (const float *)P, (const float *)CS, gW, gb));
     c.launches += 2;
-    JET_CUDA_TRY(cudaGetLastError());
     return JET_OK;
 }
 
 // Workspace of one forward (and backward) pass over n rows.
 struct Work {
     DevBuf buf;
-    float *Z[kLayers], *Y[kLayers], *H3, *logits, *dlog, *dH, *dY, *dZ, *P, *CS, *loss;
+    float *Z[kLayers], *H3, *logits, *dlog, *dY, *dZ, *P, *CS, *loss;
     double *lpart;
-    int *bad;
+    int *bad;            // then the softmax kernel's ticket
     int ce_blocks;
 };
 
@@ -607,18 +705,16 @@ int work_alloc(Ctx &c, Work &w, int32_t n, int32_t k, bool backward, float *logi
     sizes[cnt++] = nn * 2 * kF * 4;                 // Z0
     sizes[cnt++] = nn * 2 * kHd * 4;                // Z1
     sizes[cnt++] = nn * 2 * kHd * 4;                // Z2
-    for (int l = 0; l < kLayers; ++l) sizes[cnt++] = nn * kHd * 4;   // Y
     sizes[cnt++] = nn * kHd * 4;                    // H3
     sizes[cnt++] = logits_ext ? 0 : nn * k * 4;     // logits
     if (backward) {
         sizes[cnt++] = nn * k * 4;                  // dlog
-        sizes[cnt++] = nn * kHd * 4;                // dH
         sizes[cnt++] = nn * kHd * 4;                // dY
         sizes[cnt++] = nn * 2 * kHd * 4;            // dZ
         sizes[cnt++] = (size_t)nb * ptile * 4;      // P
         sizes[cnt++] = (size_t)nb * std::max(kHd, kp) * 4;   // CS
         sizes[cnt++] = (size_t)w.ce_blocks * 8;     // lpart
-        sizes[cnt++] = 16;                          // loss, bad
+        sizes[cnt++] = 16;                          // loss, spare, bad, ticket
     }
     size_t total = 0;
     for (int i = 0; i < cnt; ++i) total += align256c(sizes[i]);
@@ -627,12 +723,10 @@ int work_alloc(Ctx &c, Work &w, int32_t n, int32_t k, bool backward, float *logi
     int i = 0;
     auto take = [&]() { char *r = p; p += align256c(sizes[i++]); return r; };
     for (int l = 0; l < kLayers; ++l) w.Z[l] = reinterpret_cast<float *>(take());
-    for (int l = 0; l < kLayers; ++l) w.Y[l] = reinterpret_cast<float *>(take());
     w.H3 = reinterpret_cast<float *>(take());
     w.logits = logits_ext ? (take(), logits_ext) : reinterpret_cast<float *>(take());
     if (backward) {
         w.dlog = reinterpret_cast<float *>(take());
-        w.dH = reinterpret_cast<float *>(take());
         w.dY = reinterpret_cast<float *>(take());
         w.dZ = reinterpret_cast<float *>(take());
         w.P = reinterpret_cast<float *>(take());
@@ -662,21 +756,22 @@ int forward(Ctx &c, const Lip &m, const DGraph &g, const float *X, Work &w) {
     const Offsets o = offsets(m.k);
     const int32_t n = g.n;
     const int k = m.k, kp = pad16(k);
-    k_agg_fwd<<<grid_rows(n), kTB, 0, c.stream>>>(g, kF, X, kF, w.Z[0]);
+    JET_CUDA_TRY(launch_pdl(k_agg_fwd<kF>, std::max(1, std::min(num_sms() * 8, grid_for(n, kTB / 16))), kTB, 0, c.stream, false,
+                            g, X, kF, w.Z[0]));
     c.launches += 1;
-    JET_CUDA_TRY(cudaGetLastError());
     for (int l = 0; l < kLayers; ++l) {
         const int K = 2 * din_of(l);
         float *R = l + 1 < kLayers ? w.Z[l + 1] : w.H3;
         const int ldr = l + 1 < kLayers ? 2 * kHd : kHd;
-        JET_TRY(gemm_rows(c, false, n, K, K, kHd, kHd, w.Z[l], K, m.P + o.W[l], kHd, m.P + o.b[l], w.Y[l], kHd, R, ldr));
+        JET_TRY(gemm_rows(c, false, n, K, K, kHd, kHd, w.Z[l], K, m.P + o.W[l], kHd, m.P + o.b[l], nullptr, 0, nullptr, 0, R,
+                          ldr));
         if (l + 1 < kLayers) {
-            k_agg_fwd<<<grid_rows(n), kTB, 0, c.stream>>>(g, kHd, w.Z[l + 1], 2 * kHd, w.Z[l + 1]);
+            JET_CUDA_TRY(launch_pdl(k_agg_fwd<kHd>, grid_rows(n), kTB, 0, c.stream, true, g, (const float *)w.Z[l + 1], 2 * kHd,
+                                    w.Z[l + 1]));
             c.launches += 1;
-            JET_CUDA_TRY(cudaGetLastError());
         }
     }
-    return gemm_rows(c, false, n, kHd, kHd, kp, k, w.H3, kHd, m.P + o.W[kLayers], k, m.P + o.b[kLayers], w.logits, k,
+    return gemm_rows(c, false, n, kHd, kHd, kp, k, w.H3, kHd, m.P + o.W[kLayers], k, m.P + o.b[kLayers], nullptr, 0, w.logits, k,
                      nullptr, 0);
 }
 
@@ -685,26 +780,22 @@ int backward(Ctx &c, const Lip &m, const DGraph &g, const int32_t *labels, Work 
     const Offsets o = offsets(m.k);
     const int32_t n = g.n;
     const int k = m.k, kp = pad16(k);
-    JET_CUDA_TRY(cudaMemsetAsync(w.bad, 0, 4, c.stream));
-    k_softmax_ce<<<w.ce_blocks, kTB, 0, c.stream>>>(n, k, w.logits, labels, w.dlog, w.lpart, w.bad);
-    k_loss_total<<<1, 256, 0, c.stream>>>(w.ce_blocks, w.lpart, n, w.loss);
-    c.launches += 2;
-    JET_CUDA_TRY(cudaGetLastError());
-    // output layer: dWo = H3^T dlog, dbo = colsum dlog, dH3 = dlog Wo^T
+    JET_CUDA_TRY(cudaMemsetAsync(w.bad, 0, 8, c.stream));
+    JET_CUDA_TRY(launch_pdl(k_softmax_ce, w.ce_blocks, kTB, 0, c.stream, false, n, k, (const float *)w.logits, labels, w.dlog,
+                            w.lpart, w.bad, reinterpret_cast<unsigned *>(w.bad + 1), w.loss));
+    c.launches += 1;
+    // output layer: dWo = H3^T dlog, dbo = colsum dlog, dY3 = dlog Wo^T where H3 > 0
     JET_TRY(gemm_tn(c, n, kHd, kHd, kp, k, w.H3, kHd, w.dlog, k, w.P, w.CS, grad + o.W[kLayers], grad + o.b[kLayers]));
-    JET_TRY(gemm_rows(c, true, n, kp, k, kHd, kHd, w.dlog, k, m.P + o.W[kLayers], k, nullptr, w.dH, kHd, nullptr, 0));
+    JET_TRY(gemm_rows(c, true, n, kp, k, kHd, kHd, w.dlog, k, m.P + o.W[kLayers], k, nullptr, w.H3, kHd, w.dY, kHd, nullptr, 0));
     for (int l = kLayers - 1; l >= 0; --l) {
-        const int d = din_of(l), K = 2 * d;
-        k_relu_bwd<<<grid_elems((int64_t)n * kHd), kTB, 0, c.stream>>>((int64_t)n * kHd, w.dH, w.Y[l], w.dY);
-        c.launches += 1;
-        JET_CUDA_TRY(cudaGetLastError());
+        const int K = 2 * din_of(l);
         JET_TRY(gemm_tn(c, n, K, K, kHd, kHd, w.Z[l], K, w.dY, kHd, w.P, w.CS, grad + o.W[l], grad + o.b[l]));
         if (l > 0) {
-            // dZ = dY W^T (n x 2d); dH_{l-1} = dZ[:, :d] + aggregation transpose of dZ[:, d:]
-            JET_TRY(gemm_rows(c, true, n, kHd, kHd, K, K, w.dY, kHd, m.P + o.W[l], kHd, nullptr, w.dZ, K, nullptr, 0));
-            k_agg_bwd<<<grid_rows(n), kTB, 0, c.stream>>>(g, d, w.dZ, w.dH);
+            // dZ = dY W^T (n x 2d); dY_{l-1} = dZ[:, :d] + aggregation transpose of dZ[:, d:], where H_{l-1} > 0
+            JET_TRY(gemm_rows(c, true, n, kHd, kHd, K, K, w.dY, kHd, m.P + o.W[l], kHd, nullptr, nullptr, 0, w.dZ, K, nullptr, 0));
+            JET_CUDA_TRY(launch_pdl(k_agg_bwd, grid_rows(n), kTB, 0, c.stream, true, g, (const float *)w.dZ,
+                                    (const float *)w.Z[l], 2 * kHd, w.dY));
             c.launches += 1;
-            JET_CUDA_TRY(cudaGetLastError());
         }
     }
     return JET_OK;
@@ -898,7 +989,7 @@ int jet_lip_forward(jet_ctx *ctx, const jet_lip *h, int32_t n, const int64_t *xa
     JET_TRY(use_device(c));
     DGraph g;
     DevBuf ones;
-    JET_TRY(graph_of(c, n, xadj, adjncy, nullptr, nullptr, g, ones));
+    JET_TRY(prepare_graph(c, n, xadj, adjncy, nullptr, nullptr, g, ones, false));
     if (n == 0) return JET_OK;
     Work w;
     JET_TRY(work_alloc(c, w, n, h->m.k, false, logits_out));
@@ -910,7 +1001,7 @@ static int loss_grad(Ctx &c, const Lip &m, int32_t n, const int64_t *xadj, const
                      const int32_t *labels, float *loss_out, float *grad) {
     DGraph g;
     DevBuf ones;
-    JET_TRY(graph_of(c, n, xadj, adjncy, nullptr, nullptr, g, ones));
+    JET_TRY(prepare_graph(c, n, xadj, adjncy, nullptr, nullptr, g, ones, false));
     if (n == 0) {
         JET_CUDA_TRY(cudaMemsetAsync(grad, 0, (size_t)m.np * 4, c.stream));
         if (loss_out) *loss_out = 0.f;
