@@ -14,6 +14,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <mutex>
 
 namespace jet {
 
@@ -39,19 +40,13 @@ __global__ void __launch_bounds__(1024) k_scan_sums(int64_t *tile_sums, int64_t 
     if (threadIdx.x == 0 && total_dev) *total_dev = carry;
 }
 
+// Matching state between the rounds of the launched form.
 struct HemCtl {
     int32_t stop;
+    int32_t nbig, nhuge;     // rows in the lists of k_hem_start
     int32_t pad;
     int64_t added[64];
 };
-
-__device__ __forceinline__ bool hem_better(int32_t w1, uint64_t h1, int32_t u1, int32_t w2, uint64_t h2, int32_t u2) {
-    if (u2 < 0) return u1 >= 0;
-    if (u1 < 0) return false;
-    if (w1 != w2) return w1 > w2;
-    if (h1 != h2) return h1 < h2;
-    return u1 < u2;
-}
 
 __device__ __forceinline__ uint64_t hem_hash(uint64_t seed, uint64_t salt, int32_t u) {
     return splitmix64(seed ^ salt ^ (uint64_t)(uint32_t)u);
@@ -61,215 +56,339 @@ __device__ __forceinline__ bool hem_skip(const HemCtl *hc, int r) {
     return r > 0 && (hc->stop || hc->added[r - 1] == 0);
 }
 
-// One proposal round (short rows): prop[v] = chosen neighbour or -1.
+// The best proposal so far of a lane, a group of lanes or a block: larger
+// weight, then smaller hash (splitmix64 is one to one, so that no two neighbours
+// tie and their ids need no look).
+struct HemBest {
+    int32_t u = -1, w = INT32_MIN;
+    uint64_t h = ~0ull;
+    __device__ __forceinline__ void take(bool ok, int32_t ou, int32_t ow, uint64_t oh) {   // ou >= 0 where ok; no branch
+        const bool better = ok & ((ow > w) | ((ow == w) & (oh < h)) | (u < 0));
+        u = better ? ou : u;
+        w = better ? ow : w;
+        h = better ? oh : h;
+    }
+    // over lanes that differ in the bits below `lanes` (a power of two); the whole warp calls it
+    __device__ __forceinline__ void reduce(int lanes) {
+        for (int o = lanes >> 1; o > 0; o >>= 1) {
+            const int32_t ou = __shfl_xor_sync(0xffffffffu, u, o);
+            const int32_t ow = __shfl_xor_sync(0xffffffffu, w, o);
+            const uint64_t oh = __shfl_xor_sync(0xffffffffu, h, o);
+            take(ou >= 0, ou, ow, oh);
+        }
+    }
+};
+
+// The heaviest unmatched neighbour over the entries first, first + step, ...
+// < end of a row, U at a time (ids and weights, then their matched bits, in
+// flight together); folds into best.  A bit per vertex instead of its mate: the
+// gathers of a whole mesh level fit in L1, and a hub-heavy graph's mostly do.
+template <bool EW, int U = 4>
+__device__ __forceinline__ void hem_row(const DGraph &g, const uint32_t *matched, uint64_t seed, uint64_t salt,
+                                        int64_t first, int64_t end, int64_t step, HemBest &best) {
+    for (int64_t j0 = first; j0 < end; j0 += U * step) {
+        int32_t u[U], w[U];
+        bool open[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const int64_t j = j0 + q * step;
+            u[q] = j < end ? __ldg(g.adj + j) : -1;
+            w[q] = j < end ? cw<EW>(g, j) : 0;
+        }
+#pragma unroll
+        for (int q = 0; q < U; ++q) open[q] = u[q] >= 0 && !(matched[u[q] >> 5] >> (u[q] & 31) & 1u);
+#pragma unroll
+        for (int q = 0; q < U; ++q) best.take(open[q], u[q], w[q], hem_hash(seed, salt, u[q]));
+    }
+}
+
+// The whole block's best (blockDim.x <= 1024); valid in thread 0.
+__device__ __forceinline__ void hem_block_best(HemBest &best, HemBest *sh) {
+    best.reduce(32);
+    if (lane_id() == 0) sh[threadIdx.x >> 5] = best;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        best = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : HemBest{};
+        best.reduce(32);
+    }
+    __syncthreads();
+}
+
+// ---- one cluster, all rounds in one launch ----
+//
+// Small levels are bound by launches (three per round) and by dependent trips to
+// L2.  Here a cluster keeps a matched bit of every vertex in each block's shared
+// memory; a round is: the block's unmatched vertices are listed, groups of lanes
+// scan their rows against the local bits, one cluster barrier, mutual proposals
+// match, one cluster barrier, and every block copies the other blocks' bits.
+// Rows longer than kHemLong are scanned by the whole block.  Ends with the first
+// round that matches nothing, as the launched form does.  Whole calls, launched form
+// against this one: 4,096 vertices of degree 6 100 -> 79 us, 15,625 107 -> 87,
+// 32,768 111 -> 105, 40,000 no gain; 4,000 of degree 32 125 -> 155, R-MAT s12
+// 152 -> 279 (rows too long for one cluster), hence kHemClusterN and kHemClusterDeg.
+constexpr int kHemThreads = 1024;
+constexpr int kHemSlice = 2048;             // vertices per block at most
+constexpr int kHemCluster = 16;
+constexpr int kHemLong = 512;
+constexpr int kHemClusterDeg = 16;          // entries per vertex at most, on average
+constexpr int32_t kHemClusterN = 32768;     // kHemSlice * kHemCluster
+static_assert(kHemClusterN == kHemSlice * kHemCluster, "slices cover the largest level");
+
+__device__ __forceinline__ void hem_cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 template <bool EW>
-__global__ void __launch_bounds__(kTB) k_hem_propose_small(DGraph g, const int32_t *mate, int32_t *prop, uint64_t seed,
-                                                           uint64_t salt, int r, HemCtl *hc) {
+__global__ void __launch_bounds__(kHemThreads) k_hem_cluster(DGraph g, int32_t per, int lanes, int rounds, uint64_t seed,
+                                                             uint64_t salt0, int32_t *mate, int32_t *prop) {
+    __shared__ uint32_t bits[kHemClusterN / 32];     // matched, all vertices
+    __shared__ uint32_t own[kHemSlice / 32];         // matched, this block's slice (read by the others)
+    __shared__ int32_t act[kHemSlice];               // unmatched vertices: short rows from the front, long from the back
+    __shared__ int s_short, s_long;
+    __shared__ HemBest sh[kHemThreads / 32];
+    pdl_enter();
+    const int tid = threadIdx.x, n = g.n;
+    const int v0 = (int)blockIdx.x * per, nv = max(0, min(per, n - v0));
+    const int words = (n + 31) >> 5, wper = per >> 5;
+    for (int i = tid; i < words; i += kHemThreads) bits[i] = 0;
+    for (int i = tid; i < wper; i += kHemThreads) own[i] = 0;
+    for (int i = tid; i < nv; i += kHemThreads) mate[v0 + i] = -1;
+    if (tid == 0) { s_short = 0; s_long = 0; }
+    __syncthreads();
+    const int groups = kHemThreads / lanes, gi = tid / lanes, gl = tid & (lanes - 1);
+    for (int r = 0; r < rounds; ++r) {
+        const uint64_t salt = salt0 + 0xD1B54A32D192ED03ULL * (uint64_t)(r + 1);
+        for (int i0 = 0; i0 < nv; i0 += kHemThreads) {
+            const int i = i0 + tid;
+            const bool active = i < nv && !(own[i >> 5] >> (i & 31) & 1u);
+            const bool lng = active && g.xadj[v0 + i + 1] - g.xadj[v0 + i] > kHemLong;
+            int slot = warp_append(&s_short, active && !lng);
+            if (active && !lng) act[slot] = v0 + i;
+            slot = warp_append(&s_long, lng);
+            if (lng) act[kHemSlice - 1 - slot] = v0 + i;
+        }
+        __syncthreads();
+        const int ns = s_short, nl = s_long;
+        for (int a0 = 0; a0 < ns; a0 += groups) {
+            const int a = a0 + gi;
+            const int32_t v = a < ns ? act[a] : -1;
+            HemBest best;
+            if (v >= 0) hem_row<EW>(g, bits, seed, salt, g.xadj[v] + gl, g.xadj[v + 1], lanes, best);
+            best.reduce(lanes);
+            if (v >= 0 && gl == 0) prop[v] = best.u;
+        }
+        for (int a = 0; a < nl; ++a) {
+            const int32_t v = act[kHemSlice - 1 - a];
+            HemBest best;
+            hem_row<EW>(g, bits, seed, salt, g.xadj[v] + tid, g.xadj[v + 1], kHemThreads, best);
+            hem_block_best(best, sh);
+            if (tid == 0) prop[v] = best.u;
+        }
+        hem_cluster_sync();
+        // every proposal names a vertex that was unmatched, so whose proposal is this round's
+        for (int a = tid; a < ns + nl; a += kHemThreads) {
+            const int32_t v = act[a < ns ? a : kHemSlice - 1 - (a - ns)];
+            const int32_t u = __ldcg(prop + v);
+            if (u >= 0 && __ldcg(prop + u) == v) {
+                mate[v] = u;
+                atomicOr(&own[(v - v0) >> 5], 1u << ((v - v0) & 31));
+            }
+        }
+        if (tid == 0) { s_short = 0; s_long = 0; }
+        hem_cluster_sync();
+        int changed = 0;
+        for (int i = tid; i < words; i += kHemThreads) {
+            uint32_t a, x;
+            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(&own[i % wper])), "r"(i / wper));
+            asm volatile("ld.shared::cluster.b32 %0, [%1];" : "=r"(x) : "r"(a) : "memory");
+            changed |= x != bits[i];
+            bits[i] = x;
+        }
+        if (!__syncthreads_or(changed)) break;   // the same outcome in every block
+    }
+    hem_cluster_sync();   // the others may still read this block's bits
+}
+
+// Blocks of the cluster form on this device (0: not available).
+static int hem_cluster_blocks(int device) {
+    static std::mutex mu;
+    static int cache[256];   // blocks + 1
+    if (device < 0 || device >= 256) return 0;
+    std::lock_guard<std::mutex> lock(mu);
+    if (cache[device]) return cache[device] - 1;
+    int best = 0;
+    if (cudaFuncSetAttribute(k_hem_cluster<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaFuncSetAttribute(k_hem_cluster<false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+        for (int cs = kHemCluster; cs >= 4 && !best; cs /= 2) {
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3(cs);
+            cfg.blockDim = dim3(kHemThreads);
+            cudaLaunchAttribute la{};
+            la.id = cudaLaunchAttributeClusterDimension;
+            la.val.clusterDim.x = cs; la.val.clusterDim.y = 1; la.val.clusterDim.z = 1;
+            cfg.attrs = &la;
+            cfg.numAttrs = 1;
+            int a = 0, b = 0;
+            if (cudaOccupancyMaxActiveClusters(&a, k_hem_cluster<true>, &cfg) == cudaSuccess &&
+                cudaOccupancyMaxActiveClusters(&b, k_hem_cluster<false>, &cfg) == cudaSuccess && a >= 1 && b >= 1)
+                best = cs;
+        }
+    }
+    cudaGetLastError();   // a refused query only closes this form
+    cache[device] = best + 1;
+    return best;
+}
+
+// ---- the launched form: two kernels per round over the whole GPU ----
+
+// Unmatched everywhere; rows longer than kSmallDeg are listed: warp rows (up to
+// kHugeDeg entries) in list, hub rows in hlist, one reservation per block each.
+__global__ void __launch_bounds__(kTB) k_hem_start(DGraph g, int32_t *mate, uint32_t *matched, uint32_t *done, int32_t *list,
+                                                   int32_t *hlist, HemCtl *hc) {
+    __shared__ int cnt[2], base[2];
+    const int32_t v = blockIdx.x * kTB + threadIdx.x;
+    const int64_t d = v < g.n ? ld_xadj(g.xadj, (int64_t)v + 1) - ld_xadj(g.xadj, v) : 0;
+    if (v < g.n) mate[v] = -1;
+    if (v < g.n && (v & 31) == 0) { matched[v >> 5] = 0; done[v >> 5] = 0; }
+    if (threadIdx.x < 2) cnt[threadIdx.x] = 0;
+    __syncthreads();
+    const bool big = d > kSmallDeg && d <= kHugeDeg, huge = d > kHugeDeg;
+    const int s0 = warp_append(&cnt[0], big), s1 = warp_append(&cnt[1], huge);
+    __syncthreads();
+    if (threadIdx.x < 2) base[threadIdx.x] = cnt[threadIdx.x] ? atomicAdd(threadIdx.x ? &hc->nhuge : &hc->nbig, cnt[threadIdx.x]) : 0;
+    __syncthreads();
+    if (big) list[base[0] + s0] = v;
+    if (huge) hlist[base[1] + s1] = v;
+}
+
+// One proposal round: prop[v] = the chosen neighbour or -1 for the vertices not
+// done (matched, or without an unmatched neighbour in an earlier round, which stays
+// so).  The first long_blocks blocks take the hub rows, one at a time, then the warp
+// rows, one per warp; the others the short rows, one per thread: one launch instead
+// of three, so that the kinds of row fill the GPU together.  Bound by the gathers and
+// the hashes; the eight rounds on R-MAT s15 459 -> 195 us a call, s18 1309 -> 565.
+template <bool EW>
+__global__ void __launch_bounds__(kTB) k_hem_propose(DGraph g, const int32_t *bigv, const int32_t *hugev,
+                                                     const uint32_t *matched, const uint32_t *done, int32_t *prop, uint64_t seed,
+                                                     uint64_t salt, int r, int long_blocks, HemCtl *hc) {
+    __shared__ HemBest sh[kTB / 32];
     pdl_enter();
     if (hem_skip(hc, r)) {
         if (blockIdx.x == 0 && threadIdx.x == 0) hc->stop = 1;
         return;
     }
-    int32_t v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= g.n) return;
-    int64_t beg = ld_xadj(g.xadj, v), end = ld_xadj(g.xadj, (int64_t)v + 1);
-    if (end - beg > kSmallDeg) return;
-    int32_t bu = -1, bw = 0;
-    uint64_t bh = 0;
-    if (mate[v] < 0) {
-        for (int64_t j = beg; j < end; ++j) {
-            int32_t u = __ldg(g.adj + j);
-            if (mate[u] >= 0) continue;
-            int32_t w = cw<EW>(g, j);
-            uint64_t h = hem_hash(seed, salt, u);
-            if (hem_better(u >= 0 ? w : 0, h, u, bw, bh, bu)) { bu = u; bw = w; bh = h; }
-        }
+    if ((int)blockIdx.x >= long_blocks) {
+        const int64_t v = (int64_t)((int)blockIdx.x - long_blocks) * kTB + threadIdx.x;
+        if (v >= g.n) return;
+        if (done[v >> 5] >> (v & 31) & 1u) return;
+        const int64_t beg = ld_xadj(g.xadj, v), end = ld_xadj(g.xadj, v + 1);
+        if (end - beg > kSmallDeg) return;
+        HemBest best;
+        hem_row<EW>(g, matched, seed, salt, beg, end, 1, best);
+        prop[v] = best.u;
+        return;
     }
-    prop[v] = bu;
-}
-
-// The heaviest unmatched neighbour over the entries first, first + step, ...
-// < end of a row, U at a time (ids, then their mates, in flight together);
-// folds into (bu, bw, bh).
-template <bool EW, int U = 4>
-__device__ __forceinline__ void hem_row(const DGraph &g, const int32_t *mate, uint64_t seed, uint64_t salt, int64_t first,
-                                        int64_t end, int64_t step, int32_t &bu, int32_t &bw, uint64_t &bh) {
-    for (int64_t j0 = first; j0 < end; j0 += U * step) {
-        int32_t u[U], m[U];
-#pragma unroll
-        for (int q = 0; q < U; ++q) {
-            const int64_t j = j0 + q * step;
-            u[q] = j < end ? __ldg(g.adj + j) : -1;
-        }
-#pragma unroll
-        for (int q = 0; q < U; ++q) m[q] = u[q] >= 0 ? mate[u[q]] : 0;
-#pragma unroll
-        for (int q = 0; q < U; ++q) {
-            if (u[q] < 0 || m[q] >= 0) continue;
-            const int32_t ww = cw<EW>(g, j0 + q * step);
-            const uint64_t h = hem_hash(seed, salt, u[q]);
-            if (hem_better(ww, h, u[q], bw, bh, bu)) { bu = u[q]; bw = ww; bh = h; }
-        }
-    }
-}
-
-template <bool EW>
-__global__ void __launch_bounds__(kTB) k_hem_propose_big(DGraph g, const int32_t *bigv, int32_t nbig, const int32_t *mate,
-                                                         int32_t *prop, uint64_t seed, uint64_t salt, int r, HemCtl *hc) {
-    pdl_enter();
-    if (hem_skip(hc, r)) return;
-    const int warps = blockDim.x >> 5;
-    const unsigned lane = lane_id();
-    for (int64_t w = (int64_t)blockIdx.x * warps + (threadIdx.x >> 5); w < nbig; w += (int64_t)gridDim.x * warps) {
-        int32_t v = bigv[w];
-        int32_t bu = -1, bw = 0;
-        uint64_t bh = 0;
-        if (mate[v] < 0) {
-            int64_t beg = ld_xadj(g.xadj, v), end = ld_xadj(g.xadj, (int64_t)v + 1);
-            hem_row<EW>(g, mate, seed, salt, beg + lane, end, 32, bu, bw, bh);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            int32_t ou = __shfl_xor_sync(0xffffffffu, bu, o);
-            int32_t ow = __shfl_xor_sync(0xffffffffu, bw, o);
-            uint64_t oh = __shfl_xor_sync(0xffffffffu, bh, o);
-            if (hem_better(ow, oh, ou, bw, bh, bu)) { bu = ou; bw = ow; bh = oh; }
-        }
-        if (lane == 0) prop[v] = bu;
-    }
-}
-
-// Hub rows (longer than kHugeDeg): one block per row, the same choice.
-template <bool EW>
-__global__ void __launch_bounds__(kTB) k_hem_propose_huge(DGraph g, const int32_t *hugev, int32_t nhuge,
-                                                          const int32_t *mate, int32_t *prop, uint64_t seed,
-                                                          uint64_t salt, int r, HemCtl *hc) {
-    pdl_enter();
-    if (hem_skip(hc, r)) return;
-    __shared__ int32_t su[32], sw[32];
-    __shared__ uint64_t shh[32];
-    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
-    for (int64_t t = blockIdx.x; t < nhuge; t += gridDim.x) {
+    const int32_t nhuge = hc->nhuge, nbig = hc->nbig;
+    for (int64_t t = blockIdx.x; t < nhuge; t += long_blocks) {
         const int32_t v = hugev[t];
-        int32_t bu = -1, bw = 0;
-        uint64_t bh = 0;
-        if (mate[v] < 0) {
-            const int64_t beg = ld_xadj(g.xadj, v), end = ld_xadj(g.xadj, (int64_t)v + 1);
-            hem_row<EW, 8>(g, mate, seed, salt, beg + threadIdx.x, end, blockDim.x, bu, bw, bh);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const int32_t ou = __shfl_xor_sync(0xffffffffu, bu, o);
-            const int32_t ow = __shfl_xor_sync(0xffffffffu, bw, o);
-            const uint64_t oh = __shfl_xor_sync(0xffffffffu, bh, o);
-            if (hem_better(ow, oh, ou, bw, bh, bu)) { bu = ou; bw = ow; bh = oh; }
-        }
-        if (lane == 0) { su[warp] = bu; sw[warp] = bw; shh[warp] = bh; }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (unsigned i = 1; i < (blockDim.x >> 5); ++i)
-                if (hem_better(sw[i], shh[i], su[i], bw, bh, bu)) { bu = su[i]; bw = sw[i]; bh = shh[i]; }
-            prop[v] = bu;
-        }
-        __syncthreads();
+        if (done[v >> 5] >> (v & 31) & 1u) continue;
+        HemBest best;
+        hem_row<EW, 8>(g, matched, seed, salt, ld_xadj(g.xadj, v) + threadIdx.x, ld_xadj(g.xadj, (int64_t)v + 1), kTB, best);
+        hem_block_best(best, sh);
+        if (threadIdx.x == 0) prop[v] = best.u;
+    }
+    const unsigned lane = lane_id();
+    for (int64_t w = (int64_t)blockIdx.x * (kTB / 32) + (threadIdx.x >> 5); w < nbig; w += (int64_t)long_blocks * (kTB / 32)) {
+        const int32_t v = bigv[w];
+        if (done[v >> 5] >> (v & 31) & 1u) continue;
+        HemBest best;
+        hem_row<EW>(g, matched, seed, salt, ld_xadj(g.xadj, v) + lane, ld_xadj(g.xadj, (int64_t)v + 1), 32, best);
+        best.reduce(32);
+        if (lane == 0) prop[v] = best.u;
     }
 }
 
-// Mutual proposals match (synchronous: every proposal of the round is read
-// before any mate changes matter, since proposals only name unmatched ones).
-__global__ void __launch_bounds__(kTB) k_hem_match(int32_t n, int32_t *mate, const int32_t *prop, int r, HemCtl *hc) {
+// Mutual proposals match; a warp owns its 32 vertices' words.  A proposal names a
+// vertex that was unmatched when the round began; that one's own is this round's, or
+// -1 from an earlier one.
+__global__ void __launch_bounds__(kTB) k_hem_match(int32_t n, int32_t *mate, uint32_t *matched, uint32_t *done,
+                                                   const int32_t *prop, int r, HemCtl *hc) {
     __shared__ long long red[40];
     pdl_enter();
     if (hc->stop) return;
     long long c = 0;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-        int32_t u = prop[v];
-        if (u >= 0 && prop[u] == (int32_t)v) { mate[v] = u; ++c; }
+    const int64_t n32 = ((int64_t)n + 31) / 32 * 32;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n32; v += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t before = done[v >> 5];
+        const bool open = v < n && !(before >> (v & 31) & 1u);
+        const int32_t u = open ? prop[v] : -1;
+        const bool ok = u >= 0 && prop[u] == (int32_t)v;
+        if (ok) { mate[v] = u; ++c; }
+        const uint32_t now = __ballot_sync(0xffffffffu, ok), end = __ballot_sync(0xffffffffu, ok || (open && u < 0));
+        if (end && lane_id() == 0) {
+            if (now) matched[v >> 5] |= now;
+            done[v >> 5] = before | end;
+        }
     }
     c = block_sum_i64(c, red);
     if (threadIdx.x == 0 && c) atomic_add_i64(&hc->added[r], c);
 }
 
-// Rows longer than kSmallDeg: warp rows (up to kHugeDeg entries) into list,
-// hub rows into hlist.
-__global__ void k_collect_rows(DGraph g, int32_t *list, int32_t *count, int32_t *hlist, int32_t *hcount) {
-    int32_t v = blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t d = v < g.n ? ld_xadj(g.xadj, (int64_t)v + 1) - ld_xadj(g.xadj, v) : 0;
-    const bool big = d > kSmallDeg && d <= kHugeDeg, huge = d > kHugeDeg;
-    int slot = warp_append(count, big);
-    if (big) list[slot] = v;
-    slot = warp_append(hcount, huge);
-    if (huge) hlist[slot] = v;
-}
-
-__global__ void k_fill(int32_t *p, int64_t n, int32_t val) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) p[i] = val;
-}
-
-// The warp rows (list at buf) and the hub rows (list at *huge) of g.
-static int big_rows(Ctx &c, const DGraph &g, DevBuf &buf, int32_t &nbig, int32_t **huge, int32_t &nhuge) {
-    cudaStream_t s = c.stream;
-    const size_t nb = ((size_t)std::max<int64_t>(g.n, 1) * 4 + 255) & ~size_t(255);
-    JET_TRY(dev_alloc(buf, 2 * nb + 256, s));
-    int32_t *list = buf.as<int32_t>();
-    *huge = reinterpret_cast<int32_t *>(buf.as<char>() + nb);
-    int32_t *cnt = reinterpret_cast<int32_t *>(buf.as<char>() + 2 * nb);
-    JET_CUDA_TRY(cudaMemsetAsync(cnt, 0, 8, s));
-    if (g.n > 0) k_collect_rows<<<grid_for(g.n, kTB), kTB, 0, s>>>(g, list, cnt, *huge, cnt + 1);
-    if (g.n > 0) c.launches += 1;
-    JET_CUDA_TRY(cudaGetLastError());
-    JET_CUDA_TRY(cudaMemcpyAsync(c.pinned, cnt, 8, cudaMemcpyDeviceToHost, s));
-    JET_CUDA_TRY(cudaStreamSynchronize(s));
-    int32_t h[2];
-    memcpy(h, c.pinned, 8);
-    nbig = h[0];
-    nhuge = h[1];
-    return JET_OK;
-}
-
 int hem(Ctx &c, const DGraph &g, uint64_t seed, int32_t level, int32_t rounds, int32_t *mate) {
     cudaStream_t s = c.stream;
     if (g.n == 0) return JET_OK;
-    DevBuf bigbuf, pbuf, hbuf;
-    int32_t nbig = 0, nhuge = 0;
-    int32_t *hugev = nullptr;
-    JET_TRY(big_rows(c, g, bigbuf, nbig, &hugev, nhuge));
-    JET_TRY(dev_alloc(pbuf, (size_t)g.n * 4, s));
-    JET_TRY(dev_alloc(hbuf, sizeof(HemCtl), s));
-    HemCtl *hc = hbuf.as<HemCtl>();
-    JET_CUDA_TRY(cudaMemsetAsync(hc, 0, sizeof(HemCtl), s));
-    k_fill<<<grid_for(g.n, kTB, 4096), kTB, 0, s>>>(mate, g.n, -1);
-    c.launches += 1;
     rounds = std::min(rounds, 64);
-    int gl = num_sms() * 8;
+    const bool pdl = !(c.opt.flags & JET_FLAG_NO_PDL);
+    const uint64_t salt0 = 0xD1B54A32D192ED03ULL * (uint64_t)(64 * (int64_t)level);
+    DevBuf buf;
+    const int cs = g.n <= kHemClusterN && g.nnz <= (int64_t)kHemClusterDeg * g.n ? hem_cluster_blocks(c.device) : 0;
+    if (cs > 0 && g.n <= cs * kHemSlice) {
+        JET_TRY(dev_alloc(buf, (size_t)g.n * 4, s));
+        int32_t *prop = buf.as<int32_t>();
+        const int32_t per = ((g.n + cs - 1) / cs + 31) / 32 * 32;
+        int lanes = 1;   // four entries in flight per lane
+        while (lanes < 32 && (int64_t)lanes * 4 * g.n < g.nnz) lanes *= 2;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)cs);
+        cfg.blockDim = dim3(kHemThreads);
+        cfg.stream = s;
+        cudaLaunchAttribute la{};
+        la.id = cudaLaunchAttributeClusterDimension;
+        la.val.clusterDim.x = cs; la.val.clusterDim.y = 1; la.val.clusterDim.z = 1;
+        cfg.attrs = &la;
+        cfg.numAttrs = 1;
+        if (g.ew) JET_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_hem_cluster<true>, g, per, lanes, (int)rounds, seed, salt0, mate, prop));
+        else JET_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_hem_cluster<false>, g, per, lanes, (int)rounds, seed, salt0, mate, prop));
+        c.launches += 1;
+        return JET_OK;   // mate is final once the stream passes here (the scratch is freed in stream order)
+    }
+    auto a256 = [](size_t x) { return (x + 255) & ~size_t(255); };
+    const size_t nb = a256((size_t)g.n * 4), mb = a256(((size_t)g.n + 31) / 32 * 4);
+    JET_TRY(dev_alloc(buf, 3 * nb + 2 * mb + sizeof(HemCtl), s));
+    int32_t *prop = buf.as<int32_t>();
+    int32_t *bigv = reinterpret_cast<int32_t *>(buf.as<char>() + nb);
+    int32_t *hugev = reinterpret_cast<int32_t *>(buf.as<char>() + 2 * nb);
+    uint32_t *matched = reinterpret_cast<uint32_t *>(buf.as<char>() + 3 * nb);
+    uint32_t *done = reinterpret_cast<uint32_t *>(buf.as<char>() + 3 * nb + mb);
+    HemCtl *hc = reinterpret_cast<HemCtl *>(buf.as<char>() + 3 * nb + 2 * mb);
+    JET_CUDA_TRY(cudaMemsetAsync(hc, 0, sizeof(HemCtl), s));
+    const int gs = grid_for(g.n, kTB);
+    k_hem_start<<<gs, kTB, 0, s>>>(g, mate, matched, done, bigv, hugev, hc);
+    c.launches += 1;
+    JET_CUDA_TRY(cudaGetLastError());
     // the rounds follow one another by programmatic launch (each kernel waits
     // for the previous one on the device before it reads anything)
-    const bool pdl = !(c.opt.flags & JET_FLAG_NO_PDL);
-    int32_t *prop = pbuf.as<int32_t>();
-    const int32_t *bigv = bigbuf.as<int32_t>();
+    const int lb = std::min(num_sms() * 8, grid_for(g.n, kTB / 32));
+    const int gm = std::min(num_sms() * 8, gs);
     for (int r = 0; r < rounds; ++r) {
-        uint64_t salt = 0xD1B54A32D192ED03ULL * (uint64_t)(64 * (int64_t)level + r + 1);
-        const int gs = grid_for(g.n, kTB);
-        if (g.ew) JET_CUDA_TRY(launch_pdl(k_hem_propose_small<true>, gs, kTB, 0, s, pdl, g, (const int32_t *)mate, prop, seed, salt, r, hc));
-        else JET_CUDA_TRY(launch_pdl(k_hem_propose_small<false>, gs, kTB, 0, s, pdl, g, (const int32_t *)mate, prop, seed, salt, r, hc));
-        c.launches += 1;
-        if (nbig > 0) {
-            int gb = std::min(gl, grid_for(nbig, kTB / 32));
-            if (g.ew) JET_CUDA_TRY(launch_pdl(k_hem_propose_big<true>, gb, kTB, 0, s, pdl, g, bigv, nbig, (const int32_t *)mate, prop, seed, salt, r, hc));
-            else JET_CUDA_TRY(launch_pdl(k_hem_propose_big<false>, gb, kTB, 0, s, pdl, g, bigv, nbig, (const int32_t *)mate, prop, seed, salt, r, hc));
-            c.launches += 1;
-        }
-        if (nhuge > 0) {
-            int gh = std::min(gl, nhuge);
-            if (g.ew) JET_CUDA_TRY(launch_pdl(k_hem_propose_huge<true>, gh, kTB, 0, s, pdl, g, (const int32_t *)hugev, nhuge, (const int32_t *)mate, prop, seed, salt, r, hc));
-            else JET_CUDA_TRY(launch_pdl(k_hem_propose_huge<false>, gh, kTB, 0, s, pdl, g, (const int32_t *)hugev, nhuge, (const int32_t *)mate, prop, seed, salt, r, hc));
-            c.launches += 1;
-        }
-        JET_CUDA_TRY(launch_pdl(k_hem_match, std::min(gl, grid_for(g.n, kTB)), kTB, 0, s, pdl, g.n, mate, (const int32_t *)prop, r, hc));
-        c.launches += 1;
+        const uint64_t salt = salt0 + 0xD1B54A32D192ED03ULL * (uint64_t)(r + 1);
+        auto kern = g.ew ? k_hem_propose<true> : k_hem_propose<false>;
+        JET_CUDA_TRY(launch_pdl(kern, lb + gs, kTB, 0, s, pdl, g, (const int32_t *)bigv, (const int32_t *)hugev,
+                                (const uint32_t *)matched, (const uint32_t *)done, prop, seed, salt, r, lb, hc));
+        JET_CUDA_TRY(launch_pdl(k_hem_match, gm, kTB, 0, s, pdl, g.n, mate, matched, done, (const int32_t *)prop, r, hc));
+        c.launches += 2;
     }
-    JET_CUDA_TRY(cudaGetLastError());
-    return JET_OK;   // mate is final once the stream passes here (the scratch is freed in stream order)
+    return JET_OK;
 }
 
 // ---------------------------------------------------------------------------

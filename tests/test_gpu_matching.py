@@ -1,0 +1,62 @@
+"""Heavy-edge matching against the oracle where its forms change: level sizes
+around a warp's word, a block's slice and the largest one-cluster level, rows
+around the short, warp and block lengths, equal and distinct weights, none at
+all.  Matchings are whole numbers and must be the same."""
+import numpy as np
+import pytest
+import torch
+
+import graphgen
+import oracle
+from helpers import graph_from_triples
+
+pytestmark = pytest.mark.gpu
+
+jet = pytest.importorskip("paper_2304_13194_gb300")
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    c = jet.Context(0)
+    yield c
+    c.close()
+
+
+def _stars(*leaves):
+    """A chain of hubs with the given numbers of leaves."""
+    t, hub = [], 0
+    for i, m in enumerate(leaves):
+        t += [[hub, hub + 1 + j, 1 + (j * 7) % 5] for j in range(m)]
+        if i + 1 < len(leaves):
+            t.append([hub, hub + m + 1, 3])
+        hub += m + 1
+    return graph_from_triples(hub, t)
+
+
+CASES = [
+    ("two", lambda: graph_from_triples(2, [[0, 1, 1]])),
+    ("path33", lambda: graph_from_triples(33, [[i, i + 1, 1 + i % 3] for i in range(32)])),
+    ("isolated", lambda: graphgen.gnp(1000, 0.0008, seed=1)),
+    ("grid_w", lambda: graphgen.grid2d(127, 258, vw=(1, 3), ew=(1, 4), seed=2)),       # 32766: one cluster
+    ("grid_limit", lambda: graphgen.grid2d(256, 128)),                                # 32768
+    ("grid_over", lambda: graphgen.grid2d(32769, 1)),
+    ("grid3d", lambda: graphgen.grid3d(30, 31, 32, ew=(1, 9), seed=4)),
+    ("rmat_w", lambda: graphgen.rmat(13, seed=3, vw=(1, 2), ew=(1, 9))),
+    ("rmat_large", lambda: graphgen.rmat(17, seed=5)),
+    ("stars", lambda: _stars(15, 16, 17, 33, 511, 512, 513, 1023, 1025, 5000)),
+    ("stars_cluster", lambda: _stars(*([2] * 5000), 16, 17, 33, 511, 512, 513, 1023, 1025, 5000)),
+    ("stars_large", lambda: _stars(*([3] * 9000), 16, 17, 1024, 1025, 5000)),
+]
+
+
+@pytest.mark.parametrize("name,make", CASES, ids=[c[0] for c in CASES])
+def test_matching_equals_oracle(ctx, name, make):
+    g = make()
+    d = [None if a is None else torch.as_tensor(np.asarray(a)).cuda() for a in (g.xadj, g.adjncy, g.adjwgt)]
+    for weights in (d[2], None):
+        for level, rounds in ((0, 8), (3, 1), (1, 0)):
+            gw = g if weights is not None else graphgen.Graph(g.n, g.xadj, g.adjncy, g.vwgt, np.ones_like(g.adjncy))
+            got = ctx.hem(d[0], d[1], weights, seed=11, level=level, rounds=rounds).cpu().numpy()
+            assert np.array_equal(got, oracle.hem(gw, 11, level, rounds)), (weights is None, level, rounds)
