@@ -24,8 +24,8 @@ __device__ __forceinline__ int32_t cw(const DGraph &g, int64_t j) {
     else return 1;
 }
 
-// Phase 2 of device_exscan: exclusive scan of the tile sums (one block).
-__global__ void __launch_bounds__(1024) k_scan_sums(int64_t *tile_sums, int64_t ntiles, int64_t *total_dev) {
+// device_exscan over many tiles: exclusive scan of the tile sums (one block).
+__global__ void __launch_bounds__(1024) k_scan_sums(int64_t *tile_sums, int64_t ntiles) {
     __shared__ long long sh[40];
     pdl_enter();
     long long carry = 0;
@@ -37,7 +37,6 @@ __global__ void __launch_bounds__(1024) k_scan_sums(int64_t *tile_sums, int64_t 
         if (t < ntiles) tile_sums[t] = carry + ex;
         carry += tot;
     }
-    if (threadIdx.x == 0 && total_dev) *total_dev = carry;
 }
 
 // Matching state between the rounds of the launched form.
@@ -413,10 +412,14 @@ __global__ void k_cmap(int32_t n, const int32_t *mate, const int64_t *cidx, int3
     }
 }
 
+// Entries of coarse row c before merging; 0 past the last row, whose number only
+// the device knows when the scan is launched.
 struct RowBound {
     const int64_t *xadj;
     const int32_t *crep, *mate;
+    const int64_t *nc;
     __device__ int64_t operator()(int64_t c) const {
+        if (c >= *nc) return 0;
         int32_t r = crep[c];
         int32_t m = mate[r];
         int64_t b = xadj[r + 1] - xadj[r];
@@ -457,35 +460,46 @@ struct HubFlag {
     __device__ int64_t operator()(int64_t c) const { return hb(c) > 0 ? 1 : 0; }
 };
 
-// Coarse vertex weights, and the coarse rows sorted into classes by their
-// bound (entries of the merged fine rows): <= 16 and <= 32 (one thread),
-// <= kWarpSort (one warp), longer (one block).  counts = {warp rows, block
-// rows, 16-entry thread rows, 32-entry thread rows}.
+// What the host learns about a coarse level in one read.
+struct LevelCount {
+    int64_t nc;            // coarse vertices
+    int64_t btotal;        // entries of all rows before merging
+    int64_t htotal, nhub;  // entries and number of the hub rows
+    int32_t rows[4];       // {warp rows, block rows, 16-entry thread rows, 32-entry thread rows}
+};
+
+// The coarse rows sorted into classes by their bound (entries of the merged fine
+// rows): <= 16 and <= 32 (one thread), <= kWarpSort (one warp), longer (one block,
+// hub rows among them).  boff has an entry past the last row (nc < n for every
+// level that is built; a level without a match is dropped).
 constexpr int kWarpSort = 256;
-__global__ void k_coarse_vw(int32_t nc, const int32_t *crep, const int32_t *mate, const int32_t *vw, int32_t *vwc,
-                            int32_t *warp_list, int32_t *large_list, int32_t *t16_list, int32_t *t32_list,
-                            int32_t *counts, const int64_t *boff, const int64_t *btot) {
+__global__ void __launch_bounds__(kTB) k_row_classes(int32_t n, const int64_t *boff, LevelCount *lc, int32_t *warp_list,
+                                                     int32_t *large_list, int32_t *t16_list, int32_t *t32_list) {
+    __shared__ int cnt[4], base[4];
     pdl_enter();
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < ((int64_t)nc + 31) / 32 * 32;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        bool valid = c < nc;
-        int64_t b = 0;
-        if (valid) {
-            int32_t r = crep[c];
-            int32_t m = mate[r];
-            vwc[c] = vw[r] + (m >= 0 ? vw[m] : 0);
-            b = (c + 1 < nc ? boff[c + 1] : *btot) - boff[c];
+    const int64_t nc = lc->nc;
+    if (nc >= n) return;
+    const int64_t rounded = (nc + kTB - 1) / kTB * kTB;
+    for (int64_t c = (int64_t)blockIdx.x * kTB + threadIdx.x; c < rounded; c += (int64_t)gridDim.x * kTB) {
+        if (threadIdx.x < 4) cnt[threadIdx.x] = 0;
+        __syncthreads();
+        const int64_t b = c < nc ? boff[c + 1] - boff[c] : -1;
+        const int cls = b < 0 ? -1 : b <= 16 ? 2 : b <= 32 ? 3 : b <= kWarpSort ? 0 : 1;
+        int slot[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) slot[q] = warp_append(&cnt[q], cls == q);
+        if (b > kSortSmem) {
+            atomic_add_i64(&lc->htotal, b);
+            atomic_add_i64(&lc->nhub, 1);
         }
-        const bool t16 = valid && b <= 16, t32 = valid && b > 16 && b <= 32;
-        const bool wr = valid && b > 32 && b <= kWarpSort, large = valid && b > kWarpSort;
-        int s0 = warp_append(&counts[2], t16);
-        if (t16) t16_list[s0] = (int32_t)c;
-        int s1 = warp_append(&counts[3], t32);
-        if (t32) t32_list[s1] = (int32_t)c;
-        int s2 = warp_append(&counts[0], wr);
-        if (wr) warp_list[s2] = (int32_t)c;
-        int s3 = warp_append(&counts[1], large);
-        if (large) large_list[s3] = (int32_t)c;
+        __syncthreads();
+        if (threadIdx.x < 4) base[threadIdx.x] = cnt[threadIdx.x] ? atomicAdd(&lc->rows[threadIdx.x], cnt[threadIdx.x]) : 0;
+        __syncthreads();
+        if (cls == 0) warp_list[base[0] + slot[0]] = (int32_t)c;
+        if (cls == 1) large_list[base[1] + slot[1]] = (int32_t)c;
+        if (cls == 2) t16_list[base[2] + slot[2]] = (int32_t)c;
+        if (cls == 3) t32_list[base[3] + slot[3]] = (int32_t)c;
+        __syncthreads();
     }
 }
 
@@ -702,12 +716,6 @@ struct CountVal {
     __device__ int64_t operator()(int64_t c) const { return cnt[c]; }
 };
 
-__global__ void k_finish_xadj(int32_t nc, const int64_t *ex, const int64_t *tot, int64_t *xadj_c) {
-    pdl_enter();
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c <= nc; c += (int64_t)gridDim.x * blockDim.x)
-        xadj_c[c] = c < nc ? ex[c] : *tot;
-}
-
 // Hub rows, step 1: every entry of hub row c becomes (rank(c) << 32 | C[u],
 // w) at its segment hoff[c] + i (one block per row).
 template <bool EW>
@@ -799,15 +807,19 @@ __global__ void __launch_bounds__(kTB) k_copy_long(const int32_t *list, const in
 // short; a warp per row left most lanes idle and serialised the rows'
 // round trips).
 constexpr int kCopyLanes = 8;
-__global__ void k_copy_rows(int32_t nc, const int64_t *boff, const int64_t *btot, const int64_t *xadj_c,
-                            const int32_t *tadj, const int32_t *tw, int32_t *adj_c, int32_t *ew_c) {
+__global__ void k_copy_rows(int32_t nc, const int64_t *boff, const int64_t *xadj_c, const int32_t *crep, const int32_t *mate,
+                            const int32_t *vw, int32_t *vw_c, const int32_t *tadj, const int32_t *tw, int32_t *adj_c,
+                            int32_t *ew_c) {
     pdl_enter();
     const int64_t groups = (int64_t)gridDim.x * blockDim.x / kCopyLanes;
     const int gl = (int)(threadIdx.x % kCopyLanes);
     for (int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kCopyLanes; c < nc; c += groups) {
+        if (gl == 0) {   // the coarse vertex weight
+            const int32_t r = crep[c], m = mate[r];
+            vw_c[c] = vw[r] + (m >= 0 ? vw[m] : 0);
+        }
         const int64_t src = boff[c], dst = xadj_c[c], len = xadj_c[c + 1] - dst;
-        const int64_t bound = (c + 1 < nc ? boff[c + 1] : *btot) - src;
-        if (bound > kWarpSort) continue;   // k_copy_long
+        if (boff[c + 1] - src > kWarpSort) continue;   // k_copy_long
         for (int64_t i = gl; i < len; i += kCopyLanes) {
             adj_c[dst + i] = tadj[src + i];
             ew_c[dst + i] = tw[src + i];
@@ -816,147 +828,130 @@ __global__ void k_copy_rows(int32_t nc, const int64_t *boff, const int64_t *btot
 }
 
 // One coarsening level: matching, map, contraction.  Returns JET_OK and sets
-// stalled=true (without building the level) when n_c > 0.95 n.
+// stalled=true (without building the level) when n_c > 0.95 n.  Small levels are
+// bound by launches and host waits: the row classes are made before the host
+// knows the number of coarse vertices, so that it waits twice per level, for the
+// sizes of the work and of the result, and empty classes are not launched (564
+// launches, four waits and 2.9 ms for the 12 levels of a 110,592-vertex mesh before).
 static int coarsen_level(Ctx &c, const DGraph &g, uint64_t seed, int32_t level, jet_hier *h, bool &stalled) {
     cudaStream_t s = c.stream;
     stalled = false;
-    int64_t n = g.n;
-    DevBuf mbuf, cidxb, scan_scr, tot;
-    JET_TRY(dev_alloc(mbuf, (size_t)n * 4, s));
-    int32_t *mate = mbuf.as<int32_t>();
+    const int64_t n = g.n;
+    auto a256 = [](size_t x) { return (x + 255) & ~size_t(255); };
+    DevBuf scratch, cmapb, work, vb, eb, hubb, hsortb, hsb;   // scratch is freed in stream order
+    const size_t nn = (size_t)n;
+    JET_TRY(dev_alloc(scratch, 256 + 2 * a256((nn + 1) * 8) + a256((size_t)(scan_tiles_for(n) + 1) * 8) + 6 * a256(nn * 4), s));
+    char *p = scratch.as<char>();
+    auto take = [&](size_t b) { char *r = p; p += a256(b); return r; };
+    LevelCount *lc = reinterpret_cast<LevelCount *>(take(sizeof(LevelCount)));
+    int64_t *boff = reinterpret_cast<int64_t *>(take((nn + 1) * 8));
+    int64_t *cidx = reinterpret_cast<int64_t *>(take((nn + 1) * 8));
+    int64_t *scan_scr = reinterpret_cast<int64_t *>(take((size_t)(scan_tiles_for(n) + 1) * 8));
+    int32_t *mate = reinterpret_cast<int32_t *>(take(nn * 4)), *crep = reinterpret_cast<int32_t *>(take(nn * 4));
+    int32_t *warp_list = reinterpret_cast<int32_t *>(take(nn * 4)), *large_list = reinterpret_cast<int32_t *>(take(nn * 4));
+    int32_t *t16_list = reinterpret_cast<int32_t *>(take(nn * 4)), *t32_list = reinterpret_cast<int32_t *>(take(nn * 4));
+    JET_TRY(dev_alloc(cmapb, nn * 4, s));   // owned by the hierarchy
+    int32_t *cmap = cmapb.as<int32_t>();
+    JET_CUDA_TRY(cudaMemsetAsync(lc, 0, sizeof(LevelCount), s));
     JET_TRY(hem(c, g, seed, level, c.opt.hem_rounds, mate));
     if (c.opt.flags & JET_FLAG_TWO_HOP) {
         int64_t added[3];
         JET_TRY(two_hop(c, g, mate, added));
     }
-    JET_TRY(dev_alloc(cidxb, (size_t)n * 8, s));
-    JET_TRY(dev_alloc(scan_scr, (size_t)std::max<int64_t>(scan_tiles_for(n), 1) * 8 * 2 + 64, s));
-    JET_TRY(dev_alloc(tot, 64, s));
-    int64_t *totp = tot.as<int64_t>();
-    c.launches += 3;
-    JET_TRY(device_exscan(RepFlag{mate}, n, cidxb.as<int64_t>(), totp, scan_scr.as<int64_t>(), s));
-    JET_CUDA_TRY(cudaMemcpyAsync(c.pinned, totp, 8, cudaMemcpyDeviceToHost, s));
+    JET_TRY(device_exscan(RepFlag{mate}, n, cidx, &lc->nc, scan_scr, s));
+    JET_CUDA_TRY(launch_pdl(k_cmap, grid_for(n, kTB, 8192), kTB, 0, s, true, g.n, (const int32_t *)mate, (const int64_t *)cidx,
+                            cmap, crep));
+    JET_TRY(device_exscan(RowBound{g.xadj, crep, mate, &lc->nc}, n, boff, &lc->btotal, scan_scr, s));
+    JET_CUDA_TRY(launch_pdl(k_row_classes, grid_for(n, kTB, num_sms() * 8), kTB, 0, s, true, g.n, (const int64_t *)boff, lc,
+                            warp_list, large_list, t16_list, t32_list));
+    c.launches += 2 + 2 * scan_launches(n);
+    JET_CUDA_TRY(cudaMemcpyAsync(c.pinned, lc, sizeof(LevelCount), cudaMemcpyDeviceToHost, s));
     JET_CUDA_TRY(cudaStreamSynchronize(s));
-    int64_t nc = c.pinned[0];
+    LevelCount hc;
+    memcpy(&hc, c.pinned, sizeof(hc));
+    const int64_t nc = hc.nc;
     if (100 * nc > 95 * n) { stalled = true; return JET_OK; }
-    // cmap (owned by the hierarchy) and representatives
-    DevBuf cmapb, crepb;
-    JET_TRY(dev_alloc(cmapb, (size_t)n * 4, s));
-    JET_TRY(dev_alloc(crepb, (size_t)std::max<int64_t>(nc, 1) * 4, s));
-    int32_t *cmap = cmapb.as<int32_t>(), *crep = crepb.as<int32_t>();
-    JET_CUDA_TRY(launch_pdl(k_cmap, grid_for(n, kTB, 8192), kTB, 0, s, true, g.n, (const int32_t *)mate,
-                            (const int64_t *)cidxb.as<int64_t>(), cmap, crep));
-    c.launches += 1;
-    // bounds of the coarse rows
-    DevBuf boffb, hoffb, hrankb;
-    JET_TRY(dev_alloc(boffb, (size_t)std::max<int64_t>(nc, 1) * 8, s));
-    JET_TRY(dev_alloc(hoffb, (size_t)std::max<int64_t>(nc, 1) * 8, s));
-    JET_TRY(dev_alloc(hrankb, (size_t)std::max<int64_t>(nc, 1) * 8, s));
-    int64_t *boff = boffb.as<int64_t>(), *hoff = hoffb.as<int64_t>(), *hrank = hrankb.as<int64_t>();
-    c.launches += 9;
-    JET_TRY(device_exscan(RowBound{g.xadj, crep, mate}, nc, boff, totp, scan_scr.as<int64_t>(), s));
-    const HubBound hb{crep, mate, g.xadj};
-    JET_TRY(device_exscan(hb, nc, hoff, totp + 1, scan_scr.as<int64_t>(), s));
-    JET_TRY(device_exscan(HubFlag{hb}, nc, hrank, totp + 3, scan_scr.as<int64_t>(), s));
-    JET_CUDA_TRY(cudaMemcpyAsync(c.pinned, totp, 32, cudaMemcpyDeviceToHost, s));
-    JET_CUDA_TRY(cudaStreamSynchronize(s));
-    int64_t btotal = c.pinned[0], htotal = c.pinned[1], nhub = c.pinned[3];
-    // coarse vertex weights and row classes
-    DevBuf vwcb, lists, tadjb, twb, cntb, hsortb, hubcb, hsb;
-    JET_TRY(dev_alloc(vwcb, (size_t)std::max<int64_t>(nc, 1) * 4, s));
-    const int64_t ncl = std::max<int64_t>(nc, 1);
-    JET_TRY(dev_alloc(lists, (size_t)ncl * 16 + 64, s));
-    int32_t *warp_list = lists.as<int32_t>(), *large_list = warp_list + ncl;
-    int32_t *t16_list = large_list + ncl, *t32_list = t16_list + ncl;
-    int32_t *counts = t32_list + ncl;
-    JET_CUDA_TRY(cudaMemsetAsync(counts, 0, 16, s));
-    JET_CUDA_TRY(launch_pdl(k_coarse_vw, grid_for(nc, kTB, 8192), kTB, 0, s, true, (int32_t)nc, (const int32_t *)crep,
-                            (const int32_t *)mate, g.vw, vwcb.as<int32_t>(), warp_list, large_list, t16_list, t32_list,
-                            counts, (const int64_t *)boff, (const int64_t *)totp));
-    JET_TRY(dev_alloc(tadjb, (size_t)std::max<int64_t>(btotal, 1) * 4, s));
-    JET_TRY(dev_alloc(twb, (size_t)std::max<int64_t>(btotal, 1) * 4, s));
-    JET_TRY(dev_alloc(cntb, (size_t)std::max<int64_t>(nc, 1) * 4, s));
-    int gl = num_sms() * 8;
-    const int gwarp = std::min(gl, grid_for(nc, kTB / 32));
-    const int glarge = std::min(num_sms() * 4, (int)std::max<int64_t>(1, nc));
-    const int gthread = std::min(gl, grid_for(nc, kTB));
-    int32_t *tadj = tadjb.as<int32_t>(), *tw = twb.as<int32_t>(), *cnt = cntb.as<int32_t>();
-    {
-        const int32_t *cm = cmap, *mt = mate, *cr = crep, *cts = counts;
-        const int64_t *bo = boff;
-        if (g.ew) {
-            JET_CUDA_TRY(launch_pdl(k_contract_thread<true, 16>, gthread, kTB, 0, s, true, g, cm, mt, cr, (const int32_t *)t16_list, cts, bo, tadj, tw, cnt));
-            JET_CUDA_TRY(launch_pdl(k_contract_thread<true, 32>, gthread, kTB, 0, s, true, g, cm, mt, cr, (const int32_t *)t32_list, cts, bo, tadj, tw, cnt));
-            JET_CUDA_TRY(launch_pdl(k_contract_warp<true>, gwarp, kTB, 0, s, true, g, cm, mt, cr, (const int32_t *)warp_list, cts, bo, tadj, tw, cnt));
-            JET_CUDA_TRY(launch_pdl(k_contract_large<true>, glarge, kTB, 0, s, true, g, cm, mt, cr, (const int32_t *)large_list, cts, bo, tadj, tw, cnt));
-        } else {
-            JET_CUDA_TRY(launch_pdl(k_contract_thread<false, 16>, gthread, kTB, 0, s, true, g, cm, mt, cr, (const int32_t *)t16_list, cts, bo, tadj, tw, cnt));
-            JET_CUDA_TRY(launch_pdl(k_contract_thread<false, 32>, gthread, kTB, 0, s, true, g, cm, mt, cr, (const int32_t *)t32_list, cts, bo, tadj, tw, cnt));
-            JET_CUDA_TRY(launch_pdl(k_contract_warp<false>, gwarp, kTB, 0, s, true, g, cm, mt, cr, (const int32_t *)warp_list, cts, bo, tadj, tw, cnt));
-            JET_CUDA_TRY(launch_pdl(k_contract_large<false>, glarge, kTB, 0, s, true, g, cm, mt, cr, (const int32_t *)large_list, cts, bo, tadj, tw, cnt));
-        }
-    }
-    c.launches += 4;
-    if (nhub > 0) {
+    const size_t ncl = (size_t)std::max<int64_t>(nc, 1);
+    // merged rows
+    const size_t bt = a256((size_t)std::max<int64_t>(hc.btotal, 1) * 4);
+    JET_TRY(dev_alloc(work, 2 * bt + a256(ncl * 4) + 256, s));
+    int32_t *tadj = work.as<int32_t>(), *tw = reinterpret_cast<int32_t *>(work.as<char>() + bt);
+    int32_t *cnt = reinterpret_cast<int32_t *>(work.as<char>() + 2 * bt);
+    int64_t *hub_total = reinterpret_cast<int64_t *>(work.as<char>() + 2 * bt + a256(ncl * 4));
+    const size_t xb = a256((ncl + 1) * 8);
+    JET_TRY(dev_alloc(vb, xb + ncl * 4, s));
+    int64_t *xc = vb.as<int64_t>();
+    int32_t *vwc = reinterpret_cast<int32_t *>(vb.as<char>() + xb);
+    const int gl = num_sms() * 8;
+    const int gwarp = std::min(gl, grid_for(hc.rows[0], kTB / 32)), glarge = std::max(1, std::min(num_sms() * 4, hc.rows[1]));
+    const int32_t *cm = cmap, *mt = mate, *cr = crep, *cts = lc->rows;
+    const int64_t *bo = boff;
+    auto contract = [&](auto kern, int slot, int grid, const int32_t *list) -> int {
+        if (hc.rows[slot] == 0) return JET_OK;
+        JET_CUDA_TRY(launch_pdl(kern, grid, kTB, 0, s, true, g, cm, mt, cr, list, cts, bo, tadj, tw, cnt));
+        c.launches += 1;
+        return JET_OK;
+    };
+    JET_TRY(contract(g.ew ? k_contract_thread<true, 16> : k_contract_thread<false, 16>, 2, std::min(gl, grid_for(hc.rows[2], kTB)), t16_list));
+    JET_TRY(contract(g.ew ? k_contract_thread<true, 32> : k_contract_thread<false, 32>, 3, std::min(gl, grid_for(hc.rows[3], kTB)), t32_list));
+    JET_TRY(contract(g.ew ? k_contract_warp<true> : k_contract_warp<false>, 0, gwarp, warp_list));
+    JET_TRY(contract(g.ew ? k_contract_large<true> : k_contract_large<false>, 1, glarge, large_list));
+    if (hc.nhub > 0) {
         // hub rows: all their entries in one stable radix sort by (rank, coarse id)
+        const int64_t htotal = hc.htotal, nhub = hc.nhub;
+        JET_TRY(dev_alloc(hubb, 2 * a256(ncl * 8) + (size_t)nhub * 4, s));
+        int64_t *hoff = hubb.as<int64_t>(), *hrank = reinterpret_cast<int64_t *>(hubb.as<char>() + a256(ncl * 8));
+        int32_t *hub_c = reinterpret_cast<int32_t *>(hubb.as<char>() + 2 * a256(ncl * 8));
+        const HubBound hb{crep, mate, g.xadj};
+        JET_TRY(device_exscan(hb, nc, hoff, nullptr, scan_scr, s));
+        JET_TRY(device_exscan(HubFlag{hb}, nc, hrank, nullptr, scan_scr, s));
         JET_TRY(dev_alloc(hsortb, sort_scratch_bytes(htotal), s));
         SortScratch sc;
         sort_scratch_carve(hsortb.as<char>(), htotal, sc);
-        JET_TRY(dev_alloc(hubcb, (size_t)nhub * 4, s));
         JET_TRY(dev_alloc(hsb, (size_t)htotal * 8 + (size_t)(scan_tiles_for(htotal) + 1) * 8 + 64, s));
-        int32_t *hub_c = hubcb.as<int32_t>();
         int64_t *hs = hsb.as<int64_t>(), *hs_scr = hs + htotal;
-        if (g.ew) k_hub_fill<true><<<glarge, kTB, 0, s>>>(g, cmap, mate, crep, large_list, counts, hoff, hrank, sc.key[0], sc.val[0], hub_c);
-        else k_hub_fill<false><<<glarge, kTB, 0, s>>>(g, cmap, mate, crep, large_list, counts, hoff, hrank, sc.key[0], sc.val[0], hub_c);
-        c.launches += 1;
+        if (g.ew) k_hub_fill<true><<<glarge, kTB, 0, s>>>(g, cmap, mate, crep, large_list, cts, hoff, hrank, sc.key[0], sc.val[0], hub_c);
+        else k_hub_fill<false><<<glarge, kTB, 0, s>>>(g, cmap, mate, crep, large_list, cts, hoff, hrank, sc.key[0], sc.val[0], hub_c);
         JET_CUDA_TRY(cudaGetLastError());
         int which = 0;
         JET_TRY(sort_pairs(c, sc, htotal, 32 + bits_for(nhub - 1), &which));
-        JET_TRY(device_exscan(HubHead{sc.key[which], hub_c}, htotal, hs, totp + 4, hs_scr, s));
+        JET_TRY(device_exscan(HubHead{sc.key[which], hub_c}, htotal, hs, hub_total, hs_scr, s));
         k_hub_emit<<<std::min(gl, grid_for(htotal, kTB)), kTB, 0, s>>>(htotal, sc.key[which], sc.val[which], hub_c, hoff, hs,
                                                                       boff, tadj, tw);
-        k_hub_rowcnt<<<grid_for(nhub, kTB, 1024), kTB, 0, s>>>(nhub, htotal, hub_c, hoff, hs, totp + 4, cnt);
-        c.launches += 5;
+        k_hub_rowcnt<<<grid_for(nhub, kTB, 1024), kTB, 0, s>>>(nhub, htotal, hub_c, hoff, hs, hub_total, cnt);
+        c.launches += 3 + 2 * scan_launches(nc) + scan_launches(htotal);
+        JET_CUDA_TRY(cudaGetLastError());
     }
-    JET_CUDA_TRY(cudaGetLastError());
     // coarse xadj
-    DevBuf xcb, exb;
-    JET_TRY(dev_alloc(xcb, (size_t)(nc + 1) * 8, s));
-    JET_TRY(dev_alloc(exb, (size_t)std::max<int64_t>(nc, 1) * 8, s));
-    c.launches += 3;
-    JET_TRY(device_exscan(CountVal{cntb.as<int32_t>()}, nc, exb.as<int64_t>(), totp + 2, scan_scr.as<int64_t>(), s));
-    JET_CUDA_TRY(launch_pdl(k_finish_xadj, grid_for(nc + 1, kTB, 8192), kTB, 0, s, true, (int32_t)nc,
-                            (const int64_t *)exb.as<int64_t>(), (const int64_t *)(totp + 2), xcb.as<int64_t>()));
-    c.launches += 1;
-    JET_CUDA_TRY(cudaMemcpyAsync(c.pinned, totp + 2, 8, cudaMemcpyDeviceToHost, s));
+    JET_TRY(device_exscan(CountVal{cnt}, nc, xc, xc + nc, scan_scr, s));
+    c.launches += scan_launches(nc);
+    JET_CUDA_TRY(cudaMemcpyAsync(c.pinned, xc + nc, 8, cudaMemcpyDeviceToHost, s));
     JET_CUDA_TRY(cudaStreamSynchronize(s));
-    int64_t nnzc = c.pinned[0];
-    DevBuf adjcb, ewcb;
-    JET_TRY(dev_alloc(adjcb, (size_t)std::max<int64_t>(nnzc, 1) * 4, s));
-    JET_TRY(dev_alloc(ewcb, (size_t)std::max<int64_t>(nnzc, 1) * 4, s));
-    JET_CUDA_TRY(launch_pdl(k_copy_long, glarge, kTB, 0, s, true, (const int32_t *)large_list, (const int32_t *)counts,
-                            (const int64_t *)boff, (const int64_t *)xcb.as<int64_t>(), (const int32_t *)tadjb.as<int32_t>(),
-                            (const int32_t *)twb.as<int32_t>(), adjcb.as<int32_t>(), ewcb.as<int32_t>()));
+    const int64_t nnzc = c.pinned[0];
+    const size_t ab = a256((size_t)std::max<int64_t>(nnzc, 1) * 4);
+    JET_TRY(dev_alloc(eb, 2 * ab, s));
+    int32_t *adj_c = eb.as<int32_t>(), *ew_c = reinterpret_cast<int32_t *>(eb.as<char>() + ab);
+    if (hc.rows[1] > 0) {
+        JET_CUDA_TRY(launch_pdl(k_copy_long, glarge, kTB, 0, s, true, (const int32_t *)large_list, cts, bo, (const int64_t *)xc,
+                                (const int32_t *)tadj, (const int32_t *)tw, adj_c, ew_c));
+        c.launches += 1;
+    }
+    JET_CUDA_TRY(launch_pdl(k_copy_rows, std::min(gl, grid_for(nc, kTB / kCopyLanes)), kTB, 0, s, true, (int32_t)nc, bo,
+                            (const int64_t *)xc, cr, mt, g.vw, vwc, (const int32_t *)tadj, (const int32_t *)tw, adj_c, ew_c));
     c.launches += 1;
-    JET_CUDA_TRY(launch_pdl(k_copy_rows, std::min(gl, grid_for(nc, kTB / kCopyLanes)), kTB, 0, s, true, (int32_t)nc,
-                            (const int64_t *)boff, (const int64_t *)totp, (const int64_t *)xcb.as<int64_t>(),
-                            (const int32_t *)tadjb.as<int32_t>(), (const int32_t *)twb.as<int32_t>(), adjcb.as<int32_t>(),
-                            ewcb.as<int32_t>()));
     JET_CUDA_TRY(cudaGetLastError());
     int32_t i = h->levels;
     h->cmap[i - 1] = cmap;
     h->n[i] = (int32_t)nc;
     h->nnz[i] = nnzc;
-    h->xadj[i] = xcb.as<int64_t>();
-    h->adj[i] = adjcb.as<int32_t>();
-    h->vw[i] = vwcb.as<int32_t>();
-    h->ew[i] = ewcb.as<int32_t>();
+    h->xadj[i] = xc;
+    h->adj[i] = adj_c;
+    h->vw[i] = vwc;
+    h->ew[i] = ew_c;
     h->levels = i + 1;
     h->bufs.push_back(std::move(cmapb));
-    h->bufs.push_back(std::move(xcb));
-    h->bufs.push_back(std::move(adjcb));
-    h->bufs.push_back(std::move(vwcb));
-    h->bufs.push_back(std::move(ewcb));
+    h->bufs.push_back(std::move(vb));
+    h->bufs.push_back(std::move(eb));
     return JET_OK;   // the next level's work follows in stream order
 }
 

@@ -496,7 +496,7 @@ int initial_partition(Ctx &c, const DGraph &g, int32_t k, int32_t *part, GreedyO
 
     // 4. weights before each vertex in that order, then P
     JET_TRY(device_exscan(SortedWeight{order, g.vw}, n, S, &ctl->total, scan_scr, s));
-    c.launches += 3;
+    c.launches += scan_launches(n);
     if (part) {
         k_assign<<<gv, kTB, 0, s>>>((int32_t)n, order, S, ctl, k, part);
         c.launches += 1;

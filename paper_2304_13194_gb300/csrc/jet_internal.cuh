@@ -2,6 +2,7 @@
 // Nothing here is part of the C ABI (include/jet.h).
 #pragma once
 
+#include <algorithm>
 #include <cuda_runtime.h>
 #include <cstdint>
 #include <cstddef>
@@ -398,13 +399,11 @@ inline int grid_for(int64_t items, int per_block, int cap = 1 << 30) {
 int num_sms();
 
 // ---------------------------------------------------------------------------
-// device-wide exclusive scan (3 phases: tile sums, scan of tile sums, tiles)
+// device-wide exclusive scan (tile sums, then every tile with the sums before it)
 // ---------------------------------------------------------------------------
 // out[i] = sum_{j<i} f(j) for i in [0, n); *total_dev = sum (device int64).
 // Functor F: __device__ int64_t operator()(int64_t i) const.
-template <class F> __global__ void k_scan_tiles(F f, int64_t n, int64_t *tile_sums);
-template <class F> __global__ void k_scan_apply(F f, int64_t n, const int64_t *tile_off, int64_t *out);
-__global__ void k_scan_sums(int64_t *tile_sums, int64_t ntiles, int64_t *total_dev);
+__global__ void k_scan_sums(int64_t *tile_sums, int64_t ntiles);
 
 constexpr int kScanItems = 8;
 constexpr int kScanTile = kTB * kScanItems;
@@ -424,11 +423,16 @@ __global__ void __launch_bounds__(kTB) k_scan_tiles(F f, int64_t n, int64_t *til
     if (threadIdx.x == 0) tile_sums[blockIdx.x] = s;
 }
 
-template <class F>
-__global__ void __launch_bounds__(kTB) k_scan_apply(F f, int64_t n, const int64_t *tile_off, int64_t *out) {
+// tile[b]: the sum of tile b, or with SCANNED of the tiles before it.
+template <bool SCANNED, class F>
+__global__ void __launch_bounds__(kTB) k_scan_apply(F f, int64_t n, const int64_t *tile, int64_t *out, int64_t *total_dev) {
     __shared__ long long sh[40];
     pdl_enter();
     int64_t base = (int64_t)blockIdx.x * kScanTile;
+    long long before = 0;
+    if (SCANNED) before = tile[blockIdx.x];
+    else
+        for (int64_t t = threadIdx.x; t < blockIdx.x; t += kTB) before += tile[t];
     long long vals[kScanItems];
     long long s = 0;
 #pragma unroll
@@ -437,7 +441,10 @@ __global__ void __launch_bounds__(kTB) k_scan_apply(F f, int64_t n, const int64_
         vals[i] = idx < n ? f(idx) : 0;
         s += vals[i];
     }
-    long long off = block_exscan_i64(s, sh, nullptr) + tile_off[blockIdx.x];
+    if (!SCANNED && blockIdx.x > 0) before = block_sum_i64(before, sh);
+    long long total = 0;
+    long long off = block_exscan_i64(s, sh, &total) + before;
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0 && total_dev) *total_dev = before + total;
 #pragma unroll
     for (int i = 0; i < kScanItems; ++i) {
         int64_t idx = base + (int64_t)threadIdx.x * kScanItems + i;
@@ -449,16 +456,27 @@ __global__ void __launch_bounds__(kTB) k_scan_apply(F f, int64_t n, const int64_
 // Scratch for a scan of n items: (ntiles) int64.
 inline int64_t scan_tiles_for(int64_t n) { return (n + kScanTile - 1) / kScanTile; }
 
+// Up to kScanDirect tiles (2 M items) every tile adds up the sums before it by
+// itself (four loads a thread at most) and one tile needs no sums: one or two
+// launches; a separate scan of the sums, a third, is for longer ones.
+constexpr int64_t kScanDirect = 1024;
+
 template <class F>
 int device_exscan(F f, int64_t n, int64_t *out, int64_t *total_dev, int64_t *tile_scratch, cudaStream_t s) {
-    int64_t nt = scan_tiles_for(n);
-    if (nt < 1) nt = 1;
-    // the three kernels (and the next one) follow by programmatic launch
-    JET_CUDA_TRY(launch_pdl(k_scan_tiles<F>, (int)nt, kTB, 0, s, true, f, n, tile_scratch));
-    JET_CUDA_TRY(launch_pdl(k_scan_sums, 1, 1024, 0, s, true, tile_scratch, nt, total_dev));
-    JET_CUDA_TRY(launch_pdl(k_scan_apply<F>, (int)nt, kTB, 0, s, true, f, n, (const int64_t *)tile_scratch, out));
+    const int64_t nt = std::max<int64_t>(scan_tiles_for(n), 1);
+    // the kernels (and the next one) follow by programmatic launch
+    if (nt > 1) JET_CUDA_TRY(launch_pdl(k_scan_tiles<F>, (int)nt, kTB, 0, s, true, f, n, tile_scratch));
+    if (nt > kScanDirect) {
+        JET_CUDA_TRY(launch_pdl(k_scan_sums, 1, 1024, 0, s, true, tile_scratch, nt));
+        JET_CUDA_TRY(launch_pdl(k_scan_apply<true, F>, (int)nt, kTB, 0, s, true, f, n, (const int64_t *)tile_scratch, out, total_dev));
+    } else {
+        JET_CUDA_TRY(launch_pdl(k_scan_apply<false, F>, (int)nt, kTB, 0, s, true, f, n, (const int64_t *)tile_scratch, out, total_dev));
+    }
     return JET_OK;
 }
+
+// Launches of device_exscan over n items (for the launch counter).
+inline int scan_launches(int64_t n) { return scan_tiles_for(n) <= 1 ? 1 : scan_tiles_for(n) <= kScanDirect ? 2 : 3; }
 
 // ---------------------------------------------------------------------------
 // context

@@ -130,7 +130,7 @@ int sort_pairs(Ctx &c, SortScratch &sc, int64_t n, int kbits, int *which) {
         JET_TRY(device_exscan(HistVal{sc.hist}, nhist, sc.off, sc.total, sc.scan, s));
         k_sort_scatter<<<(unsigned)ntiles, kTB, 0, s>>>(sc.key[cur], sc.val[cur], sc.key[cur ^ 1], sc.val[cur ^ 1], n, shift,
                                                         ntiles, sc.off);
-        c.launches += 5;
+        c.launches += 2 + scan_launches(nhist);
         JET_CUDA_TRY(cudaGetLastError());
         cur ^= 1;
     }

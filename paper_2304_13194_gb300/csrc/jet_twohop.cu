@@ -158,7 +158,7 @@ int two_hop(Ctx &c, const DGraph &g, int32_t *mate, int64_t added[3]) {
         JET_TRY(device_exscan(GroupHead{key, sentinel}, n, hb, cnt + 1, scan_scr, s));
         k_group_starts<<<gv, kTB, 0, s>>>(n, key, sentinel, hb, start);
         k_pair_groups<<<gv, kTB, 0, s>>>(n, key, val, sentinel, hb, start, mate);
-        c.launches += 5;
+        c.launches += 2 + scan_launches(n);
         JET_CUDA_TRY(cudaGetLastError());
         int64_t un2 = 0;
         JET_TRY(unmatched(un2));

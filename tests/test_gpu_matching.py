@@ -24,11 +24,14 @@ def ctx():
     c.close()
 
 
-def _stars(*leaves):
-    """A chain of hubs with the given numbers of leaves."""
+def _stars(*leaves, pairs=False):
+    """A chain of hubs with the given numbers of leaves; with pairs, neighbouring
+    leaves share a heavier edge, so that they match and the hubs' rows shrink."""
     t, hub = [], 0
     for i, m in enumerate(leaves):
         t += [[hub, hub + 1 + j, 1 + (j * 7) % 5] for j in range(m)]
+        if pairs:
+            t += [[hub + 1 + j, hub + 2 + j, 9] for j in range(0, m - 1, 2)]
         if i + 1 < len(leaves):
             t.append([hub, hub + m + 1, 3])
         hub += m + 1
@@ -60,3 +63,36 @@ def test_matching_equals_oracle(ctx, name, make):
             gw = g if weights is not None else graphgen.Graph(g.n, g.xadj, g.adjncy, g.vwgt, np.ones_like(g.adjncy))
             got = ctx.hem(d[0], d[1], weights, seed=11, level=level, rounds=rounds).cpu().numpy()
             assert np.array_equal(got, oracle.hem(gw, 11, level, rounds)), (weights is None, level, rounds)
+
+
+HIERARCHIES = [
+    ("path2048", lambda: graphgen.grid2d(2048, 1), 2),              # one scan tile
+    ("path2049", lambda: graphgen.grid2d(2049, 1), 2),              # two
+    ("path_scan_limit", lambda: graphgen.grid2d(2097152, 1), 512),  # 1,024 tiles: every tile adds up its own offset
+    ("path_scan_over", lambda: graphgen.grid2d(2097153, 1), 512),   # 1,025: a scan of the sums
+    ("no_match", lambda: graphgen.Graph(3000, np.zeros(3001, np.int64), np.zeros(0, np.int32), np.ones(3000, np.int32),
+                                        np.zeros(0, np.int32)), 2),
+    # merged rows around the thread, warp and block classes, the last one past the largest block row
+    ("row_classes", lambda: _stars(*range(10, 20), *range(27, 35), *range(250, 260), *range(510, 514),
+                                    *range(4088, 4100), 6000, pairs=True), 2),
+    ("dense", lambda: graphgen.gnp(700, 0.9, seed=6, ew=(1, 9)), 2),
+]
+
+
+@pytest.mark.parametrize("name,make,k", HIERARCHIES, ids=[c[0] for c in HIERARCHIES])
+def test_hierarchy_equals_oracle(ctx, name, make, k):
+    g = make()
+    ref = oracle.coarsen(g, k, seed=5)
+    d = [torch.as_tensor(np.asarray(a)).cuda() for a in (g.xadj, g.adjncy, g.vwgt, g.adjwgt)]
+    h = ctx.coarsen(*d, k=k, seed=5)
+    try:
+        assert h.info()[0] == len(ref)
+        for i in range(len(ref)):
+            L, R = h.level(i), ref[i].graph
+            assert L["n"] == R.n
+            for key, want in (("xadj", R.xadj), ("adjncy", R.adjncy), ("vwgt", R.vwgt), ("adjwgt", R.adjwgt)):
+                assert np.array_equal(np.asarray(L[key].cpu()), want), (i, key)
+            if i + 1 < len(ref):
+                assert np.array_equal(np.asarray(L["cmap"].cpu()), ref[i].cmap), i
+    finally:
+        h.close()
