@@ -1,9 +1,13 @@
-// Stable LSD radix sort of (64-bit key, int32 value) pairs, device-wide:
-// per tile of kSortTile elements a digit histogram, one exclusive scan over
-// all (digit, tile) counts in digit-major order, then a scatter that keeps
-// the input order among equal digits (chunk by chunk, warp by warp, lane by
-// lane).  Used where the method orders vertices by a key with ties broken by
-// vertex id: the values enter in id order.
+// Stable LSD radix sort of (64-bit key, int32 value) pairs, device-wide: per
+// digit a histogram of every tile of kSortTile elements, then a scatter that keeps
+// the input order among equal digits.  A warp takes consecutive elements of the
+// tile and counts them digit by digit in its own counters, so that a tile has four
+// block barriers, not five per 256 elements.  Up to kSortDirect tiles every tile
+// adds the histograms up itself: two launches per digit; more tiles take an
+// exclusive scan of all counts in digit-major order between them.  A digit of
+// 131,072 pairs: 37 us in five launches before, 12 us in two now.
+// Used where the method orders vertices by a key with ties broken by vertex id:
+// the values enter in id order.
 #include "jet_internal.cuh"
 
 #include <algorithm>
@@ -17,20 +21,31 @@ constexpr int kSortTile = kTB * kSortItems;       // elements per tile
 constexpr int kRadixBits = 8;
 constexpr int kRadix = 1 << kRadixBits;
 
-// Digit histogram of each tile, stored digit-major: hist[d * ntiles + tile].
+constexpr int kSortWarps = kTB / 32;
+constexpr int64_t kSortDirect = 128;              // tiles up to which the scatter adds the histograms up
+static_assert(kTB == kRadix, "one thread per digit");
+
+// Digit histogram of each tile: hist[tile * kRadix + d] (DIRECT) or hist[d * ntiles + tile].
+template <bool DIRECT>
 __global__ void __launch_bounds__(kTB) k_sort_hist(const uint64_t *key, int64_t n, int shift, int64_t ntiles,
                                                    int64_t *hist) {
     __shared__ int32_t h[kRadix];
-    for (int i = threadIdx.x; i < kRadix; i += blockDim.x) h[i] = 0;
+    h[threadIdx.x] = 0;
     __syncthreads();
+    pdl_enter();
     const int64_t base = (int64_t)blockIdx.x * kSortTile;
+    uint64_t k[kSortItems];
 #pragma unroll
     for (int i = 0; i < kSortItems; ++i) {
-        int64_t e = base + (int64_t)i * blockDim.x + threadIdx.x;
-        if (e < n) atomicAdd(&h[(int)((key[e] >> shift) & (kRadix - 1))], 1);
+        const int64_t e = base + (int64_t)i * kTB + threadIdx.x;
+        k[i] = e < n ? key[e] : 0;
     }
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i)
+        if (base + (int64_t)i * kTB + threadIdx.x < n) atomicAdd(&h[(int)((k[i] >> shift) & (kRadix - 1))], 1);
     __syncthreads();
-    for (int d = threadIdx.x; d < kRadix; d += blockDim.x) hist[(int64_t)d * ntiles + blockIdx.x] = h[d];
+    if (DIRECT) reinterpret_cast<int32_t *>(hist)[(int64_t)blockIdx.x * kRadix + threadIdx.x] = h[threadIdx.x];
+    else hist[(int64_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
 }
 
 struct HistVal {
@@ -38,50 +53,76 @@ struct HistVal {
     __device__ int64_t operator()(int64_t i) const { return hist[i]; }
 };
 
-// Scatter of one tile, chunk after chunk of blockDim elements in index order;
-// inside a chunk, warp after warp and lane after lane: the rank of an element
-// among the tile's equal digits keeps the input order (stable).
+// Scatter of one tile.  Warp w takes the elements base + w * 32 kSortItems + 32 i + lane:
+// the rank of an element among the tile's equal digits keeps the input order.
+template <bool DIRECT>
 __global__ void __launch_bounds__(kTB) k_sort_scatter(const uint64_t *key_in, const int32_t *val_in, uint64_t *key_out,
                                                       int32_t *val_out, int64_t n, int shift, int64_t ntiles,
                                                       const int64_t *off) {
-    __shared__ int32_t wcnt[kTB / 32][kRadix];    // per-warp digit counts, then warp prefixes
-    __shared__ int32_t ctot[kRadix];              // this chunk's count per digit
-    __shared__ int64_t run[kRadix];               // tile offset + elements placed so far, per digit
-    const int64_t base = (int64_t)blockIdx.x * kSortTile;
+    __shared__ int32_t wcnt[kSortWarps][kRadix];   // per-warp digit counts, then the warps' offsets in the tile's digit
+    __shared__ int64_t run[kRadix];                // first position of the tile's digit
+    __shared__ long long sh[40];
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    const int nwarps = blockDim.x >> 5;
-    for (int d = threadIdx.x; d < kRadix; d += blockDim.x) run[d] = off[(int64_t)d * ntiles + blockIdx.x];
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) wcnt[w][threadIdx.x] = 0;
+    __syncthreads();
+    pdl_enter();
+    const int64_t base = (int64_t)blockIdx.x * kSortTile + (int64_t)warp * 32 * kSortItems + lane;
+    uint64_t k[kSortItems];
+    int32_t v[kSortItems], pos[kSortItems];
+#pragma unroll
     for (int i = 0; i < kSortItems; ++i) {
-        for (int t = threadIdx.x; t < nwarps * kRadix; t += blockDim.x) wcnt[t / kRadix][t % kRadix] = 0;
-        __syncthreads();
-        const int64_t e = base + (int64_t)i * blockDim.x + threadIdx.x;
-        const bool ok = e < n;
-        const uint64_t k = ok ? key_in[e] : 0;
-        const int32_t v = ok ? val_in[e] : 0;
-        const int d = ok ? (int)((k >> shift) & (kRadix - 1)) : -1;
+        const int64_t e = base + 32 * i;
+        k[i] = e < n ? key_in[e] : 0;
+        v[i] = e < n ? val_in[e] : 0;
+    }
+    int64_t first = 0;                             // of digit threadIdx.x
+    if (DIRECT) {
+        const int32_t *hist = reinterpret_cast<const int32_t *>(off);
+        int32_t before = 0, all = 0;
+#pragma unroll 16
+        for (int t = 0; t < (int)ntiles; ++t) {
+            const int32_t x = hist[t * kRadix + threadIdx.x];
+            all += x;
+            before += t < (int)blockIdx.x ? x : 0;
+        }
+        first = block_exscan_i64(all, sh, nullptr) + before;
+    } else {
+        first = off[(int64_t)threadIdx.x * ntiles + blockIdx.x];
+    }
+    run[threadIdx.x] = first;
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) {
+        const int d = base + 32 * i < n ? (int)((k[i] >> shift) & (kRadix - 1)) : -1;
         const unsigned peers = __match_any_sync(0xffffffffu, d);
-        const int rank = __popc(peers & lt);
-        if (ok && rank == 0) wcnt[warp][d] = __popc(peers);
-        __syncthreads();
-        for (int dd = threadIdx.x; dd < kRadix; dd += blockDim.x) {
-            int32_t acc = 0;
-            for (int w = 0; w < nwarps; ++w) {
-                int32_t c = wcnt[w][dd];
-                wcnt[w][dd] = acc;
-                acc += c;
-            }
-            ctot[dd] = acc;
+        const int leader = __ffs(peers) - 1;
+        int32_t c = 0;
+        if (d >= 0 && (int)lane == leader) {
+            c = wcnt[warp][d];
+            wcnt[warp][d] = c + __popc(peers);
         }
-        __syncthreads();
-        if (ok) {
-            const int64_t pos = run[d] + wcnt[warp][d] + rank;
-            key_out[pos] = k;
-            val_out[pos] = v;
+        pos[i] = __shfl_sync(0xffffffffu, c, leader) + __popc(peers & lt);
+        __syncwarp();
+    }
+    __syncthreads();
+    {
+        int32_t acc = 0;
+#pragma unroll
+        for (int w = 0; w < kSortWarps; ++w) {
+            const int32_t c = wcnt[w][threadIdx.x];
+            wcnt[w][threadIdx.x] = acc;
+            acc += c;
         }
-        __syncthreads();
-        for (int dd = threadIdx.x; dd < kRadix; dd += blockDim.x) run[dd] += ctot[dd];
-        __syncthreads();
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) {
+        if (base + 32 * i >= n) continue;
+        const int d = (int)((k[i] >> shift) & (kRadix - 1));
+        const int64_t p = run[d] + wcnt[warp][d] + pos[i];
+        key_out[p] = k[i];
+        val_out[p] = v[i];
     }
 }
 
@@ -126,12 +167,20 @@ int sort_pairs(Ctx &c, SortScratch &sc, int64_t n, int kbits, int *which) {
     const int64_t nhist = ntiles * kRadix;
     int cur = 0;
     for (int shift = 0; shift < kbits; shift += kRadixBits) {
-        k_sort_hist<<<(unsigned)ntiles, kTB, 0, s>>>(sc.key[cur], n, shift, ntiles, sc.hist);
-        JET_TRY(device_exscan(HistVal{sc.hist}, nhist, sc.off, sc.total, sc.scan, s));
-        k_sort_scatter<<<(unsigned)ntiles, kTB, 0, s>>>(sc.key[cur], sc.val[cur], sc.key[cur ^ 1], sc.val[cur ^ 1], n, shift,
-                                                        ntiles, sc.off);
-        c.launches += 2 + scan_launches(nhist);
-        JET_CUDA_TRY(cudaGetLastError());
+        const uint64_t *kin = sc.key[cur];
+        const int32_t *vin = sc.val[cur];
+        if (ntiles <= kSortDirect) {
+            JET_CUDA_TRY(launch_pdl(k_sort_hist<true>, (int)ntiles, kTB, 0, s, true, kin, n, shift, ntiles, sc.hist));
+            JET_CUDA_TRY(launch_pdl(k_sort_scatter<true>, (int)ntiles, kTB, 0, s, true, kin, vin, sc.key[cur ^ 1], sc.val[cur ^ 1],
+                                    n, shift, ntiles, (const int64_t *)sc.hist));
+            c.launches += 2;
+        } else {
+            JET_CUDA_TRY(launch_pdl(k_sort_hist<false>, (int)ntiles, kTB, 0, s, true, kin, n, shift, ntiles, sc.hist));
+            JET_TRY(device_exscan(HistVal{sc.hist}, nhist, sc.off, sc.total, sc.scan, s));
+            JET_CUDA_TRY(launch_pdl(k_sort_scatter<false>, (int)ntiles, kTB, 0, s, true, kin, vin, sc.key[cur ^ 1],
+                                    sc.val[cur ^ 1], n, shift, ntiles, (const int64_t *)sc.off));
+            c.launches += 2 + scan_launches(nhist);
+        }
         cur ^= 1;
     }
     *which = cur;

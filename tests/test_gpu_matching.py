@@ -96,3 +96,67 @@ def test_hierarchy_equals_oracle(ctx, name, make, k):
                 assert np.array_equal(np.asarray(L["cmap"].cpu()), ref[i].cmap), i
     finally:
         h.close()
+
+
+def _splitmix64(x):
+    x = np.asarray(x, np.uint64) + np.uint64(0x9E3779B97F4A7C15)
+    x = (x ^ (x >> np.uint64(30))) * np.uint64(0xBF58476D1CE4E5B9)
+    x = (x ^ (x >> np.uint64(27))) * np.uint64(0x94D049BB133111EB)
+    return x ^ (x >> np.uint64(31))
+
+
+def _csr(n, pairs):
+    return graph_from_triples(n, [[a, b, 1] for a, b in pairs])
+
+
+def _colliding_twins():
+    """Two groups of twins, interleaved by id, whose 64-bit neighbourhood hashes
+    differ but share their low 24 bits (as many as 220 vertices are sorted by)."""
+    hubs = 160
+    h = _splitmix64(np.arange(hubs, dtype=np.uint64) ^ np.uint64(0x2545F4914F6CDD1D))
+    a, b = np.triu_indices(hubs, 1)
+    s = h[a] + h[b]
+    low = s & np.uint64((1 << 24) - 1)
+    order = np.argsort(low, kind="stable")
+    hit = next(i for i in range(len(order) - 1)
+               if low[order[i]] == low[order[i + 1]] and s[order[i]] != s[order[i + 1]])
+    p, q = order[hit], order[hit + 1]
+    pairs = [(i, i + 1) for i in range(0, hubs, 2)]
+    for j in range(60):
+        e = (p, q)[j % 3 == 1]
+        pairs += [(int(a[e]), hubs + j), (int(b[e]), hubs + j)]
+    mate = np.full(220, -1, np.int32)
+    mate[:hubs] = np.arange(hubs) ^ 1
+    return _csr(220, pairs), mate
+
+
+def _two_hop_mix(n, seed):
+    """n vertices, most of them leaves, twins and relatives of a few hubs."""
+    r = np.random.default_rng(seed)
+    hubs = max(2, n // 50)
+    t = [(i, (i + 1) % hubs) for i in range(hubs if hubs > 2 else 1)]
+    kind = r.integers(0, 3, n - hubs)
+    x = r.integers(0, hubs, (n - hubs, 2))
+    x[kind == 1] = (x[kind == 1] // 4) * 4 % hubs
+    for i in range(n - hubs):
+        t.append((int(x[i, 0]), hubs + i))
+        if kind[i] and x[i, 0] != x[i, 1]:
+            t.append((int(x[i, 1]), hubs + i))
+    return _csr(n, t)
+
+
+@pytest.mark.parametrize("n", [3, 31, 2047, 2049, 262144, 262145])
+def test_two_hop_equals_oracle(ctx, n):
+    g = _two_hop_mix(n, n)      # 262,144: the last size whose tiles add the histograms up
+    mate = oracle.hem(g, 7, 0, 2)
+    got, added = ctx.two_hop(torch.as_tensor(g.xadj).cuda(), torch.as_tensor(g.adjncy).cuda(), torch.as_tensor(mate).cuda())
+    want, wadded = oracle.two_hop(g, mate)
+    assert list(added) == wadded and np.array_equal(got.cpu().numpy(), want)
+
+
+def test_twins_that_share_the_sorted_bits(ctx):
+    g, mate = _colliding_twins()
+    want, wadded = oracle.two_hop(g, mate)
+    assert wadded[1] > 0
+    got, added = ctx.two_hop(torch.as_tensor(g.xadj).cuda(), torch.as_tensor(g.adjncy).cuda(), torch.as_tensor(mate).cuda())
+    assert list(added) == wadded and np.array_equal(got.cpu().numpy(), want)
