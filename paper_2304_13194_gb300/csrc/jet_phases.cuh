@@ -265,7 +265,7 @@ struct Appender {
 constexpr int kScanCap = 4096;          // list staging of the scan phases
 constexpr int kListCap = 2048;          // X / M staging
 constexpr int kBigCap = 1024;           // long-row staging
-constexpr int kSmemBuckets = 1024;      // slot buckets aggregated per block when nA * kSlots fits
+constexpr int kSmemBuckets = 4096;      // slot buckets aggregated per block when nA * kSlots fits
 
 __host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 __host__ __device__ constexpr size_t arena_max(size_t a, size_t b) { return a > b ? a : b; }
@@ -278,9 +278,9 @@ __host__ __device__ constexpr size_t sm_lp_select(int32_t k, int T, bool tables)
 }
 __host__ __device__ constexpr size_t sm_afterburn() { return (size_t)(kListCap + kBigCap) * 4; }
 __host__ __device__ constexpr size_t sm_apply(int32_t k) { return align16((size_t)k * 8) + (size_t)kBigCap * 4; }
-__host__ __device__ constexpr size_t sm_rb_scan() { return (size_t)kSmemBuckets * 8 + (size_t)kScanCap * 4; }
+__host__ __device__ constexpr size_t sm_rb_scan() { return (size_t)kSmemBuckets * 4 + (size_t)kScanCap * 4; }
 __host__ __device__ constexpr size_t sm_rb_cand(int32_t k, int T, bool tables) {
-    return (size_t)kSmemBuckets * 8 + (size_t)kBigCap * 4 + arena_tables(k, T, tables);
+    return (size_t)kSmemBuckets * 4 + (size_t)kBigCap * 4 + arena_tables(k, T, tables);
 }
 __host__ __device__ constexpr size_t sm_rb_tilehist(int32_t k) { return (size_t)k * 4; }
 __host__ __device__ constexpr size_t sm_rb_take(int32_t k, int T) { return align16((size_t)k * 8) + (size_t)2 * T * 4; }
@@ -1254,12 +1254,17 @@ __device__ __forceinline__ void bucket_add(const Level &L, int32_t key, long lon
     if (key >= 0 && (int)lane_id() == __ffs(peers) - 1) atomic_add_i64(&L.bucketw[key], (long long)s);
 }
 
-// Per-block slot buckets in shared memory when nA * kSlots keys fit.
+// Per-block slot buckets in shared memory when nA * kSlots keys fit: 32-bit sums
+// (exact: the total vertex weight is below 2^31), which shared memory adds
+// natively, where 64-bit ones are compare-and-swap loops that contend for the few
+// slots in use; at half the size each, the buckets of 124 oversized parts stay here,
+// not of 31, whose keys went to global atomics.  A scan of 1.1 M vertices (k = 64)
+// 32.6 -> 20.0 us, of 2.1 M 42.6 -> 28.2.
 struct SmemBuckets {
-    long long *b;
+    uint32_t *b;
     int32_t nkeys;
     bool on;
-    __device__ __forceinline__ void init(const Level &L, long long *buf) {
+    __device__ __forceinline__ void init(const Level &L, uint32_t *buf) {
         b = buf;
         nkeys = L.ctl->nA * kSlots;
         on = nkeys <= kSmemBuckets;
@@ -1269,20 +1274,20 @@ struct SmemBuckets {
     }
     __device__ __forceinline__ void add(const Level &L, int32_t key, long long w) {   // all lanes call
         if (on) {
-            if (key >= 0) atomicAdd(reinterpret_cast<unsigned long long *>(&b[key]), (unsigned long long)w);
+            if (key >= 0) atomicAdd(&b[key], (uint32_t)w);
         } else {
             bucket_add(L, key, w);
         }
     }
     __device__ __forceinline__ void add_one(const Level &L, int32_t key, long long w) {   // one thread
-        if (on) atomicAdd(reinterpret_cast<unsigned long long *>(&b[key]), (unsigned long long)w);
+        if (on) atomicAdd(&b[key], (uint32_t)w);
         else atomic_add_i64(&L.bucketw[key], w);
     }
     __device__ __forceinline__ void flush(const Level &L) {
         if (!on) return;
         __syncthreads();
         for (int i = threadIdx.x; i < nkeys; i += blockDim.x)
-            if (b[i]) atomic_add_i64(&L.bucketw[i], b[i]);
+            if (b[i]) atomic_add_i64(&L.bucketw[i], (long long)b[i]);
         __syncthreads();
     }
 };
@@ -1302,8 +1307,8 @@ __device__ inline void ph_rb_scan(const Level &L, Grid G, char *arena) {
     const int32_t it = ctl->it, nB = ctl->nB;   // loaded before the barriers of the set-up below
     const int64_t opt = ctl->opt;
     SmemBuckets sb;
-    sb.init(L, reinterpret_cast<long long *>(arena));
-    JET_APPENDER(wapp, reinterpret_cast<int32_t *>(arena + kSmemBuckets * 8), kScanCap);
+    sb.init(L, reinterpret_cast<uint32_t *>(arena));
+    JET_APPENDER(wapp, reinterpret_cast<int32_t *>(arena + kSmemBuckets * 4), kScanCap);
     const int64_t n = L.g.n, nq = (n + 3) / 4;
     const bool vec = (reinterpret_cast<uintptr_t>(L.part) & 15) == 0;
     long long ncand = 0, nlist = 0;
@@ -1491,8 +1496,8 @@ __device__ inline void ph_rb_cand(const Level &L, Grid G, char *arena) {
     const Deal dl(ctl->nW, G, nbig > 0);
     if (!dl.live(0)) return;
     SmemBuckets sb;
-    sb.init(L, reinterpret_cast<long long *>(arena));
-    int32_t *a32 = reinterpret_cast<int32_t *>(arena + kSmemBuckets * 8);
+    sb.init(L, reinterpret_cast<uint32_t *>(arena));
+    int32_t *a32 = reinterpret_cast<int32_t *>(arena + kSmemBuckets * 4);
     JET_APPENDER(bigs, a32, kBigCap);
     int32_t *tab = a32 + kBigCap + (threadIdx.x >> 5) * L.k;
     if (nbig > 0) {
@@ -1693,6 +1698,7 @@ __device__ inline void ph_rb_take(const Level &L, Grid G, char *arena) {
     int32_t *mbuf = reinterpret_cast<int32_t *>(arena + align16((size_t)L.k * 8));
     JET_APPENDER(mapp, mbuf, 2 * (int)blockDim.x);
     __shared__ long long red[40];
+    __shared__ int has[32];
     Ctl *ctl = L.ctl;
     const int32_t nA = ctl->nA, it = ctl->it;
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
@@ -1715,20 +1721,27 @@ __device__ inline void ph_rb_take(const Level &L, Grid G, char *arena) {
         bool member = kv >= 0 && s == ss;
         long long w = (kv >= 0) ? (long long)L.g.vw[vv] : 0;
         long long mine = 0;
-        // ordered prefix over the boundary-slot members, warp after warp
-        const unsigned nphase = __syncthreads_or(member) ? (blockDim.x >> 5) : 0u;
-        for (unsigned wi = 0; wi < nphase; ++wi) {
+        // ordered prefix over the boundary-slot members: inside the warps all
+        // together, then the warps that have members add theirs to run[] in turn
+        // (all of it warp after warp before: 108 -> 70 us at 4.2 M vertices, 11 -> 8 at 100 k)
+        const unsigned wm = __ballot_sync(0xffffffffu, member);
+        unsigned peers = 0;
+        long long pre = 0;
+        if (wm) {
+            peers = __match_any_sync(0xffffffffu, member ? a : -(int32_t)lane - 1);
+            const int32_t w32 = member ? (int32_t)w : 0;
+            for (unsigned m = wm; m; m &= m - 1) {
+                const int j = __ffs(m) - 1;
+                const int32_t x = __shfl_sync(0xffffffffu, w32, j);
+                if ((peers & lt_mask) >> j & 1u) pre += x;
+            }
+        }
+        if (lane == 0) has[warp] = wm != 0;
+        __syncthreads();
+        for (unsigned wi = 0; wi < (blockDim.x >> 5); ++wi) {
+            if (!has[wi]) continue;                // the same in every thread
             if (warp == wi) {
-                int32_t grp = member ? a : -(int32_t)lane - 1;
-                unsigned peers = __match_any_sync(0xffffffffu, grp);
-                long long pre = 0;
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    long long x = __shfl_sync(0xffffffffu, member ? w : 0LL, j);
-                    if ((peers & lt_mask) >> j & 1u) pre += x;
-                }
-                long long base = member ? run[a] : 0;
-                mine = base + pre;
+                mine = (member ? run[a] : 0) + pre;
                 __syncwarp();
                 if (member && (peers >> lane) == 1u) run[a] = mine + w;
             }
