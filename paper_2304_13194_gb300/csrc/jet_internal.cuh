@@ -174,7 +174,8 @@ struct Level {
     uint32_t abl;
     uint64_t seed;
     // per-vertex state
-    int32_t *part, *best, *nxt, *prio, *mstamp, *lstamp, *key;
+    int32_t *part, *best, *nxt, *prio, *mstamp, *lstamp, *key;   // mstamp: where move is null (passes that apply nothing)
+    int2 *move;          // {iteration of the vertex's last move, source << 16 | destination}; {-2, part << 16 | part} before it
     int32_t *ext;            // neighbours in other parts (exact, kept by the apply kernel)
     int32_t *wdeg;           // weighted degree (rebalancing of interior vertices)
     int32_t *rbloss;         // rebalancing loss export (single-pass API only; may be null)

@@ -90,6 +90,15 @@ __device__ __forceinline__ int32_t nxt_pack(int32_t from, int32_t to) { return (
 __device__ __forceinline__ int32_t nxt_to(int32_t x) { return x & 0xFFFF; }
 __device__ __forceinline__ int32_t nxt_from(int32_t x) { return (int32_t)((uint32_t)x >> 16); }
 
+// v is in M of iteration `it`; x: its packed move.
+__device__ __forceinline__ void mark_move(const Level &L, int32_t v, int32_t it, int32_t x) {
+    if (L.move) L.move[v] = make_int2(it, x);
+    else L.mstamp[v] = it;
+}
+__device__ __forceinline__ bool is_marked(const Level &L, int64_t v, int32_t it) {
+    return (L.move ? L.move[v].x : L.mstamp[v]) == it;
+}
+
 struct LpExport {           // optional dense outputs of the single-pass API
     int32_t *pd;            // P_d (P_s where undefined)
     int32_t *gain;          // F (kNoneGain where undefined)
@@ -399,7 +408,7 @@ __device__ __forceinline__ void reset_counters(Ctl *ctl) {
 // Algorithmic DRAM bytes of one iteration's refinement kernels, from the
 // counters the iteration gathered: every array a kernel streams is counted
 // once per launch over the subset it touches; gathers and scatters at
-// neighbours (part, prio, nxt, mstamp, ext of u) are taken as cache hits.
+// neighbours (part, prio, nxt, move, ext of u) are taken as cache hits.
 // beta = bytes per CSR entry (8 with edge weights, 4 without), n vertices,
 // k parts, T rebalancing tiles, nA oversized parts; w = rows the Jetlp select
 // reads (unlocked boundary vertices), nb = boundary vertices, c =
@@ -409,7 +418,7 @@ __device__ __forceinline__ void reset_counters(Ctl *ctl) {
 //                                          boundary ones, work-list writes
 //   lp_select    24 w + beta deg(W) + 12|X| list, xadj pair, part; rows; prio, nxt, X list
 //   afterburn    32|X| + beta deg(X) + 8|M|  X list, xadj pair, prio, nxt, part; rows;
-//                                          mstamp, M list (4|X| + 8|M| without afterburner)
+//                                          move, M list (4|X| + 8|M| without afterburner)
 //   apply        36|M| + beta deg(M) + 16k  M list, nxt, vwgt, xadj pair, ext, part
 //                                          (+4|M| lock stamps and 8|X| priority resets
 //                                          after Jetlp); rows; part weights
@@ -418,11 +427,11 @@ __device__ __forceinline__ void reset_counters(Ctl *ctl) {
 //   rb_cand      28r (+4r Jetrw) + beta deg(R)  list, xadj pair, part, key (+ destination); rows
 //   rb_tilehist  4n + 4c + 4 T nA          key, vwgt of candidates, tile sums
 //   rb_tilescan  8 T nA                    tile sums read and written
-//   rb_take      4n + 4c + 4 T nA + 8|M|   key, vwgt, tile offsets; mstamp, M list
+//   rb_take      4n + 4c + 4 T nA + 8|M|   key, vwgt, tile offsets; move, M list
 //                (Jetrs: + 8n + 8T          evicted weight per vertex and per tile,
 //                 instead of the M list)
 //   rb_cookie    8n + 8T + 16|M|           evicted weight, tile offsets; part, nxt,
-//                                          mstamp, M list
+//                                          move, M list
 // plus 8n (read P_iter, write P_best) in the kernel that copied the best
 // partition during this iteration (the afterburner for Jetlp, rb_scan for
 // rebalancing) when the previous controller asked for it; the copy after
@@ -947,7 +956,7 @@ __device__ __forceinline__ void afterburn_block_row(const Level &L, LpExport ex,
     if (threadIdx.x == 0) {
         if (ex.f2) ex.f2[v] = (int32_t)f2;
         if (f2 >= 0) {
-            L.mstamp[v] = it;
+            mark_move(L, v, it, nxt_pack(ps, pd));
             L.listM[L.g.n - 1 - atomicAdd(&L.ctl->nMh, 1)] = v;   // hub region
         }
     }
@@ -965,7 +974,7 @@ __device__ inline void ph_afterburn(const Level &L, LpExport ex, Grid G, char *a
         if (full_ab) {
             afterburn_block_row<EW>(L, ex, v, it, red);
         } else if (threadIdx.x == 0) {
-            L.mstamp[v] = it;
+            mark_move(L, v, it, L.nxt[v]);
             L.listM[L.g.n - 1 - atomicAdd(&ctl->nMh, 1)] = v;
         }
     }
@@ -983,7 +992,7 @@ __device__ inline void ph_afterburn(const Level &L, LpExport ex, Grid G, char *a
         f2 = warp_sum_i32(f2);
         if (lane == 0) {
             if (ex.f2) ex.f2[v] = f2;
-            if (f2 >= 0) L.mstamp[v] = it;
+            if (f2 >= 0) mark_move(L, v, it, nxt_pack(ps, pd));
         }
         mapp.add(lane == 0 && f2 >= 0, v);   // the block's M staging: no global atomic per row
     };
@@ -1025,7 +1034,7 @@ __device__ inline void ph_afterburn(const Level &L, LpExport ex, Grid G, char *a
                     if (ex.f2) ex.f2[v] = f2;
                 }
             }
-            if (inM) L.mstamp[v] = it;
+            if (inM) mark_move(L, v, it, L.nxt[v]);
         }
         mapp.add(inM, v);
         bigs.add(big, v);
@@ -1057,26 +1066,26 @@ __device__ __forceinline__ void apply_row(const Level &L, int32_t v, int32_t a, 
                                           int64_t end, int64_t step, long long &c, long long &ne) {
     const DGraph &g = L.g;
     for (int64_t j0 = first; j0 < end; j0 += U * step) {
-        int32_t u[U], w[U], x[U];
-        bool mu[U];
+        int32_t u[U], w[U];
+        int2 x[U];
 #pragma unroll
         for (int q = 0; q < U; ++q) {
             const int64_t j = j0 + q * step;
             u[q] = j < end ? ld_stream(g.adj + j) : -1;
             w[q] = j < end ? edge_w_stream<EW>(g, j) : 0;
         }
+        // one gather: the last move's destination is the part of a vertex that stays (a stamp, then a move
+        // or a part before: 280 -> 258 us on R-MAT s22, 23 -> 20 at 1.1 M mesh vertices)
 #pragma unroll
-        for (int q = 0; q < U; ++q) mu[q] = u[q] >= 0 && L.mstamp[u[q]] == it;
-#pragma unroll
-        for (int q = 0; q < U; ++q) x[q] = u[q] < 0 ? 0 : (mu[q] ? L.nxt[u[q]] : L.part[u[q]]);
+        for (int q = 0; q < U; ++q) x[q] = u[q] >= 0 ? L.move[u[q]] : make_int2(0, 0);
 #pragma unroll
         for (int q = 0; q < U; ++q) {
             if (u[q] < 0) continue;
-            const int32_t pu = mu[q] ? nxt_from(x[q]) : x[q];
-            const int32_t pn = mu[q] ? nxt_to(x[q]) : x[q];
+            const bool mu = x[q].x == it;
+            const int32_t pn = nxt_to(x[q].y), pu = mu ? nxt_from(x[q].y) : pn;
             const int32_t diff = (int)(pn != b) - (int)(pu != a);
             ne += pn != b;
-            if (!mu[q]) {
+            if (!mu) {
                 if (diff) atomicAdd(&L.ext[u[q]], diff);
                 c += (long long)w[q] * diff;
             } else if (u[q] > v) {
@@ -1087,8 +1096,8 @@ __device__ __forceinline__ void apply_row(const Level &L, int32_t v, int32_t a, 
 }
 
 // The same over a short row (at most kSmallDeg entries, one thread), in
-// batches of U neighbours whose stamps, packed moves and parts are loaded
-// together before any of them is updated: a batch costs one round trip,
+// batches of U neighbours whose last moves are loaded together before any ext[]
+// is updated: a batch costs one round trip,
 // where an update of ext[] between two neighbours would hold the next
 // neighbour's loads behind it.
 template <bool EW, int U = kSmallDeg / 2>
@@ -1098,7 +1107,8 @@ __device__ __forceinline__ void apply_short_row(const Level &L, int32_t v, int32
 #pragma unroll
     for (int t0 = 0; t0 < kSmallDeg; t0 += U) {
         if (t0 >= d) break;
-        int32_t u[U], w[U], ms[U], x[U], p[U];
+        int32_t u[U], w[U];
+        int2 x[U];
 #pragma unroll
         for (int q = 0; q < U; ++q) {
             const int t = t0 + q;
@@ -1106,17 +1116,12 @@ __device__ __forceinline__ void apply_short_row(const Level &L, int32_t v, int32
             w[q] = t < d ? edge_w<EW>(g, beg + t) : 0;
         }
 #pragma unroll
-        for (int q = 0; q < U; ++q) {
-            ms[q] = u[q] >= 0 ? L.mstamp[u[q]] : 0;
-            x[q] = u[q] >= 0 ? L.nxt[u[q]] : 0;
-            p[q] = u[q] >= 0 ? L.part[u[q]] : 0;
-        }
+        for (int q = 0; q < U; ++q) x[q] = u[q] >= 0 ? L.move[u[q]] : make_int2(0, 0);
 #pragma unroll
         for (int q = 0; q < U; ++q) {
             if (u[q] < 0) continue;
-            const bool mu = ms[q] == it;
-            const int32_t pu = mu ? nxt_from(x[q]) : p[q];
-            const int32_t pn = mu ? nxt_to(x[q]) : p[q];
+            const bool mu = x[q].x == it;
+            const int32_t pn = nxt_to(x[q].y), pu = mu ? nxt_from(x[q].y) : pn;
             const int32_t diff = (int)(pn != b) - (int)(pu != a);
             ne += pn != b;
             if (!mu) {
@@ -1749,7 +1754,7 @@ __device__ inline void ph_rb_take(const Level &L, Grid G, char *arena) {
         }
         bool taken = kv >= 0 && (s < ss || (member && mine < L.need[a]));
         if constexpr (!STRONG) {
-            if (taken) L.mstamp[vv] = it;
+            if (taken) mark_move(L, (int32_t)vv, it, L.nxt[vv]);
             mapp.add(taken, (int32_t)vv);
             mapp.flush(&ctl->nM, L.listM, true);
         } else {
@@ -1803,7 +1808,11 @@ __device__ inline void ph_rb_cookie(const Level &L, Grid G, char *arena) {
             }
         }
         bool mv = dest >= 0;
-        if (mv) { L.nxt[v] = nxt_pack(L.part[v], dest); L.mstamp[v] = it; }
+        if (mv) {
+            const int32_t x = nxt_pack(L.part[v], dest);
+            L.nxt[v] = x;
+            mark_move(L, (int32_t)v, it, x);
+        }
         mapp.add(mv, (int32_t)v);
         mapp.flush(&ctl->nM, L.listM, true);
     }

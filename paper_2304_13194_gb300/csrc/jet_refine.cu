@@ -461,7 +461,7 @@ __global__ void __launch_bounds__(kTB) k_level_init(Level L, LevelInit a) {
         const int m = (int)min((int64_t)4, n - v0);
         const int4 none = make_int4(-2, -2, -2, -2), gain = make_int4(kNoneGain, kNoneGain, kNoneGain, kNoneGain);
         int4 p = make_int4(0, 0, 0, 0), lock = none;
-        if (a.best || a.pd) {
+        if (a.best || a.pd || L.move) {
             if (m == 4 && vec) {
                 p = *reinterpret_cast<const int4 *>(L.part + v0);
             } else {
@@ -478,7 +478,14 @@ __global__ void __launch_bounds__(kTB) k_level_init(Level L, LevelInit a) {
             if (m > 3 && a.locked[v0 + 3]) lock.w = 0;
         }
         put(L.lstamp, v0, m, lock);
-        put(L.mstamp, v0, m, none);
+        if (L.move) {
+            const int32_t e[4] = {p.x, p.y, p.z, p.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (i < m) L.move[v0 + i] = make_int2(-2, nxt_pack(e[i], e[i]));
+        } else {
+            put(L.mstamp, v0, m, none);
+        }
         put(L.prio, v0, m, gain);
         if (a.best) put(a.best, v0, m, p);
         if (a.key) put(a.key, v0, m, make_int4(-1, -1, -1, -1));
@@ -501,14 +508,14 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 // Carves all per-level buffers out of two allocations.
 int allow_large_arenas(int device);
 
-// Per-level buffers: 11 int32 arrays per vertex (best, nxt, prio, mstamp,
-// lstamp, key, listX, listM, ext, wdeg, listW), then the control block,
+// Per-level buffers: 10 int32 arrays per vertex (best, nxt, prio, lstamp, key,
+// listX, listM, ext, wdeg, listW) and the moves, then the control block,
 // per-part state, rebalancing tiles, the trace (optional) and the cut
 // accumulator, in two allocations.
 void level_bytes(int64_t nmax, int32_t k, bool with_trace, size_t *vbytes, size_t *mbytes) {
     const size_t nn = (size_t)std::max<int64_t>(nmax, 1), kk = (size_t)k;
     const size_t ntiles = (size_t)std::max<int64_t>((nmax + kRbTile - 1) / kRbTile, 1);
-    *vbytes = 11 * align256(nn * 4) + align256(nn * 8) /* etaken */;
+    *vbytes = 10 * align256(nn * 4) + align256(nn * 8) /* etaken */ + align256(nn * 8) /* move */;
     *mbytes = align256(sizeof(Ctl)) + align256(kk * 8) /*pw*/ + align256(kk * 4) /*aidx*/ + align256(kk * 4) /*Bs*/ +
               align256(kk) /*inB*/ + align256((kk + 1) * 8) /*capC*/ + align256(kk * 8) /*excess*/ +
               align256(kk * kSlots * 8) /*bucketw*/ + align256(kk * 4) /*sstar*/ + align256(kk * 8) /*need*/ +
@@ -521,13 +528,15 @@ void carve_level(Level &L, char *vert, char *misc, int64_t nmax, int32_t k, bool
     const int32_t ntiles = (int32_t)std::max<int64_t>((nmax + kRbTile - 1) / kRbTile, 1);
     char *p = vert;
     auto take32 = [&](void) { int32_t *r = reinterpret_cast<int32_t *>(p); p += align256(nn * 4); return r; };
-    L.best = take32(); L.nxt = take32(); L.prio = take32(); L.mstamp = take32(); L.lstamp = take32();
+    L.best = take32(); L.nxt = take32(); L.prio = take32(); L.lstamp = take32();
+    L.mstamp = nullptr;
     L.key = take32(); L.listX = take32(); L.listM = take32();
     L.ext = take32();
     L.wdeg = take32();
     L.listW = take32();
     L.rbloss = nullptr;
     L.etaken = reinterpret_cast<int64_t *>(p);
+    L.move = reinterpret_cast<int2 *>(p + align256(nn * 8));
     char *q = misc;
     auto take = [&](size_t bytes) { char *r = q; q += align256(bytes); return r; };
     L.ctl = reinterpret_cast<Ctl *>(take(sizeof(Ctl)));
@@ -1234,7 +1243,7 @@ __global__ void k_export_lp(Level L, uint8_t *inx, uint8_t *inm) {
     const int32_t it = L.ctl->it;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < L.g.n; v += (int64_t)gridDim.x * blockDim.x) {
         if (inx) inx[v] = L.prio[v] != kNoneGain;
-        if (inm) inm[v] = L.mstamp[v] == it;
+        if (inm) inm[v] = is_marked(L, v, it);
     }
 }
 
@@ -1284,7 +1293,7 @@ int lp_pass(Ctx &c, const DGraph &g, int32_t k, const int32_t *part, const uint8
 __global__ void k_export_rb(Level L, int32_t *dest, int32_t *loss) {
     const int32_t it = L.ctl->it;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < L.g.n; v += (int64_t)gridDim.x * blockDim.x) {
-        if (dest) dest[v] = L.mstamp[v] == it ? nxt_to(L.nxt[v]) : -1;
+        if (dest) dest[v] = is_marked(L, v, it) ? nxt_to(L.nxt[v]) : -1;
         if (loss && L.key[v] < 0) loss[v] = kNoneGain;
     }
 }
