@@ -77,9 +77,11 @@ extern "C" {
 #define JET_FLAG_TWO_HOP 256u      /* coarsening: add two-hop matches (Sec. 3.1) after heavy-edge matching;
                                       the plain method coarsens by heavy-edge matching alone */
 #define JET_FLAG_NO_PDL 1024u      /* execution choice (results do not depend on it): launch every
-                                      refinement kernel only after the previous one has finished,
-                                      instead of letting it start early and wait on the device
-                                      (programmatic dependent launch) */
+                                      refinement kernel, from the level's start on, and the matching
+                                      rounds only after the previous one has finished, instead of
+                                      letting it start early and wait on the device (programmatic
+                                      dependent launch); the other stages of coarsening, the sorts and
+                                      the network always launch early */
 #define JET_FLAG_GRID_LOOP 2048u   /* execution choice (results do not depend on it): levels above
                                       cluster_max_n run their whole refinement loop in one
                                       cooperative launch over the GPU (phases separated by grid
@@ -513,6 +515,12 @@ void jet_debug_fail_alloc(int64_t nth);
  * contexts and threads; every stream-ordered scratch allocation counts one).
  * A diagnostic: the paper has no counterpart. */
 int64_t jet_alloc_count(void);
+
+/* Kernel launches, and kernel nodes of captured graphs, that the library has
+ * made in this process so far with leave to start before the launch ahead of
+ * them has finished (programmatic dependent launch; JET_FLAG_NO_PDL).  A
+ * diagnostic: the paper has no counterpart. */
+int64_t jet_early_launch_count(void);
 
 /* Human-readable name of a status code (static storage). */
 const char *jet_status_string(int status);

@@ -36,7 +36,7 @@ EXPORTED_SYMBOLS = [
     "jet_coarsest_refined", "jet_lip_num_params", "jet_lip_create", "jet_lip_destroy", "jet_lip_get_params",
     "jet_lip_set_params", "jet_lip_features", "jet_lip_labels", "jet_lip_forward", "jet_lip_loss_grad",
     "jet_lip_train_step", "jet_lip_decode", "jet_lip_initial_partition", "jet_partition_learned", "jet_autotune",
-    "jet_kernel_name", "jet_alloc_count", "jet_debug_fail_alloc",
+    "jet_kernel_name", "jet_alloc_count", "jet_early_launch_count", "jet_debug_fail_alloc",
 ]
 LIP_FEATURES, LIP_HIDDEN, LIP_MAX_K, LIP_MAX_N = 16, 64, 256, 1 << 20
 JET_NOALLOC_MAX_N = 262144
@@ -192,6 +192,7 @@ def load_library(path: str | None = None):
             "jet_status_string": (ctypes.c_char_p, [ctypes.c_int]),
             "jet_kernel_name": (ctypes.c_char_p, [i32]),
             "jet_alloc_count": (i64, []),
+            "jet_early_launch_count": (i64, []),
             "jet_debug_fail_alloc": (None, [i64]),
             "jet_last_error": (ctypes.c_char_p, []),
         }
@@ -212,6 +213,12 @@ def debug_fail_alloc(nth: int) -> None:
 def alloc_count() -> int:
     """Device allocations the library has made in this process so far."""
     return int(load_library().jet_alloc_count())
+
+
+def early_launch_count() -> int:
+    """Launches the library has made in this process so far that may start
+    before the launch ahead of them has finished."""
+    return int(load_library().jet_early_launch_count())
 
 
 def kernel_names() -> list[str]:

@@ -33,6 +33,8 @@ static thread_local cudaMemPool_t t_pool = nullptr;
 static std::atomic<int64_t> g_alloc_count{0};
 static std::atomic<int64_t> g_fail_at{0};
 
+std::atomic<int64_t> g_early_launches{0};
+
 int dev_alloc(DevBuf &b, size_t bytes, cudaStream_t s) {
     b.release();
     b.s = s;
@@ -960,6 +962,8 @@ int jet_initial_partition(jet_ctx *ctx, int32_t n, const int64_t *xadj, const in
 }
 
 int64_t jet_alloc_count(void) { return g_alloc_count.load(std::memory_order_relaxed); }
+
+int64_t jet_early_launch_count(void) { return g_early_launches.load(std::memory_order_relaxed); }
 
 void jet_debug_fail_alloc(int64_t nth) {
     g_fail_at.store(nth > 0 ? g_alloc_count.load(std::memory_order_relaxed) + nth : 0, std::memory_order_relaxed);

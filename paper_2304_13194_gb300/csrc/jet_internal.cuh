@@ -3,6 +3,7 @@
 #pragma once
 
 #include <algorithm>
+#include <atomic>
 #include <cuda_runtime.h>
 #include <cstdint>
 #include <cstddef>
@@ -259,6 +260,9 @@ __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// Launches made with that permission so far (jet_early_launch_count).
+extern std::atomic<int64_t> g_early_launches;
+
 // A launch that, with pdl, may be scheduled before the previous kernel in
 // the stream completes; the kernel must begin with pdl_enter().
 template <class... KArgs, class... Args>
@@ -274,6 +278,7 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), int grid, int block, size_t smem,
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = pdl ? 1 : 0;
+    if (pdl) g_early_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 

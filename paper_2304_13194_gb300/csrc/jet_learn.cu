@@ -678,6 +678,7 @@ int gemm_tn(Ctx &c, int32_t M, int Kp, int Kv, int Np, int Nv, const float *A, i
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
+    g_early_launches.fetch_add(1, std::memory_order_relaxed);
     JET_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_gemm_tn, M, Kp, Kv, Np, Nv, A, lda, B, ldb, P, CS));
     JET_CUDA_TRY(launch_pdl(k_tn_reduce, grid_elems((int64_t)Kv * Nv + Nv), kTB, 0, c.stream, true, nb, Kp, Kv, Np, Nv,
                             (const float *)P, (const float *)CS, gW, gb));

@@ -725,7 +725,7 @@ int enqueue_start(Ctx &c, const Level &L, const LevelInit &init, int32_t *wdeg) 
     c.launches += 1;
     if (n > 0) {
         const int gcut = std::min(list_grid(), grid_for(n, kTB));
-        JET_CUDA_TRY(launch_pdl(L.g.ew ? k_cut_pw<true> : k_cut_pw<false>, gcut, kTB, sm_cut_pw(L.k), s, true, L.g, L.k,
+        JET_CUDA_TRY(launch_pdl(L.g.ew ? k_cut_pw<true> : k_cut_pw<false>, gcut, kTB, sm_cut_pw(L.k), s, L.pdl != 0, L.g, L.k,
                                 (const int32_t *)L.part, L.pw, init.cut2, L.ext, wdeg, &L.ctl->nbig));
         c.launches += 1;
     }
@@ -739,7 +739,7 @@ int enqueue_init(Ctx &c, LevelBufs &B, int64_t L_lim, int64_t opt, int64_t sigma
     init.best = L.best;
     init.cut2 = B.cut2;
     JET_TRY(enqueue_start(c, L, init, L.wdeg));
-    JET_CUDA_TRY(launch_pdl(k_ctl_init, 1, 1024, 0, c.stream, true, L, (const int64_t *)B.cut2, L_lim, opt, sigma));
+    JET_CUDA_TRY(launch_pdl(k_ctl_init, 1, 1024, 0, c.stream, L.pdl != 0, L, (const int64_t *)B.cut2, L_lim, opt, sigma));
     c.launches += 1;
     return JET_OK;
 }
@@ -1336,7 +1336,7 @@ int rebalance_pass(Ctx &c, const DGraph &g, int64_t W, int32_t k, double eps, in
     init.key = L.key;
     init.cut2 = B.cut2;
     JET_TRY(enqueue_start(c, L, init, L.wdeg));
-    JET_CUDA_TRY(launch_pdl(k_rb_pass_init, 1, 1024, 0, s, true, L, (const int64_t *)B.cut2,
+    JET_CUDA_TRY(launch_pdl(k_rb_pass_init, 1, 1024, 0, s, L.pdl != 0, L, (const int64_t *)B.cut2,
                             (int32_t)(strong ? MODE_RS : MODE_RW), iter, L_lim, opt, sigma));
     int nk = 0;
     JET_TRY(enqueue_rb(L, s, strong != 0, &nk));
