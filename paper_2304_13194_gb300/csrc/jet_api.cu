@@ -35,7 +35,9 @@ static std::atomic<int64_t> g_fail_at{0};
 
 std::atomic<int64_t> g_early_launches{0};
 
-int dev_alloc(DevBuf &b, size_t bytes, cudaStream_t s) {
+int dev_alloc(DevBuf &b, size_t bytes, cudaStream_t s) { return dev_alloc_from(b, bytes, s, t_pool); }
+
+int dev_alloc_from(DevBuf &b, size_t bytes, cudaStream_t s, cudaMemPool_t pool) {
     b.release();
     b.s = s;
     const int64_t idx = g_alloc_count.fetch_add(1, std::memory_order_relaxed) + 1;
@@ -45,7 +47,7 @@ int dev_alloc(DevBuf &b, size_t bytes, cudaStream_t s) {
         return JET_ENOMEM;
     }
     bytes = std::max<size_t>(256, (bytes + 255) & ~size_t(255));
-    cudaError_t e = t_pool ? cudaMallocFromPoolAsync(&b.p, bytes, t_pool, s) : cudaMallocAsync(&b.p, bytes, s);
+    cudaError_t e = pool ? cudaMallocFromPoolAsync(&b.p, bytes, pool, s) : cudaMallocAsync(&b.p, bytes, s);
     if (e != cudaSuccess) {
         b.p = nullptr;
         record_cuda_error(e, "cudaMallocAsync", __FILE__, __LINE__);
@@ -185,7 +187,8 @@ int check_input(Ctx &c, int32_t n, const int64_t *xadj, const int32_t *adjncy, c
     cudaStream_t s = c.stream;
     // four 16-byte loads a thread and pass; the entry count is not known here
     const int blocks = adjwgt ? num_sms() * 8 : std::min(num_sms() * 8, grid_for(n, kTB * 16));
-    k_check_input<<<blocks, kTB, 0, s>>>(n, xadj, vwgt, adjwgt, part, k, c.check, reinterpret_cast<CheckOut *>(c.pinned));
+    k_check_input<<<blocks, kTB, 0, s>>>(n, xadj, vwgt, adjwgt, part, k, c.check.as<CheckState>(),
+                                           reinterpret_cast<CheckOut *>(c.pinned));
     JET_CUDA_TRY(cudaGetLastError());
     JET_CUDA_TRY(cudaStreamSynchronize(s));
     memcpy(&out, c.pinned, sizeof(out));
@@ -512,18 +515,18 @@ int jet_ctx_create(int device, void *cuda_stream, const jet_options *opt, jet_ct
         c->c.pool = nullptr;
     }
     // state of the input checks (zero between them)
-    void *chk = nullptr;
-    cudaError_t e = c->c.pool ? cudaMallocFromPoolAsync(&chk, sizeof(CheckState), c->c.pool, c->c.stream)
-                              : cudaMallocAsync(&chk, sizeof(CheckState), c->c.stream);
-    if (e == cudaSuccess) {
-        c->c.check = static_cast<CheckState *>(chk);
-        e = cudaMemsetAsync(chk, 0, sizeof(CheckState), c->c.stream);
+    int r = dev_alloc_from(c->c.check, sizeof(CheckState), c->c.stream, c->c.pool);
+    if (r == JET_OK) {
+        cudaError_t e = cudaMemsetAsync(c->c.check.p, 0, sizeof(CheckState), c->c.stream);
+        if (e != cudaSuccess) {
+            record_cuda_error(e, "context state", __FILE__, __LINE__);
+            cudaGetLastError();
+            r = JET_ECUDA;
+        }
     }
-    if (e != cudaSuccess) {
-        record_cuda_error(e, "context state", __FILE__, __LINE__);
-        cudaGetLastError();
+    if (r < 0) {
         jet_ctx_destroy(c);
-        return e == cudaErrorMemoryAllocation ? JET_ENOMEM : JET_ECUDA;
+        return r;
     }
     *out = c;
     return JET_OK;
@@ -532,7 +535,7 @@ int jet_ctx_create(int device, void *cuda_stream, const jet_options *opt, jet_ct
 void jet_ctx_destroy(jet_ctx *ctx) {
     if (!ctx) return;
     cudaSetDevice(ctx->c.device);
-    if (ctx->c.check) cudaFreeAsync(ctx->c.check, ctx->c.stream);
+    ctx->c.check.release();
     cudaStreamSynchronize(ctx->c.stream);
     if (ctx->c.pinned) cudaFreeHost(ctx->c.pinned);
     if (t_pool == ctx->c.pool) t_pool = nullptr;

@@ -86,7 +86,10 @@ struct DevBuf {
 };
 
 // Allocate `bytes` (rounded up to 256) on stream s; returns JET_OK/JET_ENOMEM.
+// From the pool of the context whose entry point runs on this thread, or from
+// the one given (null: the device's default pool).
 int dev_alloc(DevBuf &b, size_t bytes, cudaStream_t s);
+int dev_alloc_from(DevBuf &b, size_t bytes, cudaStream_t s, cudaMemPool_t pool);
 
 // ---------------------------------------------------------------------------
 // graph view
@@ -533,7 +536,7 @@ struct Ctx {
     cudaStream_t stream = nullptr;
     jet_options opt{};
     int64_t *pinned = nullptr;   // pinned host buffer (layout: kPinned* below)
-    CheckState *check = nullptr; // device: state of the input checks
+    DevBuf check;                // state of the input checks (CheckState)
     cudaMemPool_t pool = nullptr; // the context's stream-ordered pool (keeps its memory between calls)
     TraceHost last_trace;
 };
