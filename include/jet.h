@@ -102,8 +102,8 @@ extern "C" {
  *                                   chain of them (coarsest first) in one launch; larger levels, and
  *                                   dense ones (more than 400,000 CSR entries and more than 40 per
  *                                   vertex), use the CUDA-graph loop; 0 = never.  Levels of up to 4096
- *                                   vertices (with a value above the default: of up to that many)
- *                                   run in one cluster launch also when they do not fit
+ *                                   vertices (with any other value than the default: of up to that
+ *                                   many) run in one cluster launch also when they do not fit
  *   cluster_blocks = 0              blocks of that cluster: 0 = chosen by the level's size (up to
  *                                   16), else a power of two in [2, 16]
  *   barrier_polls = 0               polls a block of the persistent level loop (JET_FLAG_GRID_LOOP)

@@ -1024,13 +1024,14 @@ int run_grid(Ctx &c, const Level &L, int *ran) {
 size_t cluster_smem(int32_t k) { return (arena_bytes(k, kClusterThreads) + 255) & ~size_t(255); }
 
 // Cluster size usable for this level (0: use the graph loop).  Levels that
-// the resident chain cannot hold get here: up to kClusterLoopMaxN vertices
-// this loop is the faster one, beyond that only on request (a cluster_max_n
-// above the default).
+// the resident chain does not take get here: up to kClusterLoopMaxN vertices
+// this loop is the faster one, beyond that it runs on request only: a
+// cluster_max_n that the caller chose (any value but the default) holds for it
+// as well.
 int pick_cluster(Ctx &c, const Level &L, int *cs) {
     *cs = 0;
-    if (L.g.n <= 0 || L.g.n > c.opt.cluster_max_n) return JET_OK;
-    if (L.g.n > kClusterLoopMaxN && c.opt.cluster_max_n <= kClusterMaxNDefault) return JET_OK;
+    const int32_t most = c.opt.cluster_max_n == kClusterMaxNDefault ? kClusterLoopMaxN : c.opt.cluster_max_n;
+    if (L.g.n <= 0 || L.g.n > most) return JET_OK;
     if (L.g.ew) JET_TRY(cluster_size<true>(c.device, cluster_smem(L.k), cs));
     else JET_TRY(cluster_size<false>(c.device, cluster_smem(L.k), cs));
     if (c.opt.cluster_blocks > 0 && *cs > c.opt.cluster_blocks) *cs = c.opt.cluster_blocks;
