@@ -99,11 +99,15 @@ extern "C" {
  * Execution choice (no counterpart in the paper; results do not depend on it):
  *   cluster_max_n = 65536           levels with at most this many vertices that fit the shared
  *                                   memory of one thread-block cluster are refined there, the whole
- *                                   chain of them (coarsest first) in one launch; larger levels, and
- *                                   dense ones (more than 400,000 CSR entries and more than 40 per
- *                                   vertex), use the CUDA-graph loop; 0 = never.  Levels of up to 4096
- *                                   vertices (with any other value than the default: of up to that
- *                                   many) run in one cluster launch also when they do not fit
+ *                                   chain of them (coarsest first) in one launch.  What fits depends
+ *                                   on k: about 65,200 vertices at k = 8, 60,400 at 64, 50,200 at 128,
+ *                                   34,400 at 256, 21,400 at 257, 4,300 at 480, 500 at 530.
+ *                                   Larger levels, and those with more CSR entries than one cluster
+ *                                   walks as fast as the whole GPU (480,000 / (1 + k / 160), less for
+ *                                   many parts on up to 8,192 vertices), use the CUDA-graph loop;
+ *                                   0 = never.  Levels of up to 4096 vertices (with any other value
+ *                                   than the default: of up to that many) run in one cluster launch
+ *                                   on their state in global memory where the first form is not used
  *   cluster_blocks = 0              blocks of that cluster: 0 = chosen by the level's size (up to
  *                                   16), else a power of two in [2, 16]
  *   barrier_polls = 0               polls a block of the persistent level loop (JET_FLAG_GRID_LOOP)

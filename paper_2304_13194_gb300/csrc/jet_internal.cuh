@@ -602,7 +602,7 @@ struct ResChainLevel {
     bool is_finest = false;
 };
 // Blocks of the cluster that keeps a level of n vertices and nnz entries (0: it
-// does not fit, or the options exclude it).
+// does not fit, another loop is faster, or the options exclude it).
 int resident_cluster(Ctx &c, int64_t n, int64_t nnz, int32_t k, int *cs);
 // Enqueues the chain (no host wait); init: the partition its first level
 // starts from.  Outcomes are read by refine_level_finish.

@@ -1462,9 +1462,31 @@ int device_info(int device, int32_t k, ResDevice &out) {
     return JET_OK;
 }
 
-// Dense levels stay with the per-kernel loop: their rows outgrow the cluster's
-// shared memory and 16 SMs read them slower than the whole GPU does.
-constexpr int64_t kResDenseNnz = 400000, kResDenseDeg = 40;
+// Entries up to which a level of n vertices and k parts is kept.  Sixteen SMs
+// read a level's rows slower than the whole GPU does, and a row that meets more
+// than kSeen parts is walked again by a warp that then scans k table entries;
+// how many rows a pass reads is not known here, so the lines are those of
+// graphs without locality, where nearly every row lies on a boundary (uniform
+// random graphs, R-MAT).  Measured there (the loop such a level takes otherwise
+// / this one): n = 60,000, k = 8: 479,000 entries 1.05, 900,000 0.56; k = 64:
+// n = 48,000, 335,000 entries 1.06, 479,000 0.84; n = 60,000, 299,000 1.11,
+// 659,000 0.60; k = 128: n = 48,000, 239,000 1.14, 335,000 0.88; k = 256:
+// n = 24,000, 191,000 1.04, 287,000 0.85; R-MAT s15 (883,000), k = 256: 0.51.
+// Meshes and geometric graphs gain further on (k = 64: 1.9 at n = 60,000 and
+// 477,000 entries), but their sizes do not tell them apart.
+// Up to 8,192 vertices 512 threads a block walk the rows: n = 8,000, k = 8,
+// 342,000 entries 1.11, 398,000 0.93; n = 6,000, k = 192: 149,000 1.01,
+// 197,000 0.87; k = 256: 59,000 1.11, 149,000 0.94; k = 384: 29,000 1.05,
+// 95,000 0.91.  Up to 4,096 the loop to beat is the cluster loop: k = 256:
+// 147,000 1.02, 198,000 0.98; k = 384: 99,000 1.13, 147,000 0.94; k = 480:
+// 59,000 1.03, 147,000 0.86; above 400,000 entries this loop does not gain on it,
+// nor on longer rows with few blocks (n = 1,000, k = 64: 258,000 1.05, 322,000 0.97).
+int64_t res_entry_limit(int64_t n, int32_t k) {
+    const int64_t wide = 76800000 / (160 + k);       // 480,000 / (1 + k / 160)
+    if (n > 8192) return wide;
+    if (n > 4096) return std::min<int64_t>({350000, wide, 5000000000 / ((int64_t)k * k)});
+    return std::min<int64_t>({400000, 280 * n, 40000000 / k});
+}
 
 bool res_fits(int64_t n, int32_t k, int cs, uint32_t arena) {
     if (n <= 0 || n > 262144) return false;
@@ -1478,10 +1500,11 @@ bool res_fits(int64_t n, int32_t k, int cs, uint32_t arena) {
 
 int resident_cluster(Ctx &c, int64_t n, int64_t nnz, int32_t k, int *cs) {
     *cs = 0;
-    if (n <= 0 || n > c.opt.cluster_max_n || (nnz > kResDenseNnz && nnz > kResDenseDeg * n)) return JET_OK;
+    const int want = c.opt.cluster_blocks;
+    // fewer blocks by choice: fewer entries (a small level's few blocks are enough for its rows)
+    if (n <= 0 || n > c.opt.cluster_max_n || nnz > res_entry_limit(n, k) * (want > 0 ? want : 16) / 16) return JET_OK;
     ResDevice d;
     JET_TRY(device_info(c.device, k, d));
-    const int want = c.opt.cluster_blocks;
     if (want > 0) {
         if (want <= d.cluster && res_fits(n, k, want, d.arena)) *cs = want;
         return JET_OK;
