@@ -259,7 +259,9 @@ int jet_partition_host(jet_ctx *ctx, int32_t n, const int64_t *xadj, const int32
  * bit-identical to a jet_partition call with the same arguments); `workers`
  * host threads (<= 0: 8) each drive their own stream and memory pool on the
  * context's device; a graph's coarse levels occupy a few SMs, so that graphs
- * whose refinement is latency-bound share the GPU.  The work starts after what is already enqueued on the
+ * whose refinement is latency-bound share the GPU.  Many graphs of up to 4,096
+ * vertices on few workers are coarsened by these and then refined together in
+ * one persistent launch.  The work starts after what is already enqueued on the
  * context's stream and is complete when the call returns.  Returns JET_OK
  * when every item succeeded or returned a warning, else the status of the
  * first failed item (each item's own status is in its `status`). */

@@ -702,6 +702,40 @@ int jet_partition(jet_ctx *ctx, int32_t n, const int64_t *xadj, const int32_t *a
 // and pool) take graphs from a counter and partition them one after another,
 // each bit-identical to jet_partition.  A graph's coarse levels are one
 // resident-chain launch on a few SMs, so the workers' graphs share the GPU.
+//
+// Graphs of up to kClusterLoopMaxN vertices may take another way: the workers
+// coarsen them and make their greedy starts, and one persistent launch refines
+// all of them (refine_small_graphs).  An iteration is slower there, but its
+// clusters take some 30 graphs at once, where a worker has one in flight.  With
+// q such graphs, one launch lasts about as long as a worker takes for `graphs`
+// of them, per 30 graphs; the sums below compare the two.  Measured (whole
+// calls of 64 graphs of 1,000 to 4,000 vertices; partition by partition /
+// launch, ms): k <= 64, 1 worker 143 / 56, 2: 76 / 41, 3: 54 / 57, 8: 30 / 52;
+// k = 256, 1: 195 / 55, 4: 56 / 42, 8: 38 / 50; k = 600 (no resident loop), 1:
+// 209 / 51, 4: 59 / 39, 8: 62 / 40; 16 graphs, 1 worker, k <= 64: 35 / 19, 8
+// graphs: 18 / 20; k = 256, 8 graphs, 1 worker: 29 / 15, 8 workers: 9 / 18.
+static bool queue_small_graphs(Ctx &c, int32_t count, const jet_batch_item *items, int32_t workers,
+                               std::vector<char> &small, int *status) {
+    *status = JET_OK;
+    if (c.opt.flags & (JET_FLAG_HOSTLOOP | JET_FLAG_PROFILE)) return false;
+    int32_t q = 0;
+    double load = 0;   // in launches of up to 30 graphs
+    for (int32_t i = 0; i < count; ++i) {
+        const jet_batch_item &it = items[i];
+        if (it.n <= 0 || it.n > std::min(kClusterLoopMaxN, c.opt.cluster_max_n)) continue;
+        int cs = 0;
+        *status = resident_cluster(c, it.n, 0, it.k, &cs);   // entries are not known here
+        if (*status < 0) return false;
+        // graphs that a worker partitions in the time of one launch
+        const double graphs = cs == 0 ? 3.0 : std::max(3.9, std::min(12.0, 12.0 * 64 / it.k));
+        small[(size_t)i] = 1;
+        load += 1.0 / graphs;
+        ++q;
+    }
+    // more than 8 workers do not help: a resident cluster has up to 16 of the SMs
+    return load > std::min(workers, 8) * std::max(1.0, q / 30.0);
+}
+
 int jet_partition_batch(jet_ctx *ctx, int32_t count, jet_batch_item *items, int32_t workers) {
     if (!ctx || count < 0 || (count > 0 && !items)) return JET_EINVAL;
     if (count == 0) return JET_OK;
@@ -737,40 +771,116 @@ int jet_partition_batch(jet_ctx *ctx, int32_t count, jet_batch_item *items, int3
         JET_TRY(jet_ctx_create(c.device, w.s, &wo, &w.wc));
     }
     JET_TRY(use_device(c));
-    std::vector<int> wstat((size_t)workers, JET_OK);
-    std::atomic<int32_t> next{0};
-    auto body = [&](int w) {
-        jet_ctx *wc = wk[(size_t)w].wc;
-        for (;;) {
-            const int32_t i = next.fetch_add(1);
-            if (i >= count) break;
-            jet_batch_item &it = items[i];
-            auto t0 = std::chrono::steady_clock::now();
-            it.cut = 0;
-            it.status = it.n == 0 ? JET_OK
-                                  : jet_partition(wc, it.n, it.xadj, it.adjncy, it.vwgt, it.adjwgt, it.k, it.eps,
-                                                  it.seed, it.part_out, &it.cut, nullptr);
-            it.ms = (float)std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
-        }
-        if (cudaStreamSynchronize(wk[(size_t)w].s) != cudaSuccess) {
-            cudaGetLastError();
-            wstat[(size_t)w] = JET_ECUDA;
+    struct Item {
+        jet_hier *h = nullptr;
+        DevBuf init;                 // greedy start of the coarsest level (worker's pool)
+        ~Item() {
+            if (h) jet_hier_destroy(h);
         }
     };
-    std::vector<std::thread> pool;
-    int started = 0;
-    try {
-        pool.reserve((size_t)workers);
-        for (int w = 0; w < workers; ++w) {
-            pool.emplace_back(body, w);
-            ++started;
+    std::vector<Item> st((size_t)count);
+    std::vector<char> small((size_t)count, 0);
+    std::vector<int> wstat((size_t)workers, JET_OK);
+    int qs = JET_OK;
+    const bool queue = queue_small_graphs(c, count, items, workers, small, &qs);
+    JET_TRY(qs);
+    // runs fn(worker context, item) over all items on the workers, timed
+    auto run_workers = [&](auto &&fn) {
+        std::atomic<int32_t> next{0};
+        auto body = [&](int w) {
+            jet_ctx *wc = wk[(size_t)w].wc;
+            for (;;) {
+                const int32_t i = next.fetch_add(1);
+                if (i >= count) break;
+                auto t0 = std::chrono::steady_clock::now();
+                fn(wc, i);
+                items[i].ms += (float)std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
+            }
+            if (cudaStreamSynchronize(wk[(size_t)w].s) != cudaSuccess) {
+                cudaGetLastError();
+                wstat[(size_t)w] = JET_ECUDA;
+            }
+        };
+        std::vector<std::thread> pool;
+        int started = 0;
+        try {
+            pool.reserve((size_t)workers);
+            for (int w = 0; w < workers; ++w) {
+                pool.emplace_back(body, w);
+                ++started;
+            }
+        } catch (...) {   // no exception crosses the C ABI: the workers that started take every item
+            if (started == 0) body(0);   // none did: the calling thread takes the whole batch
         }
-    } catch (...) {   // no exception crosses the C ABI: the workers that started take every item
-        if (started == 0) body(0);   // none did: the calling thread takes the whole batch
-    }
-    for (auto &t : pool) t.join();
+        for (auto &t : pool) t.join();
+    };
+    // a small graph up to its start partition (queued), any other one whole
+    run_workers([&](jet_ctx *wc, int32_t i) {
+        jet_batch_item &it = items[i];
+        it.cut = 0;
+        it.ms = 0.f;
+        it.status = JET_OK;
+        if (it.n == 0) return;
+        if (!queue || !small[(size_t)i]) {
+            it.status = jet_partition(wc, it.n, it.xadj, it.adjncy, it.vwgt, it.adjwgt, it.k, it.eps, it.seed, it.part_out,
+                                      &it.cut, nullptr);
+            return;
+        }
+        Item &s1 = st[(size_t)i];
+        int r = jet_coarsen(wc, it.n, it.xadj, it.adjncy, it.vwgt, it.adjwgt, it.k, it.seed, &s1.h);
+        if (r >= 0) {
+            const jet_hier *h = s1.h;
+            const int32_t l = h->levels - 1;
+            DGraph g;
+            g.n = h->n[l]; g.nnz = h->nnz[l]; g.xadj = h->xadj[l]; g.adj = h->adj[l]; g.vw = h->vw[l]; g.ew = h->ew[l];
+            r = dev_alloc(s1.init, (size_t)g.n * 4, wc->c.stream);
+            if (r >= 0) r = initial_partition(wc->c, g, it.k, s1.init.as<int32_t>());
+        }
+        if (r < 0) it.status = r;
+    });
     for (int w = 0; w < workers; ++w)
         if (wstat[(size_t)w] != JET_OK) return wstat[(size_t)w];
+    if (queue) {
+        std::vector<SmallGraph> graphs;
+        std::vector<int32_t> at;
+        for (int32_t i = 0; i < count; ++i) {
+            if (!small[(size_t)i] || items[i].status < 0) continue;
+            const jet_batch_item &it = items[i];
+            SmallGraph sg;
+            sg.h = st[(size_t)i].h;
+            sg.k = it.k;
+            sg.eps = it.eps;
+            sg.seed = it.seed;
+            sg.init = st[(size_t)i].init.as<int32_t>();
+            sg.out = it.part_out;
+            graphs.push_back(sg);
+            at.push_back(i);
+        }
+        int ran = 0;
+        JET_TRY(use_device(c));
+        const int r = refine_small_graphs(c, graphs.data(), (int32_t)graphs.size(), &ran);
+        if (r < 0) {
+            cudaStreamSynchronize(c.stream);   // nothing of the call may still read the hierarchies
+            return r;
+        }
+        if (ran) {
+            for (size_t j = 0; j < graphs.size(); ++j) {
+                items[at[j]].cut = graphs[j].cut;
+                items[at[j]].status = graphs[j].status;
+            }
+        } else {
+            run_workers([&](jet_ctx *wc, int32_t i) {
+                jet_batch_item &it = items[i];
+                if (!small[(size_t)i] || it.status < 0) return;
+                it.status = use_device(wc->c);
+                if (it.status >= 0)
+                    it.status = uncoarsen(wc->c, st[(size_t)i].h, it.k, it.eps, it.seed, st[(size_t)i].init.as<int32_t>(),
+                                          it.part_out, &it.cut, nullptr);
+            });
+            for (int w = 0; w < workers; ++w)
+                if (wstat[(size_t)w] != JET_OK) return wstat[(size_t)w];
+        }
+    }
     for (int32_t i = 0; i < count; ++i)
         if (items[i].status < 0) return items[i].status;
     return JET_OK;

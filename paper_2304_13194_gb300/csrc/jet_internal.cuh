@@ -608,6 +608,21 @@ int resident_cluster(Ctx &c, int64_t n, int64_t nnz, int32_t k, int *cs);
 // starts from.  Outcomes are read by refine_level_finish.
 int resident_enqueue(Ctx &c, const ResChainLevel *lv, int32_t nlv, int32_t k, double eps, int64_t W, int cs,
                      const int32_t *init, bool want_trace);
+// The batched form's small graphs: each one's whole hierarchy, refined with
+// those of the others in one persistent cluster launch (k_refine_batch).
+struct SmallGraph {
+    const jet_hier *h = nullptr;
+    int32_t k = 2;
+    double eps = 0.03;
+    uint64_t seed = 1;               // the partition's seed (level seeds derive from it)
+    const int32_t *init = nullptr;   // device: start partition of the coarsest level
+    int32_t *out = nullptr;          // device: receives the partition
+    int64_t cut = 0;                 // out
+    int32_t status = JET_OK;         // out
+};
+// Every graph's `out` and outcome when *ran is 1; 0: the device cannot run one
+// cluster of the launch, nothing is done.
+int refine_small_graphs(Ctx &c, SmallGraph *graphs, int32_t count, int *ran);
 uint64_t level_seed(uint64_t seed, int32_t level);   // Jetrw seed of hierarchy level `level`
 
 // Enqueue + synchronise + finish.

@@ -422,6 +422,119 @@ __global__ void __launch_bounds__(kTB, JET_ROW_MINB) k_refine_grid(Level L) {
 }
 
 // ---------------------------------------------------------------------------
+// batched form: the small graphs of a batch in one persistent launch
+// ---------------------------------------------------------------------------
+// A job is one small graph's whole hierarchy, coarsest level first.  The
+// clusters of one launch take jobs from a counter; a cluster runs per level the
+// projection of the coarser level's partition, the level's start state, the
+// whole Alg. 3 loop and the P_best copy, then takes the next job.  Every
+// decision is the one the per-level launches take, so results are
+// bit-identical.  An iteration takes longer here than in the resident loop
+// (its steps are trips to L2), but some 30 graphs run at once whatever the
+// number of host threads: where the choice lies and why is at the caller.
+struct BatchLevel {
+    DGraph g;
+    const int32_t *cmap;     // this level -> the next coarser one (unused on the job's coarsest level)
+    uint64_t seed;           // Jetrw seed of the level
+    int32_t cq16;            // first-filter ratio c of the level (c_fine on level 0)
+    int32_t pad;
+};
+struct BatchStat {           // the finest level's outcome
+    int64_t best_cut;
+    int32_t best_bal, hit_cap;
+};
+struct BatchJob {
+    Level L;                 // buffers sized for the graph's largest level; the level fields are set per level
+    const BatchLevel *lv;    // [nlv], coarsest first
+    BatchStat *stat;
+    const int32_t *init;     // start partition of the coarsest level
+    int32_t *part[2];        // level partitions, alternating (level i in part[i & 1])
+    int32_t *out;            // receives the finest level's partition
+    int64_t *cut2;           // scratch: twice the start cut of a level
+    int64_t Llim, opt, sigma;
+    int32_t nlv, pad;
+};
+
+// Start of one level inside a job (all blocks of the cluster): projection,
+// per-vertex start values, cut / part weights / ext / weighted degree and
+// whether there are long rows, then the control block (block 0) and P_best = P_0.
+__device__ inline void batch_level_start(const BatchJob &job, const Level &L, int32_t i, Grid G, char *arena,
+                                         cg::cluster_group &cl) {
+    const int64_t n = L.g.n;
+    const int64_t t0 = (int64_t)G.bid * blockDim.x + threadIdx.x, stride = (int64_t)G.nb * blockDim.x;
+    const int32_t *prev = i == 0 ? job.init : job.part[(i - 1) & 1];
+    const int32_t *cmap = job.lv[i].cmap;
+    for (int64_t v = t0; v < n; v += stride) {
+        const int32_t p = prev[i == 0 ? v : (int64_t)cmap[v]];
+        L.part[v] = L.best[v] = p;
+        L.lstamp[v] = -2;
+        L.move[v] = make_int2(-2, nxt_pack(p, p));
+        L.prio[v] = kNoneGain;
+    }
+    if (G.bid == 0) {
+        int64_t *w = reinterpret_cast<int64_t *>(L.ctl);
+        for (int q = threadIdx.x; q < (int)(sizeof(Ctl) / 8); q += blockDim.x) w[q] = 0;
+        for (int p = threadIdx.x; p < L.k; p += blockDim.x) L.pw[p] = 0;
+        if (threadIdx.x == 0) job.cut2[0] = 0;
+    }
+    cl.sync();
+    if (L.g.ew) ph_cut_pw<true>(L.g, L.k, L.part, L.pw, job.cut2, L.ext, L.wdeg, G, arena, &L.ctl->nbig);
+    else ph_cut_pw<false>(L.g, L.k, L.part, L.pw, job.cut2, L.ext, L.wdeg, G, arena, &L.ctl->nbig);
+    cl.sync();
+    if (G.bid == 0) {
+        if (threadIdx.x == 0) {
+            L.ctl->L = job.Llim;
+            L.ctl->opt = job.opt;
+            L.ctl->sigma = job.sigma;
+        }
+        __syncthreads();
+        ph_ctl_init(L, job.cut2);
+    }
+    cl.sync();
+}
+
+__global__ void __launch_bounds__(kClusterThreads, 1) k_refine_batch(const BatchJob *jobs, int32_t njobs,
+                                                                     int32_t *queue) {
+    cg::cluster_group cl = cg::this_cluster();
+    const Grid G{(int)cl.block_rank(), (int)cl.num_blocks()};
+    char *arena = JET_ARENA;
+    __shared__ int s_job;
+    __shared__ Level L;   // the level's parameters, in shared memory rather than on each thread's stack
+    for (;;) {
+        if (G.bid == 0 && threadIdx.x == 0) s_job = atomicAdd(queue, 1);
+        cl.sync();
+        const int j = *cl.map_shared_rank(&s_job, 0);
+        cl.sync();   // every block has read the job before block 0 takes the next (or leaves)
+        if (j >= njobs) break;
+        const BatchJob &job = jobs[j];
+        for (int32_t i = 0; i < job.nlv; ++i) {
+            if (threadIdx.x == 0) {
+                const BatchLevel &bl = job.lv[i];
+                L = job.L;
+                L.g = bl.g;
+                L.seed = bl.seed;
+                L.cq16 = bl.cq16;
+                L.ntiles = (int32_t)(((int64_t)bl.g.n + kClusterThreads - 1) / kClusterThreads);
+                if (L.ntiles < 1) L.ntiles = 1;
+                L.part = job.part[i & 1];
+            }
+            __syncthreads();
+            batch_level_start(job, L, i, G, arena, cl);
+            if (L.g.ew) cluster_level_loop<true>(L, G, arena, cl);
+            else cluster_level_loop<false>(L, G, arena, cl);
+            cl.sync();
+            // P_best is the level's result
+            const int64_t n = L.g.n, t0 = (int64_t)G.bid * blockDim.x + threadIdx.x, stride = (int64_t)G.nb * blockDim.x;
+            int32_t *dst = i + 1 == job.nlv ? job.out : L.part;
+            for (int64_t v = t0; v < n; v += stride) dst[v] = L.best[v];
+            if (i + 1 == job.nlv && G.bid == 0 && threadIdx.x == 0)
+                *job.stat = BatchStat{L.ctl->best_cut, L.ctl->best_bal, L.ctl->hit_cap};
+            cl.sync();
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
 // Start values of a level's arrays in one pass over the vertices (one launch
@@ -1236,6 +1349,144 @@ int refine_level(Ctx &c, const DGraph &g, int32_t k, double eps, int32_t is_fine
         return JET_ECUDA;
     }
     return refine_level_finish(c, run, cut_out, maxw_out, rep_out);
+}
+
+// ---- batched form: the small graphs of a batch -------------------------------
+
+// Clusters of `cs` blocks of k_refine_batch that run at once on this device (0:
+// none).  The kernel's largest arena is set once per device, so that calls with
+// fewer parts cannot lower it under a concurrent one.
+static int batch_clusters(int device, int cs, size_t smem, int *out) {
+    static std::mutex mu;
+    static bool done[256];
+    *out = 0;
+    if (device < 0 || device >= 256) return JET_OK;
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        if (!done[device]) {
+            JET_CUDA_TRY(cudaFuncSetAttribute(k_refine_batch, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+            JET_CUDA_TRY(cudaFuncSetAttribute(k_refine_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)cluster_smem(JET_MAX_K)));
+            done[device] = true;
+        }
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(cs);
+    cfg.blockDim = dim3(kClusterThreads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = cs;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(out, k_refine_batch, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        *out = 0;
+    }
+    return JET_OK;
+}
+
+int refine_small_graphs(Ctx &c, SmallGraph *graphs, int32_t count, int *ran) {
+    *ran = 0;
+    if (count <= 0) return JET_OK;
+    cudaStream_t s = c.stream;
+    int32_t kmax = 1;
+    int64_t nlv_total = 0;
+    for (int32_t j = 0; j < count; ++j) {
+        kmax = std::max(kmax, graphs[j].k);
+        nlv_total += graphs[j].h->levels;
+    }
+    // launch shape: clusters of cluster_blocks blocks (default 4), as many as are co-resident
+    const size_t smem = cluster_smem(kmax);
+    int cs = c.opt.cluster_blocks > 0 ? c.opt.cluster_blocks : 4, nclusters = 0;
+    for (; cs >= 2; cs /= 2) {
+        JET_TRY(batch_clusters(c.device, cs, smem, &nclusters));
+        if (nclusters >= 1) break;
+    }
+    if (nclusters < 1) return JET_OK;   // the caller takes the graphs one by one
+    nclusters = std::min(nclusters, count);
+    // a graph's buffers: level arrays and two level partitions, sized for its finest level
+    size_t total = 0;
+    std::vector<size_t> off((size_t)count);
+    for (int32_t j = 0; j < count; ++j) {
+        const int64_t n = graphs[j].h->n[0];
+        size_t vb = 0, mb = 0;
+        level_bytes(n, graphs[j].k, false, &vb, &mb);
+        off[(size_t)j] = total;
+        total += align256(vb) + align256(mb) + 2 * align256((size_t)n * 4);
+    }
+    const size_t jobs_off = total;
+    const size_t lv_off = jobs_off + align256(sizeof(BatchJob) * (size_t)count);
+    const size_t st_off = lv_off + align256(sizeof(BatchLevel) * (size_t)nlv_total);
+    const size_t q_off = st_off + align256(sizeof(BatchStat) * (size_t)count);
+    DevBuf buf;
+    JET_TRY(dev_alloc(buf, q_off + 256, s));
+    char *base = buf.as<char>();
+    BatchJob *d_jobs = reinterpret_cast<BatchJob *>(base + jobs_off);
+    BatchLevel *d_lv = reinterpret_cast<BatchLevel *>(base + lv_off);
+    BatchStat *d_st = reinterpret_cast<BatchStat *>(base + st_off);
+    int32_t *d_queue = reinterpret_cast<int32_t *>(base + q_off);
+    std::vector<BatchJob> jobs((size_t)count);
+    std::vector<BatchLevel> lvs((size_t)nlv_total);
+    int64_t li = 0;
+    for (int32_t j = 0; j < count; ++j) {
+        const SmallGraph &sg = graphs[j];
+        const jet_hier *h = sg.h;
+        const int64_t n = h->n[0];
+        size_t vb = 0, mb = 0;
+        level_bytes(n, sg.k, false, &vb, &mb);
+        char *p = base + off[(size_t)j];
+        BatchJob &jb = jobs[(size_t)j];
+        memset(&jb, 0, sizeof(jb));
+        carve_level(jb.L, p, p + align256(vb), n, sg.k, false, &jb.cut2);
+        fill_level_params(c, jb.L, 0, 0);   // per-level fields (c, seed, graph) are set in the kernel
+        jb.part[0] = reinterpret_cast<int32_t *>(p + align256(vb) + align256(mb));
+        jb.part[1] = jb.part[0] + align256((size_t)n * 4) / 4;
+        jb.init = sg.init;
+        jb.out = sg.out;
+        jb.lv = d_lv + li;
+        jb.stat = d_st + j;
+        jb.nlv = h->levels;
+        jb.Llim = balance_limit(h->W, sg.k, sg.eps, &jb.opt);
+        jb.sigma = jb.opt + (jb.Llim - jb.opt) / 2;
+        for (int32_t lv = h->levels - 1; lv >= 0; --lv, ++li) {
+            BatchLevel &bl = lvs[(size_t)li];
+            memset(&bl, 0, sizeof(bl));
+            bl.g.n = h->n[lv]; bl.g.nnz = h->nnz[lv]; bl.g.xadj = h->xadj[lv]; bl.g.adj = h->adj[lv];
+            bl.g.vw = h->vw[lv]; bl.g.ew = h->ew[lv];
+            bl.cmap = h->cmap[lv];
+            bl.seed = level_seed(sg.seed, lv);
+            bl.cq16 = (int32_t)llround((lv == 0 ? c.opt.c_fine : c.opt.c_coarse) * 65536.0);
+        }
+    }
+    JET_CUDA_TRY(cudaMemcpyAsync(d_jobs, jobs.data(), sizeof(BatchJob) * (size_t)count, cudaMemcpyHostToDevice, s));
+    JET_CUDA_TRY(cudaMemcpyAsync(d_lv, lvs.data(), sizeof(BatchLevel) * (size_t)nlv_total, cudaMemcpyHostToDevice, s));
+    JET_CUDA_TRY(cudaMemsetAsync(d_queue, 0, 4, s));
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(nclusters * cs));
+    cfg.blockDim = dim3(kClusterThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = cs;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    JET_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_refine_batch, (const BatchJob *)d_jobs, count, d_queue));
+    c.launches += 1;
+    std::vector<BatchStat> st((size_t)count);
+    JET_CUDA_TRY(cudaMemcpyAsync(st.data(), d_st, sizeof(BatchStat) * (size_t)count, cudaMemcpyDeviceToHost, s));
+    JET_CUDA_TRY(cudaStreamSynchronize(s));   // also keeps the host arrays of the copies alive until done
+    for (int32_t j = 0; j < count; ++j) {
+        graphs[j].cut = st[(size_t)j].best_cut;
+        graphs[j].status = !st[(size_t)j].best_bal ? JET_WUNBALANCED : (st[(size_t)j].hit_cap ? JET_WITERLIMIT : JET_OK);
+    }
+    *ran = 1;
+    return JET_OK;
 }
 
 // ---- single passes --------------------------------------------------------
