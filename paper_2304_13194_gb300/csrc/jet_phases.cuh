@@ -417,8 +417,8 @@ __device__ __forceinline__ void reset_counters(Ctl *ctl) {
 //   lp_scan      4n + 4 nb + 4 w           ext of every vertex, lock stamp of the
 //                                          boundary ones, work-list writes
 //   lp_select    24 w + beta deg(W) + 12|X| list, xadj pair, part; rows; prio, nxt, X list
-//   afterburn    32|X| + beta deg(X) + 8|M|  X list, xadj pair, prio, nxt, part; rows;
-//                                          move, M list (4|X| + 8|M| without afterburner)
+//   afterburn    32|X| + beta deg(X) + 12|M|  X list, xadj pair, prio, nxt, part; rows;
+//                                          move, M list (4|X| + 16|M| without afterburner: + nxt)
 //   apply        36|M| + beta deg(M) + 16k  M list, nxt, vwgt, xadj pair, ext, part
 //                                          (+4|M| lock stamps and 8|X| priority resets
 //                                          after Jetlp); rows; part weights
@@ -427,10 +427,10 @@ __device__ __forceinline__ void reset_counters(Ctl *ctl) {
 //   rb_cand      28r (+4r Jetrw) + beta deg(R)  list, xadj pair, part, key (+ destination); rows
 //   rb_tilehist  4n + 4c + 4 T nA          key, vwgt of candidates, tile sums
 //   rb_tilescan  8 T nA                    tile sums read and written
-//   rb_take      4n + 4c + 4 T nA + 8|M|   key, vwgt, tile offsets; move, M list
+//   rb_take      4n + 4c + 4 T nA + 16|M|  key, vwgt, tile offsets; nxt, move, M list
 //                (Jetrs: + 8n + 8T          evicted weight per vertex and per tile,
-//                 instead of the M list)
-//   rb_cookie    8n + 8T + 16|M|           evicted weight, tile offsets; part, nxt,
+//                 instead of the moves)
+//   rb_cookie    8n + 8T + 20|M|           evicted weight, tile offsets; part, nxt,
 //                                          move, M list
 // plus 8n (read P_iter, write P_best) in the kernel that copied the best
 // partition during this iteration (the afterburner for Jetlp, rb_scan for
@@ -452,7 +452,7 @@ __device__ __forceinline__ void iter_bytes(int64_t n, int64_t beta, int64_t T, i
         const int64_t w = q.nexam, X = q.nx, M = q.nm;
         b[JET_K_LP_SCAN] = 4 * n + 4 * q.nbnd + 4 * w;
         b[JET_K_LP_SELECT] = 24 * w + beta * q.degexam + 12 * X;
-        b[JET_K_AFTERBURN] = cp + (ab ? 32 * X + beta * q.degx : 4 * X) + 8 * M;
+        b[JET_K_AFTERBURN] = cp + (ab ? 32 * X + beta * q.degx + 12 * M : 4 * X + 16 * M);
         b[JET_K_APPLY] = 40 * M + beta * q.degm + 16 * k + 8 * X;
     } else {
         const bool rs = kind == MODE_RS;
@@ -461,8 +461,8 @@ __device__ __forceinline__ void iter_bytes(int64_t n, int64_t beta, int64_t T, i
         b[JET_K_RB_CAND] = (rs ? 28 : 32) * r + beta * q.degexam;
         b[JET_K_RB_TILEHIST] = 4 * n + 4 * c + 4 * tn;
         b[JET_K_RB_TILESCAN] = 8 * tn;
-        b[JET_K_RB_TAKE] = 4 * n + 4 * c + 4 * tn + (rs ? 8 * n + 8 * T : 8 * M);
-        if (rs) b[JET_K_RB_COOKIE] = 8 * n + 8 * T + 16 * M;
+        b[JET_K_RB_TAKE] = 4 * n + 4 * c + 4 * tn + (rs ? 8 * n + 8 * T : 16 * M);
+        if (rs) b[JET_K_RB_COOKIE] = 8 * n + 8 * T + 20 * M;
         b[JET_K_APPLY] = 36 * M + beta * q.degm + 16 * k;
     }
 }
