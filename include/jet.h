@@ -159,8 +159,9 @@ typedef struct {
     int64_t fin_edge_iters;    /* the same, finest level only */
     float ms_coarsen, ms_init, ms_refine, ms_refine_finest, ms_total;
     int64_t cut, max_part_w;
-    int64_t bytes_model;        /* algorithmic DRAM bytes of all refinement passes (byte model:
-                                   compulsory streams, neighbour gathers taken as cache hits) */
+    int64_t bytes_model;        /* algorithmic bytes of all refinement passes (byte model: compulsory
+                                   streams, neighbour gathers taken as cache hits); DRAM bytes, but on
+                                   levels that a cluster keeps in its shared memory most stay there */
     int64_t kernel_launches;    /* kernels executed by this call, device-loop iterations included */
     int64_t sel_launches[JET_MAX_LEVELS];  /* Jetlp select passes per level */
     int64_t sel_bytes[JET_MAX_LEVELS];     /* their algorithmic bytes, summed */
@@ -170,7 +171,7 @@ typedef struct {
     int32_t cluster_blocks[JET_MAX_LEVELS]; /* blocks of the thread-block cluster that ran the level's
                                                loop; 0 where the CUDA-graph or host loop ran it */
     /* per level and refinement kernel (JET_K_*): launches (0 where one cluster or cooperative launch
-     * ran the whole loop), algorithmic DRAM bytes (the byte model of bytes_model, split by kernel)
+     * ran the whole loop), algorithmic bytes (the byte model of bytes_model, split by kernel)
      * and, with JET_FLAG_PROFILE, the CUDA-event time of the kernel's launches */
     int64_t kern_launches[JET_MAX_LEVELS][JET_KERNELS];
     int64_t kern_bytes[JET_MAX_LEVELS][JET_KERNELS];

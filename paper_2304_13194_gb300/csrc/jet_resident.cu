@@ -1346,7 +1346,10 @@ __device__ __forceinline__ int64_t global_ns() {
     return (int64_t)t;
 }
 
-// The level's bytes by kernel (the byte model is linear in the sums).
+// The level's bytes by the kernel that does the same work in the other loops
+// (the byte model is linear in the sums).  They are the algorithm's traffic: here
+// most of it stays in shared memory.  Eviction has no tiles in this loop: nothing is
+// counted for them.
 __device__ __noinline__ void res_bytes(int64_t *kb) {
     const ResShared &s = rs();
     const ResView &v = s.v;
@@ -1354,13 +1357,14 @@ __device__ __noinline__ void res_bytes(int64_t *kb) {
 #pragma unroll 1
     for (int kind = 0; kind < 3; ++kind) {
         const unsigned long long *q = s.acc[kind];
-        const int64_t its = s.ctl.kcount[kind], T = (v.n + 1023) / 1024;
+        const int64_t its = s.ctl.kcount[kind];
         const bool lp = kind == MODE_LP;
         IterCounts c{lp ? (int64_t)q[kfNX] : 0, (int64_t)q[kfNM], (int64_t)q[kfDegx], (int64_t)q[kfDegm],
                      (int64_t)q[kfNbnd], (int64_t)q[kfNexam], (int64_t)q[kfDegexam], (int64_t)q[kfNcand],
-                     T * (int64_t)q[kPartFields], 8 * (int64_t)v.n * (int64_t)q[kPartFields + 1]};
+                     0, 8 * (int64_t)v.n * (int64_t)q[kPartFields + 1]};
         int64_t b[JET_K_COUNT];
-        iter_bytes(v.n * its, v.gew ? 8 : 4, T * its, v.k * its, v.abl, kind, c, b);
+        iter_bytes(v.n * its, v.gew ? 8 : 4, 0, v.k * its, v.abl, kind, c, b);
+        b[JET_K_RB_TILEHIST] = 0;
         for (int i = 0; i < JET_K_COUNT; ++i) kb[i] += b[i];
     }
 }

@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 jet = pytest.importorskip("paper_2304_13194_gb300")
 
 TILE = 256                                  # vertices per rebalancing tile of the CUDA-graph loop
-LOOPS = {"graph": {"cluster_max_n": 0}}
+LOOPS = {"graph": {"cluster_max_n": 0}, "resident": {}}
 
 
 def _run(g, k, eps, **opts):
