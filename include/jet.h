@@ -66,7 +66,8 @@ extern "C" {
                                       instead of the device-resident CUDA-graph loop */
 #define JET_FLAG_PROFILE 4u        /* implies JET_FLAG_HOSTLOOP; records a CUDA event before every
                                       refinement kernel launch and after the last of each iteration
-                                      (same kernels, same launch configuration) and fills
+                                      (the CUDA-graph loop's kernels and launch configuration, also
+                                      on levels that a cluster refines without this flag) and fills
                                       jet_stats.kern_ms and sel_ms */
 #define JET_FLAG_NO_LOCKS 16u      /* Jetlp ablations (Sec. 6.1.4, Table 2): ignore lock bits */
 #define JET_FLAG_NO_AFTERBURN 32u  /*   M = X (skip the second filter) */
