@@ -171,7 +171,6 @@ __global__ void __launch_bounds__(kTB) k_check_input(int32_t n, const int64_t *x
             out->sum_vw = vw ? (int64_t)atomicExch(&st->sum_vw, 0ull) : n;
             out->sum_ew = ew ? (int64_t)atomicExch(&st->sum_ew, 0ull) : (end > beg ? end - beg : 0);
             out->bad_part = (int64_t)atomicExch(&st->bad_part, 0ull);
-            out->bad = 0;
             out->nnz = end;
             st->ticket = 0;
         }

@@ -106,7 +106,7 @@ struct DGraph {
 // Outcome of the input checks, written into pinned host memory, and the
 // device state of the kernel that makes them (zero between its launches).
 struct CheckOut {
-    int64_t sum_vw, sum_ew, bad, bad_part, nnz;
+    int64_t sum_vw, sum_ew, bad_part, nnz;
 };
 struct CheckState {
     unsigned long long sum_vw, sum_ew, bad_part;

@@ -1051,13 +1051,14 @@ __device__ inline void ph_afterburn(const Level &L, LpExport ex, Grid G, char *a
 // Apply M (Alg. 3 updatePartsAndDS) and commit it: exact cut change, part
 // weights, neighbour counts ext, P_s[v] <- P_d[v]; Jetlp movers are locked
 // for the next Jetlp (Sec. 4.1.3) and the priorities of X go back to
-// kNoneGain.  A neighbour that moves too is recognised by its stamp and its
-// old part read from nxt, never from part[] (which the commit overwrites);
-// for an edge with both ends moving the smaller id accounts for the cut.
+// kNoneGain.  A neighbour's old and new part come from the word of its last
+// move, never from part[] (which the commit overwrites): this iteration's move
+// names both, an older one the part that the neighbour has and keeps.  For an
+// edge with both ends moving the smaller id accounts for the cut.
 // ---------------------------------------------------------------------------
 // Effect of v's move a -> b over the entries first, first + step, ... < end
-// of its row, batched as row_to_table: the stamps of a batch are loaded
-// together, then the move or the part of each neighbour, whichever it needs.
+// of its row, batched as row_to_table: the last moves of a batch of
+// neighbours are loaded together.
 // A neighbour that stays gets its ext[] updated; c receives the cut change
 // (an edge whose ends both move counts once, at the smaller id), ne the
 // neighbours in other parts after the move.

@@ -2,18 +2,19 @@
 // Jetrs (Sec. 4.2.2) and the driver of Alg. 3, for sm_103a.
 //
 // The passes themselves are device functions in jet_phases.cuh.  Levels that a
-// cluster's shared memory can hold are refined in jet_resident.cu; for the
-// others the passes run in one of two ways:
+// cluster's shared memory holds, and whose rows it walks fast enough, are
+// refined in jet_resident.cu; for the others the passes run in one of two ways:
 //  * large levels: one kernel per phase, and the whole level loop is a CUDA
 //    graph with a WHILE node around SWITCH nodes over {Jetlp, Jetrw, Jetrs}
 //    (two iterations per loop body); the controller, in the last block of
 //    the apply kernel, sets the conditionals, so no host round trip happens
 //    per iteration (the paper blames that round trip for its weaker
 //    coarse-level speedup, Sec. 6.2);
-//  * small levels whose state does not fit there (many parts): one thread
-//    block cluster (up to 16 SMs) runs every iteration of the level in a
-//    single launch on the state in global memory, the phases separated by the
-//    hardware cluster barrier — no launch or graph node per phase.
+//  * small levels (many parts, or dense): one thread block cluster (up to 16
+//    SMs) runs every iteration of the level in a single launch on the state in
+//    global memory, the phases separated by the hardware cluster barrier — no
+//    launch or graph node per phase.  The small graphs of a batch run the same
+//    loop, many clusters at once (k_refine_batch).
 #include "jet_phases.cuh"
 
 #include <cooperative_groups.h>

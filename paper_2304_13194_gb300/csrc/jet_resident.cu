@@ -142,7 +142,7 @@ __host__ __device__ inline uint32_t res_layout(ResView &v, int32_t n, int32_t S,
     v.oBig = take((uint32_t)S * 2);
     v.oAct = take((uint32_t)S * 2);
     v.oFlag = take((uint32_t)S);
-    v.oKey = take((uint32_t)S);      // key and D together also hold the Jetlp pass's third row class (2 S bytes)
+    v.oKey = take((uint32_t)S);
     v.oD = take((uint32_t)S * ptb);
     v.oPw = take((uint32_t)k * 4);
     v.oDelta = take((uint32_t)k * 8);
@@ -219,16 +219,15 @@ __device__ __forceinline__ int32_t own_vw(const ResView &v, int i) {
     return v.oVw != kNone ? arena_at<int32_t>(v.oVw)[i] : __ldg(v.gvw + i);
 }
 
-// Appends from any subset of a warp's lanes (all lanes call it); dir -1: the
-// list grows downwards.
+// Appends from any subset of a warp's lanes (all lanes call it).
 template <class T>
-__device__ __forceinline__ void append(int *cnt, T *list, bool pred, T x, int dir = 1) {
+__device__ __forceinline__ void append(int *cnt, T *list, bool pred, T x) {
     const unsigned m = __ballot_sync(0xffffffffu, pred);
     if (!m) return;
     int b = 0;
     if (lane_id() == 0) b = atomicAdd(cnt, __popc(m));
     b = __shfl_sync(0xffffffffu, b, 0);
-    if (pred) list[dir * (b + __popc(m & ((1u << lane_id()) - 1u)))] = x;
+    if (pred) list[b + __popc(m & ((1u << lane_id()) - 1u))] = x;
 }
 
 __device__ __forceinline__ void sum_to(uint32_t *dst, uint32_t x) {   // all lanes; one shared atomic per warp
