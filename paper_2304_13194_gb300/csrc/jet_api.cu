@@ -149,7 +149,8 @@ __device__ __forceinline__ void for_each_i32(const int32_t *p, int64_t count, F 
 // one thread walked each row and the longest row set the time).  The last
 // block hands the outcome to the host and clears the state.
 __global__ void __launch_bounds__(kTB) k_check_input(int32_t n, const int64_t *xadj, const int32_t *vw, const int32_t *ew,
-                                                     const int32_t *part, int32_t k, CheckState *st, CheckOut *out) {
+                                                     const int32_t *part, int32_t k, int rows, CheckState *st,
+                                                     CheckOut *out) {
     __shared__ long long sh[40];
     __shared__ int s_last;
     const int64_t beg = xadj[0], end = xadj[n];
@@ -157,6 +158,13 @@ __global__ void __launch_bounds__(kTB) k_check_input(int32_t n, const int64_t *x
     if (vw) for_each_i32(vw, n, [&](int32_t x) { svw += x; });
     if (ew && beg >= 0 && end > beg) for_each_i32(ew + beg, end - beg, [&](int32_t x) { sew += x; });
     if (part) for_each_i32(part, n, [&](int32_t x) { bad |= x < 0 || x >= k; });
+    if (rows) {   // the longest row (small graphs only; one atomic per warp)
+        int32_t d = 0;
+        for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
+            d = max(d, (int32_t)min(xadj[v + 1] - xadj[v], (int64_t)INT32_MAX));
+        d = __reduce_max_sync(0xffffffffu, d);
+        if (lane_id() == 0 && d > 0) atomicMax(&st->longest, d);
+    }
     svw = block_sum_i64(svw, sh);
     sew = block_sum_i64(sew, sh);
     bad = block_sum_i64(bad, sh);
@@ -172,6 +180,7 @@ __global__ void __launch_bounds__(kTB) k_check_input(int32_t n, const int64_t *x
             out->sum_ew = ew ? (int64_t)atomicExch(&st->sum_ew, 0ull) : (end > beg ? end - beg : 0);
             out->bad_part = (int64_t)atomicExch(&st->bad_part, 0ull);
             out->nnz = end;
+            out->longest = atomicExch(&st->longest, 0);
             st->ticket = 0;
         }
     }
@@ -182,11 +191,11 @@ __global__ void k_ones32(int32_t *p, int64_t n) {
 }
 
 int check_input(Ctx &c, int32_t n, const int64_t *xadj, const int32_t *adjncy, const int32_t *vwgt, const int32_t *adjwgt,
-                const int32_t *part, int32_t k, CheckOut &out) {
+                const int32_t *part, int32_t k, CheckOut &out, bool rows) {
     cudaStream_t s = c.stream;
     // four 16-byte loads a thread and pass; the entry count is not known here
-    const int blocks = adjwgt ? num_sms() * 8 : std::min(num_sms() * 8, grid_for(n, kTB * 16));
-    k_check_input<<<blocks, kTB, 0, s>>>(n, xadj, vwgt, adjwgt, part, k, c.check.as<CheckState>(),
+    const int blocks = adjwgt ? num_sms() * 8 : std::min(num_sms() * 8, grid_for(n, rows ? kTB * 2 : kTB * 16));
+    k_check_input<<<blocks, kTB, 0, s>>>(n, xadj, vwgt, adjwgt, part, k, rows ? 1 : 0, c.check.as<CheckState>(),
                                            reinterpret_cast<CheckOut *>(c.pinned));
     JET_CUDA_TRY(cudaGetLastError());
     JET_CUDA_TRY(cudaStreamSynchronize(s));
@@ -201,11 +210,12 @@ int check_input(Ctx &c, int32_t n, const int64_t *xadj, const int32_t *adjncy, c
 // into `ones` when vwgt is NULL.
 int prepare_graph(Ctx &c, int32_t n, const int64_t *xadj, const int32_t *adjncy, const int32_t *vwgt,
                   const int32_t *adjwgt, DGraph &g, DevBuf &ones, bool need_vw, bool check_part, const int32_t *part,
-                  int32_t k, int64_t *W) {
+                  int32_t k, int64_t *W, int64_t *longest) {
     if (n < 0 || !xadj) return JET_EINVAL;
     cudaStream_t s = c.stream;
     CheckOut h;
-    JET_TRY(check_input(c, n, xadj, adjncy, vwgt, adjwgt, check_part ? part : nullptr, k, h));
+    const bool rows = longest && n <= kHemClusterN;
+    JET_TRY(check_input(c, n, xadj, adjncy, vwgt, adjwgt, check_part ? part : nullptr, k, h, rows));
     if (c.opt.flags & JET_FLAG_VALIDATE) {
         DevBuf cb;
         JET_TRY(dev_alloc(cb, 16, s));
@@ -221,6 +231,7 @@ int prepare_graph(Ctx &c, int32_t n, const int64_t *xadj, const int32_t *adjncy,
     if (h.sum_vw >= (1LL << 31) || h.sum_ew >= (1LL << 31)) return JET_EOVERFLOW;
     if (check_part && n > 0 && (!part || h.bad_part)) return JET_EINVAL;
     if (W) *W = h.sum_vw;
+    if (longest) *longest = rows ? h.longest : -1;
     g.n = n;
     g.nnz = h.nnz;
     g.xadj = xadj;
@@ -552,12 +563,13 @@ int jet_coarsen(jet_ctx *ctx, int32_t n, const int64_t *xadj, const int32_t *adj
     JET_TRY(use_device(c));
     DGraph g;
     DevBuf ones;
-    int64_t W = 0;
-    JET_TRY(prepare_graph(c, n, xadj, adjncy, vwgt, adjwgt, g, ones, false, false, nullptr, 0, &W));
+    int64_t W = 0, longest = -1;
+    JET_TRY(prepare_graph(c, n, xadj, adjncy, vwgt, adjwgt, g, ones, false, false, nullptr, 0, &W, &longest));
     jet_hier *h = new (std::nothrow) jet_hier;
     if (!h) return JET_ENOMEM;
     h->ctx = ctx;
     h->W = W;
+    h->longest0 = longest;
     EventTimer ev;
     cudaEventRecord(ev.e[0], c.stream);
     int64_t l0 = c.launches;
@@ -1043,8 +1055,9 @@ int jet_hem(jet_ctx *ctx, int32_t n, const int64_t *xadj, const int32_t *adjncy,
     JET_TRY(use_device(c));
     DGraph g;
     DevBuf ones;
-    JET_TRY(prepare_graph(c, n, xadj, adjncy, nullptr, adjwgt, g, ones, false));
-    JET_TRY(hem(c, g, seed, level, rounds, mate_out));
+    int64_t longest = -1;
+    JET_TRY(prepare_graph(c, n, xadj, adjncy, nullptr, adjwgt, g, ones, false, false, nullptr, 0, nullptr, &longest));
+    JET_TRY(hem(c, g, longest, seed, level, rounds, mate_out));
     return sync_stream(c);
 }
 

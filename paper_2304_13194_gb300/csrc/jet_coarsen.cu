@@ -120,17 +120,21 @@ __device__ __forceinline__ void hem_block_best(HemBest &best, HemBest *sh) {
 // memory; a round is: the block's unmatched vertices are listed, groups of lanes
 // scan their rows against the local bits, one cluster barrier, mutual proposals
 // match, one cluster barrier, and every block copies the other blocks' bits.
-// Rows longer than kHemLong are scanned by the whole block.  Ends with the first
-// round that matches nothing, as the launched form does.  Whole calls, launched form
-// against this one: 4,096 vertices of degree 6 100 -> 79 us, 15,625 107 -> 87,
-// 32,768 111 -> 105, 40,000 no gain; 4,000 of degree 32 125 -> 155, R-MAT s12
-// 152 -> 279 (rows too long for one cluster), hence kHemClusterN and kHemClusterDeg.
+// Ends with the first round that matches nothing, as the launched form does.  Whole
+// calls, launched form against this one: 4,096 vertices of degree 6 100 -> 79 us,
+// 15,625 107 -> 87, 32,768 111 -> 105, 40,000 no gain; 4,000 of degree 32 125 -> 155,
+// hence kHemClusterN and kHemClusterDeg.  A lane group takes a row whole, so that one
+// long row holds a round up: R-MAT of two entries per vertex, scale 12 (longest row
+// 367) 228 -> 516, scale 15 (1,431) 281 -> 708 against the rounds before both forms;
+// with rows of up to 127 entries nothing lost (R-MAT s11, 2,048 vertices 1.29 times as
+// fast), hence kHemClusterRow; and 32,768 vertices with 459,000 entries 253 -> 261,
+// with 328,000 1.1 times as fast, hence kHemClusterNnz.
 constexpr int kHemThreads = 1024;
 constexpr int kHemSlice = 2048;             // vertices per block at most
 constexpr int kHemCluster = 16;
-constexpr int kHemLong = 512;
 constexpr int kHemClusterDeg = 16;          // entries per vertex at most, on average
-constexpr int32_t kHemClusterN = 32768;     // kHemSlice * kHemCluster
+constexpr int kHemClusterRow = 128;         // entries of a row at most
+constexpr int64_t kHemClusterNnz = 400000;  // entries at most
 static_assert(kHemClusterN == kHemSlice * kHemCluster, "slices cover the largest level");
 
 __device__ __forceinline__ void hem_cluster_sync() {
@@ -142,9 +146,8 @@ __global__ void __launch_bounds__(kHemThreads) k_hem_cluster(DGraph g, int32_t p
                                                              uint64_t salt0, int32_t *mate, int32_t *prop) {
     __shared__ uint32_t bits[kHemClusterN / 32];     // matched, all vertices
     __shared__ uint32_t own[kHemSlice / 32];         // matched, this block's slice (read by the others)
-    __shared__ int32_t act[kHemSlice];               // unmatched vertices: short rows from the front, long from the back
-    __shared__ int s_short, s_long;
-    __shared__ HemBest sh[kHemThreads / 32];
+    __shared__ int32_t act[kHemSlice];               // unmatched vertices
+    __shared__ int s_act;
     pdl_enter();
     const int tid = threadIdx.x, n = g.n;
     const int v0 = (int)blockIdx.x * per, nv = max(0, min(per, n - v0));
@@ -152,7 +155,7 @@ __global__ void __launch_bounds__(kHemThreads) k_hem_cluster(DGraph g, int32_t p
     for (int i = tid; i < words; i += kHemThreads) bits[i] = 0;
     for (int i = tid; i < wper; i += kHemThreads) own[i] = 0;
     for (int i = tid; i < nv; i += kHemThreads) mate[v0 + i] = -1;
-    if (tid == 0) { s_short = 0; s_long = 0; }
+    if (tid == 0) s_act = 0;
     __syncthreads();
     const int groups = kHemThreads / lanes, gi = tid / lanes, gl = tid & (lanes - 1);
     for (int r = 0; r < rounds; ++r) {
@@ -160,14 +163,11 @@ __global__ void __launch_bounds__(kHemThreads) k_hem_cluster(DGraph g, int32_t p
         for (int i0 = 0; i0 < nv; i0 += kHemThreads) {
             const int i = i0 + tid;
             const bool active = i < nv && !(own[i >> 5] >> (i & 31) & 1u);
-            const bool lng = active && g.xadj[v0 + i + 1] - g.xadj[v0 + i] > kHemLong;
-            int slot = warp_append(&s_short, active && !lng);
-            if (active && !lng) act[slot] = v0 + i;
-            slot = warp_append(&s_long, lng);
-            if (lng) act[kHemSlice - 1 - slot] = v0 + i;
+            const int slot = warp_append(&s_act, active);
+            if (active) act[slot] = v0 + i;
         }
         __syncthreads();
-        const int ns = s_short, nl = s_long;
+        const int ns = s_act;
         for (int a0 = 0; a0 < ns; a0 += groups) {
             const int a = a0 + gi;
             const int32_t v = a < ns ? act[a] : -1;
@@ -176,24 +176,17 @@ __global__ void __launch_bounds__(kHemThreads) k_hem_cluster(DGraph g, int32_t p
             best.reduce(lanes);
             if (v >= 0 && gl == 0) prop[v] = best.u;
         }
-        for (int a = 0; a < nl; ++a) {
-            const int32_t v = act[kHemSlice - 1 - a];
-            HemBest best;
-            hem_row<EW>(g, bits, seed, salt, g.xadj[v] + tid, g.xadj[v + 1], kHemThreads, best);
-            hem_block_best(best, sh);
-            if (tid == 0) prop[v] = best.u;
-        }
         hem_cluster_sync();
         // every proposal names a vertex that was unmatched, so whose proposal is this round's
-        for (int a = tid; a < ns + nl; a += kHemThreads) {
-            const int32_t v = act[a < ns ? a : kHemSlice - 1 - (a - ns)];
+        for (int a = tid; a < ns; a += kHemThreads) {
+            const int32_t v = act[a];
             const int32_t u = __ldcg(prop + v);
             if (u >= 0 && __ldcg(prop + u) == v) {
                 mate[v] = u;
                 atomicOr(&own[(v - v0) >> 5], 1u << ((v - v0) & 31));
             }
         }
-        if (tid == 0) { s_short = 0; s_long = 0; }
+        if (tid == 0) s_act = 0;
         hem_cluster_sync();
         int changed = 0;
         for (int i = tid; i < words; i += kHemThreads) {
@@ -333,14 +326,16 @@ __global__ void __launch_bounds__(kTB) k_hem_match(int32_t n, int32_t *mate, uin
     if (threadIdx.x == 0 && c) atomic_add_i64(&hc->added[r], c);
 }
 
-int hem(Ctx &c, const DGraph &g, uint64_t seed, int32_t level, int32_t rounds, int32_t *mate) {
+int hem(Ctx &c, const DGraph &g, int64_t longest, uint64_t seed, int32_t level, int32_t rounds, int32_t *mate) {
     cudaStream_t s = c.stream;
     if (g.n == 0) return JET_OK;
     rounds = std::min(rounds, 64);
     const bool pdl = !(c.opt.flags & JET_FLAG_NO_PDL);
     const uint64_t salt0 = 0xD1B54A32D192ED03ULL * (uint64_t)(64 * (int64_t)level);
     DevBuf buf;
-    const int cs = g.n <= kHemClusterN && g.nnz <= (int64_t)kHemClusterDeg * g.n ? hem_cluster_blocks(c.device) : 0;
+    const bool small = g.n <= kHemClusterN && g.nnz <= std::min(kHemClusterNnz, (int64_t)kHemClusterDeg * g.n) &&
+                       longest >= 0 && longest <= kHemClusterRow;
+    const int cs = small ? hem_cluster_blocks(c.device) : 0;
     if (cs > 0 && g.n <= cs * kHemSlice) {
         JET_TRY(dev_alloc(buf, (size_t)g.n * 4, s));
         int32_t *prop = buf.as<int32_t>();
@@ -466,6 +461,7 @@ struct LevelCount {
     int64_t btotal;        // entries of all rows before merging
     int64_t htotal, nhub;  // entries and number of the hub rows
     int32_t rows[4];       // {warp rows, block rows, 16-entry thread rows, 32-entry thread rows}
+    int32_t longest, pad;  // entries of the longest row before merging (up to kHemClusterN rows)
 };
 
 // The coarse rows sorted into classes by their bound (entries of the merged fine
@@ -484,6 +480,10 @@ __global__ void __launch_bounds__(kTB) k_row_classes(int32_t n, const int64_t *b
         if (threadIdx.x < 4) cnt[threadIdx.x] = 0;
         __syncthreads();
         const int64_t b = c < nc ? boff[c + 1] - boff[c] : -1;
+        if (nc <= kHemClusterN) {   // the next level's matching asks for it
+            const int32_t most = __reduce_max_sync(0xffffffffu, (int32_t)b);
+            if (lane_id() == 0 && most > 0) atomicMax(&lc->longest, most);
+        }
         const int cls = b < 0 ? -1 : b <= 16 ? 2 : b <= 32 ? 3 : b <= kWarpSort ? 0 : 1;
         int slot[4];
 #pragma unroll
@@ -916,13 +916,14 @@ __global__ void k_copy_rows(int32_t nc, const int64_t *boff, const int64_t *xadj
     }
 }
 
-// One coarsening level: matching, map, contraction.  Returns JET_OK and sets
+// One coarsening level: matching, map, contraction.  longest: the level's longest
+// row (-1: not known), then a bound on the coarse level's.  Returns JET_OK and sets
 // stalled=true (without building the level) when n_c > 0.95 n.  Small levels are
 // bound by launches and host waits: the row classes are made before the host
 // knows the number of coarse vertices, so that it waits twice per level, for the
 // sizes of the work and of the result, and empty classes are not launched (564
 // launches, four waits and 2.9 ms for the 12 levels of a 110,592-vertex mesh before).
-static int coarsen_level(Ctx &c, const DGraph &g, uint64_t seed, int32_t level, jet_hier *h, bool &stalled) {
+static int coarsen_level(Ctx &c, const DGraph &g, int64_t &longest, uint64_t seed, int32_t level, jet_hier *h, bool &stalled) {
     cudaStream_t s = c.stream;
     stalled = false;
     const int64_t n = g.n;
@@ -942,7 +943,7 @@ static int coarsen_level(Ctx &c, const DGraph &g, uint64_t seed, int32_t level, 
     JET_TRY(dev_alloc(cmapb, nn * 4, s));   // owned by the hierarchy
     int32_t *cmap = cmapb.as<int32_t>();
     JET_CUDA_TRY(cudaMemsetAsync(lc, 0, sizeof(LevelCount), s));
-    JET_TRY(hem(c, g, seed, level, c.opt.hem_rounds, mate));
+    JET_TRY(hem(c, g, longest, seed, level, c.opt.hem_rounds, mate));
     if (c.opt.flags & JET_FLAG_TWO_HOP) {
         int64_t added[3];
         JET_TRY(two_hop(c, g, mate, added));
@@ -959,6 +960,7 @@ static int coarsen_level(Ctx &c, const DGraph &g, uint64_t seed, int32_t level, 
     LevelCount hc;
     memcpy(&hc, c.pinned, sizeof(hc));
     const int64_t nc = hc.nc;
+    longest = hc.longest;
     if (100 * nc > 95 * n) { stalled = true; return JET_OK; }
     const size_t ncl = (size_t)std::max<int64_t>(nc, 1);
     // merged rows
@@ -1076,12 +1078,13 @@ int coarsen(Ctx &c, const DGraph &g0, int32_t k, uint64_t seed, jet_hier *h) {
     }
     int32_t T = c.opt.coarsen_target > 0 ? c.opt.coarsen_target : std::max(8 * k, 256);
     int32_t maxl = std::min<int32_t>(c.opt.max_levels, JET_MAX_LEVELS);
+    int64_t longest = h->longest0;
     while (h->n[h->levels - 1] > T && h->levels < maxl) {
         int32_t i = h->levels - 1;
         DGraph gi;
         gi.n = h->n[i]; gi.nnz = h->nnz[i]; gi.xadj = h->xadj[i]; gi.adj = h->adj[i]; gi.vw = h->vw[i]; gi.ew = h->ew[i];
         bool stalled = false;
-        JET_TRY(coarsen_level(c, gi, seed, i, h, stalled));
+        JET_TRY(coarsen_level(c, gi, longest, seed, i, h, stalled));
         if (stalled) break;
     }
     return JET_OK;

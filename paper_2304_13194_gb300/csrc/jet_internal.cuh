@@ -106,11 +106,12 @@ struct DGraph {
 // Outcome of the input checks, written into pinned host memory, and the
 // device state of the kernel that makes them (zero between its launches).
 struct CheckOut {
-    int64_t sum_vw, sum_ew, bad_part, nnz;
+    int64_t sum_vw, sum_ew, bad_part, nnz, longest;   // longest row, where it was asked for
 };
 struct CheckState {
     unsigned long long sum_vw, sum_ew, bad_part;
-    uint32_t ticket, pad;
+    uint32_t ticket;
+    int32_t longest;
 };
 
 // ---------------------------------------------------------------------------
@@ -556,6 +557,7 @@ struct jet_hier {
     int64_t W = 0;            // total vertex weight (every level's)
     int32_t n[JET_MAX_LEVELS] = {};
     int64_t nnz[JET_MAX_LEVELS] = {};
+    int64_t longest0 = -1;    // longest row of level 0 (-1: not known)
     const int64_t *xadj[JET_MAX_LEVELS] = {};
     const int32_t *adj[JET_MAX_LEVELS] = {};
     const int32_t *vw[JET_MAX_LEVELS] = {};
@@ -647,7 +649,9 @@ int rebalance_pass(Ctx &c, const DGraph &g, int64_t W, int32_t k, double eps, in
 int cut_and_weights(Ctx &c, const DGraph &g, int32_t k, const int32_t *part, int64_t *cut_out, int64_t *pw_dev);
 
 // jet_coarsen.cu
-int hem(Ctx &c, const DGraph &g, uint64_t seed, int32_t level, int32_t rounds, int32_t *mate);
+constexpr int32_t kHemClusterN = 32768;     // largest level that one cluster may match
+// longest: entries of the longest row or a bound on them (-1: not known).
+int hem(Ctx &c, const DGraph &g, int64_t longest, uint64_t seed, int32_t level, int32_t rounds, int32_t *mate);
 int coarsen(Ctx &c, const DGraph &g0, int32_t k, uint64_t seed, jet_hier *h);
 // The greedy order behind the initial partition (component, BFS distance,
 // id), for the learned initial partition's features and labels.  Device
@@ -686,15 +690,17 @@ int64_t balance_limit(int64_t W, int32_t k, double eps, int64_t *opt);
 int sync_stream(Ctx &c);
 int use_device(Ctx &c);
 bool bad_k_eps(int32_t k, double eps);
-// Weight sums, entry count and (part not null) the part range of an input in
-// one launch and one host wait; JET_OK when the sums could be taken.
+// Weight sums, entry count, (part not null) the part range and (rows) the longest
+// row of an input in one launch and one host wait; JET_OK when the sums could be taken.
 int check_input(Ctx &c, int32_t n, const int64_t *xadj, const int32_t *adjncy, const int32_t *vwgt, const int32_t *adjwgt,
-                const int32_t *part, int32_t k, CheckOut &out);
+                const int32_t *part, int32_t k, CheckOut &out, bool rows = false);
 // Argument and overflow checks; fills g (W: the total vertex weight).  With
-// check_part also JET_EINVAL unless every part is in [0, k).
+// check_part also JET_EINVAL unless every part is in [0, k).  longest: the longest
+// row where one cluster may match the graph, else -1.
 int prepare_graph(Ctx &c, int32_t n, const int64_t *xadj, const int32_t *adjncy, const int32_t *vwgt,
                   const int32_t *adjwgt, DGraph &g, DevBuf &ones, bool need_vw, bool check_part = false,
-                  const int32_t *part = nullptr, int32_t k = 0, int64_t *W = nullptr);
+                  const int32_t *part = nullptr, int32_t k = 0, int64_t *W = nullptr,
+                  int64_t *longest = nullptr);
 // Alg. 1 after coarsening; init_coarsest (device, n of the coarsest level)
 // replaces the greedy initial partition when not null.
 int uncoarsen(Ctx &c, const jet_hier *h, int32_t k, double eps, uint64_t seed, const int32_t *init_coarsest,
