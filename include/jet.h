@@ -105,7 +105,8 @@ extern "C" {
  *                                   34,400 at 256, 21,400 at 257, 4,300 at 480, 500 at 530.
  *                                   Larger levels, and those with more CSR entries than one cluster
  *                                   walks as fast as the whole GPU (480,000 / (1 + k / 160), less for
- *                                   many parts on up to 8,192 vertices), use the CUDA-graph loop;
+ *                                   many parts on up to 8,192 vertices, twice that on sparse levels
+ *                                   whose contraction merges entries), use the CUDA-graph loop;
  *                                   0 = never.  Levels of up to 4096 vertices (with any other value
  *                                   than the default: of up to that many) run in one cluster launch
  *                                   on their state in global memory where the first form is not used

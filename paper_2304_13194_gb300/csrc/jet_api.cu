@@ -336,6 +336,8 @@ int uncoarsen(Ctx &c, const jet_hier *h, int32_t k, double eps, uint64_t seed, c
         }
     } runs;
     runs.s = s;
+    // entries that contraction left of level i's (the coarsest level: all; a level by itself: not known)
+    auto merged = [&](int32_t i) -> int64_t { return l == 0 ? -1 : h->nnz[i < l ? i + 1 : l]; };
     // the coarse levels that a cluster can hold: one launch for the whole
     // chain, from the coarsest to level `chain_end`
     int32_t next = l;                      // coarsest level not in the chain
@@ -343,7 +345,7 @@ int uncoarsen(Ctx &c, const jet_hier *h, int32_t k, double eps, uint64_t seed, c
     if (!(c.opt.flags & (JET_FLAG_HOSTLOOP | JET_FLAG_PROFILE))) {
         for (int32_t i = l; i >= 0; --i) {
             int cs = 0;
-            JET_TRY(resident_cluster(c, h->n[i], h->nnz[i], k, &cs));
+            JET_TRY(resident_cluster(c, h->n[i], h->nnz[i], merged(i), k, &cs));
             if (cs == 0) break;
             chain_cs = std::max(chain_cs, cs);
             chain_end = i;
@@ -391,6 +393,7 @@ int uncoarsen(Ctx &c, const jet_hier *h, int32_t k, double eps, uint64_t seed, c
         LevelRun &run = runs.r[i];
         run.slot = i;
         run.want_trace = i == 0;
+        run.nnz_coarser = merged(i);
         runs.lo = std::min(runs.lo, i);
         runs.hi = std::max(runs.hi, i);
         JET_TRY(refine_level_enqueue(c, g, k, eps, i == 0, level_seed(seed, i), cur, W, run));
@@ -735,7 +738,7 @@ static bool queue_small_graphs(Ctx &c, int32_t count, const jet_batch_item *item
         const jet_batch_item &it = items[i];
         if (it.n <= 0 || it.n > std::min(kClusterLoopMaxN, c.opt.cluster_max_n)) continue;
         int cs = 0;
-        *status = resident_cluster(c, it.n, 0, it.k, &cs);   // entries are not known here
+        *status = resident_cluster(c, it.n, 0, -1, it.k, &cs);   // entries are not known here
         if (*status < 0) return false;
         // graphs that a worker partitions in the time of one launch
         const double graphs = cs == 0 ? 3.0 : std::max(3.9, std::min(12.0, 12.0 * 64 / it.k));

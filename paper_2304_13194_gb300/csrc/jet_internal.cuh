@@ -583,6 +583,7 @@ struct LevelRun {
     DGraph g;
     int32_t k = 0;
     int32_t cluster = 0, grid = 0, hostloop = 0;
+    int64_t nnz_coarser = -1;         // entries of the next coarser level (resident_cluster)
     int32_t resident = 0;             // blocks of the cluster whose resident chain runs the level (0: none)
     int nk_branch[3] = {0, 0, 0}, nk_tail = 0;
     cudaGraphExec_t exec = nullptr;   // the level's CUDA-graph loop (destroyed by refine_level_finish)
@@ -604,8 +605,9 @@ struct ResChainLevel {
     bool is_finest = false;
 };
 // Blocks of the cluster that keeps a level of n vertices and nnz entries (0: it
-// does not fit, another loop is faster, or the options exclude it).
-int resident_cluster(Ctx &c, int64_t n, int64_t nnz, int32_t k, int *cs);
+// does not fit, another loop is faster, or the options exclude it).  nnz_coarser:
+// entries of the next coarser level (the level's own on the coarsest one; -1: a level by itself).
+int resident_cluster(Ctx &c, int64_t n, int64_t nnz, int64_t nnz_coarser, int32_t k, int *cs);
 // Enqueues the chain (no host wait); init: the partition its first level
 // starts from.  Outcomes are read by refine_level_finish.
 int resident_enqueue(Ctx &c, const ResChainLevel *lv, int32_t nlv, int32_t k, double eps, int64_t W, int cs,

@@ -1209,7 +1209,7 @@ int refine_level_enqueue(Ctx &c, const DGraph &g, int32_t k, double eps, int32_t
     run.k = k;
     if (run.slot < 0 || run.slot >= JET_MAX_LEVELS) return JET_EINVAL;
     run.hostloop = (c.opt.flags & (JET_FLAG_HOSTLOOP | JET_FLAG_PROFILE)) != 0;
-    if (!run.hostloop) JET_TRY(resident_cluster(c, g.n, g.nnz, k, &run.resident));
+    if (!run.hostloop) JET_TRY(resident_cluster(c, g.n, g.nnz, run.nnz_coarser, k, &run.resident));
     if (run.resident > 0) {
         ResChainLevel lv;
         lv.g = g;

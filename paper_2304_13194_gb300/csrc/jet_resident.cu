@@ -1475,8 +1475,18 @@ int device_info(int device, int32_t k, ResDevice &out) {
 // n = 48,000, 335,000 entries 1.06, 479,000 0.84; n = 60,000, 299,000 1.11,
 // 659,000 0.60; k = 128: n = 48,000, 239,000 1.14, 335,000 0.88; k = 256:
 // n = 24,000, 191,000 1.04, 287,000 0.85; R-MAT s15 (883,000), k = 256: 0.51.
-// Meshes and geometric graphs gain further on (k = 64: 1.9 at n = 60,000 and
-// 477,000 entries), but their sizes do not tell them apart.
+// Meshes and geometric graphs gain further on.  Inside a hierarchy they are told
+// apart by the next coarser level: where the neighbours of a matched pair are
+// neighbours of each other, contraction merges their entries, and it keeps 0.4 to
+// 0.8 of them (random graphs, R-MAT and levels that stall keep 0.85 to 1).  Such
+// levels of up to 16 entries per vertex may have twice as many (graph loop / this
+// one): weighted 48^3 mesh, n = 59,800, 504,000 entries, k = 64 1.28; 80^3, n =
+// 46,000, 591,000, k = 31 1.28; 60^3, n = 63,300, 671,000, k = 8 1.39; geometric
+// of degree 12, n = 60,000, 714,000, k = 31 1.71; 15 to 20 entries per vertex,
+// 632,000 k = 64 1.72.  Levels of up to 8,192 vertices of any hierarchy gain up to
+// about 400,000 entries whatever k <= 256 is, since the partition they start from is
+// a refined one: means over R-MAT and random graphs of 350,000 to 400,000 entries 1.1
+// (k = 2) to 2.4 (k = 64) at n <= 4,096, 1.1 to 1.8 up to 8,192.
 // Up to 8,192 vertices 512 threads a block walk the rows: n = 8,000, k = 8,
 // 342,000 entries 1.11, 398,000 0.93; n = 6,000, k = 192: 149,000 1.01,
 // 197,000 0.87; k = 256: 59,000 1.11, 149,000 0.94; k = 384: 29,000 1.05,
@@ -1484,11 +1494,15 @@ int device_info(int device, int32_t k, ResDevice &out) {
 // 147,000 1.02, 198,000 0.98; k = 384: 99,000 1.13, 147,000 0.94; k = 480:
 // 59,000 1.03, 147,000 0.86; above 400,000 entries this loop does not gain on it,
 // nor on longer rows with few blocks (n = 1,000, k = 64: 258,000 1.05, 322,000 0.97).
-int64_t res_entry_limit(int64_t n, int32_t k) {
+int64_t res_entry_limit(int64_t n, int64_t nnz, int64_t nnz_coarser, int32_t k) {
     const int64_t wide = 76800000 / (160 + k);       // 480,000 / (1 + k / 160)
-    if (n > 8192) return wide;
-    if (n > 4096) return std::min<int64_t>({350000, wide, 5000000000 / ((int64_t)k * k)});
-    return std::min<int64_t>({400000, 280 * n, 40000000 / k});
+    int64_t most;
+    if (n > 8192) most = wide;
+    else if (nnz_coarser >= 0 && k <= 256) most = std::min<int64_t>(400000, 280 * n);
+    else if (n > 4096) most = std::min<int64_t>({350000, wide, 5000000000 / ((int64_t)k * k)});
+    else most = std::min<int64_t>({400000, 280 * n, 40000000 / k});
+    const bool local = nnz_coarser >= 0 && 10 * nnz_coarser <= 8 * nnz && nnz <= 16 * n;
+    return local ? 2 * most : most;
 }
 
 bool res_fits(int64_t n, int32_t k, int cs, uint32_t arena) {
@@ -1501,11 +1515,13 @@ bool res_fits(int64_t n, int32_t k, int cs, uint32_t arena) {
 
 }  // namespace
 
-int resident_cluster(Ctx &c, int64_t n, int64_t nnz, int32_t k, int *cs) {
+int resident_cluster(Ctx &c, int64_t n, int64_t nnz, int64_t nnz_coarser, int32_t k, int *cs) {
     *cs = 0;
     const int want = c.opt.cluster_blocks;
     // fewer blocks by choice: fewer entries (a small level's few blocks are enough for its rows)
-    if (n <= 0 || n > c.opt.cluster_max_n || nnz > res_entry_limit(n, k) * (want > 0 ? want : 16) / 16) return JET_OK;
+    if (n <= 0 || n > c.opt.cluster_max_n ||
+        nnz > res_entry_limit(n, nnz, nnz_coarser, k) * (want > 0 ? want : 16) / 16)
+        return JET_OK;
     ResDevice d;
     JET_TRY(device_info(c.device, k, d));
     if (want > 0) {

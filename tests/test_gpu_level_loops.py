@@ -180,3 +180,24 @@ def test_levels_on_both_sides_of_the_threshold():
         assert [b > 0 for b in st.cluster_blocks] == small
         cuts.append(cut)
     assert cuts[0] == cuts[1]
+
+
+@pytest.mark.parametrize("name,make,k,cluster", [
+    ("mesh", lambda: graphgen.grid3d(48, 48, 48, vw=(1, 4), ew=(1, 10), seed=4), 64, True),       # 59,783 vertices
+    ("geometric", lambda: graphgen.rgg(60000, seed=2), 64, True),
+    ("random", lambda: _random_graph(60000, 480000, 9), 64, False),
+], ids=["mesh", "geometric", "random"])
+def test_levels_whose_contraction_merges_entries_stay_longer(name, make, k, cluster):
+    """Beyond the line for levels without locality, a level of 50,000 to 65,536
+    vertices stays in the resident loop where the next coarser level has at most
+    0.8 of its entries; the partition is the graph loop's."""
+    g = make()
+    t = _dev(g, name == "geometric")
+    with jet.Context(0) as a, jet.Context(0, cluster_max_n=0) as b:
+        pa, ca, st = a.partition(*t, k=k, seed=2, return_stats=True)
+        pb, cb = b.partition(*t, k=k, seed=2)
+    assert ca == cb and torch.equal(pa, pb)
+    i = next(i for i, n in enumerate(st.n) if n <= 65536)
+    assert 50000 <= st.n[i] and 2 * st.m[i] > 76800000 // (160 + k) and 2 * st.m[i] <= 16 * st.n[i]
+    assert (10 * st.m[i + 1] <= 8 * st.m[i]) == cluster
+    assert (st.cluster_blocks[i] > 0) == cluster
