@@ -1482,8 +1482,10 @@ int device_info(int device, int32_t k, ResDevice &out) {
 // levels of up to 16 entries per vertex may have twice as many (graph loop / this
 // one): weighted 48^3 mesh, n = 59,800, 504,000 entries, k = 64 1.28; 80^3, n =
 // 46,000, 591,000, k = 31 1.28; 60^3, n = 63,300, 671,000, k = 8 1.39; geometric
-// of degree 12, n = 60,000, 714,000, k = 31 1.71; 15 to 20 entries per vertex,
-// 632,000 k = 64 1.72.  Levels of up to 8,192 vertices of any hierarchy gain up to
+// of degree 12, n = 60,000, 714,000, k = 31 1.71; of degree 16, n = 40,000, 632,000,
+// k = 64 1.72.  So may denser ones (400,000 entries where there are more than 40 per
+// vertex) of which 0.65 is left: R-MAT s17 with two-hop matches, n = 8,400, 397,000,
+// k = 64 1.9; between 0.65 and 0.8 such levels lose at times (0.81 to 1.5).  Levels of up to 8,192 vertices of any hierarchy gain up to
 // about 400,000 entries whatever k <= 256 is, since the partition they start from is
 // a refined one: means over R-MAT and random graphs of 350,000 to 400,000 entries 1.1
 // (k = 2) to 2.4 (k = 64) at n <= 4,096, 1.1 to 1.8 up to 8,192.
@@ -1501,7 +1503,8 @@ int64_t res_entry_limit(int64_t n, int64_t nnz, int64_t nnz_coarser, int32_t k) 
     else if (nnz_coarser >= 0 && k <= 256) most = std::min<int64_t>(400000, 280 * n);
     else if (n > 4096) most = std::min<int64_t>({350000, wide, 5000000000 / ((int64_t)k * k)});
     else most = std::min<int64_t>({400000, 280 * n, 40000000 / k});
-    const bool local = nnz_coarser >= 0 && 10 * nnz_coarser <= 8 * nnz && nnz <= 16 * n;
+    const bool local = nnz_coarser >= 0 && ((10 * nnz_coarser <= 8 * nnz && nnz <= 16 * n) ||
+                                            (20 * nnz_coarser <= 13 * nnz && (nnz <= 400000 || nnz <= 40 * n)));
     return local ? 2 * most : most;
 }
 

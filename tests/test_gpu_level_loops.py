@@ -201,3 +201,40 @@ def test_levels_whose_contraction_merges_entries_stay_longer(name, make, k, clus
     assert 50000 <= st.n[i] and 2 * st.m[i] > 76800000 // (160 + k) and 2 * st.m[i] <= 16 * st.n[i]
     assert (10 * st.m[i + 1] <= 8 * st.m[i]) == cluster
     assert (st.cluster_blocks[i] > 0) == cluster
+
+
+def _stays(n, nnz, coarser, k):
+    """The entry rule of the resident loop inside a hierarchy (k <= 256)."""
+    if n <= 8192:
+        most = min(400000, 280 * n)
+    else:
+        most = 76800000 // (160 + k)
+    local = (10 * coarser <= 8 * nnz and nnz <= 16 * n) or \
+        (20 * coarser <= 13 * nnz and (nnz <= 400000 or nnz <= 40 * n))
+    return nnz <= (2 * most if local else most)
+
+
+HIERARCHIES = [
+    ("geometric_of_degree_20", lambda: graphgen.rgg(31000, mean_degree=20.0, seed=3), 64, 0),
+    ("rmat_two_hop", lambda: graphgen.rmat(16, seed=5), 64, jet.FLAG_TWO_HOP),
+    ("rmat_sparse", lambda: graphgen.rmat(15, 6, seed=2, vw=(1, 3), ew=(1, 5)), 31, 0),
+    ("mesh", lambda: graphgen.grid3d(60, 60, 60, vw=(1, 4), ew=(1, 10), seed=4), 128, 0),
+]
+
+
+@pytest.mark.parametrize("name,make,k,flags", HIERARCHIES, ids=[h[0] for h in HIERARCHIES])
+def test_every_level_of_a_hierarchy_takes_its_loop(name, make, k, flags):
+    g = make()
+    t = _dev(g, False)
+    with jet.Context(0, flags=flags) as a, jet.Context(0, flags=flags, cluster_max_n=0) as b:
+        pa, ca, st = a.partition(*t, k=k, seed=2, return_stats=True)
+        pb, cb = b.partition(*t, k=k, seed=2)
+    assert ca == cb and torch.equal(pa, pb)
+    nnz = [2 * m for m in st.m]
+    seen = set()
+    for i, n in enumerate(st.n):
+        if 4096 < n <= 50000:                      # fits; up to 4,096 one of the cluster loops runs in any case
+            stays = _stays(n, nnz[i], nnz[min(i + 1, st.levels - 1)], k)
+            assert (st.cluster_blocks[i] > 0) == stays, (i, n, nnz[i])
+            seen.add(stays)
+    assert seen
